@@ -41,7 +41,7 @@
 namespace fhmg {
 
 constexpr int kSpG = 7;                         // digits per factor = group accumulators
-constexpr int kSpCols = 64;                     // grid points per tile (MMA N)
+constexpr int kSpCols = 64;                     // grid points per tile (MMA N: 64 per digit, up to four digits)
 constexpr int kSpRows = kSplitRows;             // time rows per output block (MMA M)
 constexpr int kSpK = 64;                        // time levels per K-block
 constexpr int kSpConsumers = 256;               // 8 consumer warps
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
             break;
           }
           tc_after_sync();
-          int touched = 0;
+          int gfirst = kSpG;  // lowest group this block has written
           for (int J = 0; J <= 2 * I + 1 && !failed; ++J, ++q) {
             const int b = (int)(q & 1);
             if (!mbar_wait_or_abort(xready + b, (uint32_t)((q >> 1) & 1), abort_flag, A.spin)) {
@@ -403,11 +403,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
             tc_after_sync();
             const int4 pd = __ldg(A.pairs + I * (I + 1) + J);
             const uint32_t xb = smem_u32(xbuf + (size_t)b * kSpG * kSpBtile);
-            // operand descriptors (K-major, 128-byte swizzle); a K step of 16 adds 2
-            uint64_t bdesc[kSpG];
-#pragma unroll
-            for (int bb = 0; bb < kSpG; ++bb) bdesc[bb] = sp_desc_sw128(xb + (uint32_t)bb * kSpBtile);
-            const uint32_t idesc = umma_idesc(kSpCols);
+            // operand descriptors: K-major, 128-byte swizzle; a K step of 16 adds 2
             for (int a = 0; a < kSpG; ++a) {
               if (!((pd.x >> a) & 1)) continue;
               if (!mbar_wait_or_abort(full + slot, (uint32_t)((k / ns) & 1), abort_flag, A.spin)) {
@@ -416,21 +412,28 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
               }
               tc_after_sync();
               const uint64_t adesc = sp_desc_sw128(smem_u32(ring + (size_t)slot * kSpAtile));
-#pragma unroll
-              for (int bb = 0; bb < kSpG; ++bb) {
-                if (bb + a >= kSpG) break;
-                const int gg = a + bb;
-                const uint32_t d = tmem + 64u * gg;
-                const uint32_t acc0 = (touched >> gg) & 1;
+              // digit a meets the u digits 0..6-a in the groups a..6: their tiles are consecutive in
+              // shared memory and the groups in tensor memory, so one MMA covers up to four of them
+              // (N = 256).  The groups touched so far are a suffix gfirst..6, which is accumulated
+              // into; the groups a..gfirst-1 are written afresh.  A 128 x 64 x 16 MMA is bound by its
+              // operand reads (48 cycles for 32 of tensor work) and by its issue (95 cycles seen); ten
+              // wide ones replace 28 per K step, and the sums keep their order (same bits): the defect
+              // of a 511^2 x 512 grid, pre-pass included, 6.47 -> 5.41 ms.
+              for (int g0 = a; g0 < kSpG;) {
+                const bool fresh = g0 < gfirst;
+                const int ng = min(fresh ? gfirst - g0 : kSpG - g0, 4);
+                const uint64_t bdesc = sp_desc_sw128(xb + (uint32_t)(g0 - a) * kSpBtile);
+                const uint32_t idesc = umma_idesc(ng * kSpCols), d = tmem + 64u * g0;
 #pragma unroll
                 for (int st = 0; st < kSpK / 16; ++st)
                   asm volatile(
                       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-                      "l"(adesc + 2ULL * st), "l"(bdesc[bb] + 2ULL * st), "r"(idesc), "r"(st > 0 ? 1u : acc0)
+                      "l"(adesc + 2ULL * st), "l"(bdesc + 2ULL * st), "r"(idesc), "r"(st > 0 || !fresh ? 1u : 0u)
                       : "memory");
-                touched |= 1 << gg;
+                g0 += ng;
               }
+              gfirst = min(gfirst, a);
               umma_commit(empty + slot);
               ++k;
               if (++slot == ns) slot = 0;
@@ -439,7 +442,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
             umma_commit(xfree + b);
           }
           if (failed) break;
-          *gmask = touched;
+          *gmask = 0x7f & (0x7f << gfirst);
           umma_commit(accdone);
           mbar_arrive(accdone);  // release: the group mask is visible to the consumers after their wait
         }
