@@ -176,33 +176,44 @@ __device__ __forceinline__ void sp_two_sum(float a, float b, float& h, float& l)
 }
 
 
-// two digits as a BF16 pair (the first in the low half)
-__device__ __forceinline__ uint32_t sp_bf16pair(int d0, int d1) {
-  // small integers are exact in FP32 via the 1.5 * 2^23 offset; their BF16 is the high half
-  const uint32_t f0 = __float_as_uint(__int_as_float(0x4B400000 + d0) - 12582912.0f);
-  const uint32_t f1 = __float_as_uint(__int_as_float(0x4B400000 + d1) - 12582912.0f);
-  return __byte_perm(f0, f1, 0x7632);
+// The balanced base-2^7 digits of an integer |X| <= 2^49, X = sum_b d_b 2^{7(G-1-b)}, d_1..d_6 in
+// [-64, 63] and |d_0| <= 129, are the 7-bit fields of Y = X + kSpBias less 64 (d_0: the bits above
+// them, unbiased): the bias carries into the next field exactly where a digit would leave its
+// range, so no digit waits for the one below it.
+constexpr long long kSpBias = (1LL << 6) | (1LL << 13) | (1LL << 20) | (1LL << 27) | (1LL << 34) | (1LL << 41);
+
+// X + kSpBias for X = round(mt 2^{e - fe - 4}) (half away from zero) of the FP64 value with these
+// bits, fe the largest biased exponent of its column (e <= fe: the shift is at least 4); subnormals
+// as 0
+__device__ __forceinline__ long long sp_biased(unsigned long long bits, int fe) {
+  const int e = (int)(bits >> 52) & 0x7FF;
+  const unsigned long long mt = (bits & 0xFFFFFFFFFFFFFULL) | (1ULL << 52);
+  const int s1 = e == 0 ? 63 : min(fe + 3 - e, 63);  // shift less one; mt >> 63 is 0, its rounding too
+  const unsigned long long r = ((mt >> s1) + 1) >> 1;
+  const long long sg = (long long)bits >> 63;
+  return ((long long)r ^ sg) - sg + kSpBias;
 }
 
-// the G balanced base-2^7 digits of an integer |X| <= 2^49 (X = sum_b d_b 2^{7(G-1-b)}), most
-// significant first; 32-bit operations: the low 28 bits give digits G-1..G-4, the rest d_0..d_2
-__device__ __forceinline__ void sp_digits(long long X, int (&d)[kSpG]) {
-  uint32_t lo = (uint32_t)X & 0x0FFFFFFFu;
-  int hi = (int)(X >> 28);
+// The BF16 pairs (y0's digit in the low half) of the digits of two biased integers.  A field v in
+// 0..127 is the BF16 128 + v with the bits 0x4300 | v, and 128 + v - 192 = v - 64 is exact in BF16:
+// three integer instructions and one packed subtraction per pair of digits.  d_0 goes through FP32
+// (1.5 2^23 + d_0, whose last bits are d_0): it may need 8 bits.
+__device__ __forceinline__ void sp_digit_pairs(long long y0, long long y1, uint32_t (&pk)[kSpG]) {
+  const uint32_t l0 = (uint32_t)y0, l1 = (uint32_t)y1;
+  const uint32_t m0 = (uint32_t)(y0 >> 21), m1 = (uint32_t)(y1 >> 21);  // fields 3, 4, 5 at bits 0, 7, 14
+  const __nv_bfloat162 c = __halves2bfloat162(__ushort_as_bfloat16(0x4340), __ushort_as_bfloat16(0x4340));  // 192
 #pragma unroll
-  for (int b = kSpG - 1; b >= kSpG - 4; --b) {
-    const int v = (int)((lo + 64u) & 127u) - 64;
-    d[b] = v;
-    lo = (uint32_t)((int)lo - v) >> 7;
+  for (int b = 1; b < kSpG; ++b) {
+    const int f = kSpG - 1 - b;  // field
+    const uint32_t w0 = f < 3 ? l0 >> (7 * f) : m0 >> (7 * (f - 3));
+    const uint32_t w1 = f < 3 ? l1 >> (7 * f) : m1 >> (7 * (f - 3));
+    uint32_t q = (__byte_perm(w0, w1, 0x5410) & 0x007F007Fu) | 0x43004300u;
+    const __nv_bfloat162 d = __hsub2(*reinterpret_cast<__nv_bfloat162*>(&q), c);
+    pk[b] = *reinterpret_cast<const uint32_t*>(&d);
   }
-  hi += (int)lo;  // carry
-#pragma unroll
-  for (int b = kSpG - 5; b >= 1; --b) {
-    const int v = ((hi + 64) & 127) - 64;
-    d[b] = v;
-    hi = (hi - v) >> 7;
-  }
-  d[0] = hi;
+  const uint32_t f0 = __float_as_uint(__int_as_float(0x4B400000 + (int)(y0 >> 42)) - 12582912.0f);
+  const uint32_t f1 = __float_as_uint(__int_as_float(0x4B400000 + (int)(y1 >> 42)) - 12582912.0f);
+  pk[0] = __byte_perm(f0, f1, 0x7632);
 }
 
 // FP64 value of the integer D times 2^k (D exact up to 53 bits, else rounded half up), by integer
@@ -602,7 +613,6 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
     }
     const SpCol mine = col[sn];
     const long long ps = mine.valid ? p0 + sn : 0;
-    const int fshift = mine.fe + 4;  // X = round(u 2^{49 - F_c}) = round(mt 2^{e - fe - 4})
     // this thread's 16 values of K-block J, staged in shared memory by cp.async (the next block's
     // copies are issued once this one's digits are published); each thread reads back only its own
     unsigned long long* mystage = stage + (size_t)sk * kSpCols + sn;
@@ -634,19 +644,14 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
       unsigned char* xb = xbuf + (size_t)b * kSpG * kSpBtile;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        uint32_t pk[kSpG][4];
+        uint32_t pk[4][kSpG];
 #pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-          int d0[kSpG], d1[kSpG];
-          sp_digits(sp_fixed(v[8 * h + j], fshift), d0);
-          sp_digits(sp_fixed(v[8 * h + j + 1], fshift), d1);
-#pragma unroll
-          for (int a = 0; a < kSpG; ++a) pk[a][j / 2] = sp_bf16pair(d0[a], d1[a]);
-        }
+        for (int j = 0; j < 4; ++j)
+          sp_digit_pairs(sp_biased(v[8 * h + 2 * j], mine.fe), sp_biased(v[8 * h + 2 * j + 1], mine.fe), pk[j]);
 #pragma unroll
         for (int a = 0; a < kSpG; ++a)
           *reinterpret_cast<uint4*>(xb + (size_t)a * kSpBtile + sp_sw128_off(sn, sk + 8 * h)) =
-              make_uint4(pk[a][0], pk[a][1], pk[a][2], pk[a][3]);
+              make_uint4(pk[0][a], pk[1][a], pk[2][a], pk[3][a]);
       }
       async_proxy_fence();
       __syncwarp();
