@@ -44,7 +44,7 @@ constexpr int kSpG = 7;                         // digits per factor = group acc
 constexpr int kSpCols = 64;                     // grid points per tile (MMA N: 64 per digit, up to four digits)
 constexpr int kSpRows = kSplitRows;             // time rows per output block (MMA M)
 constexpr int kSpK = 64;                        // time levels per K-block
-constexpr int kSpConsumers = 256;               // 8 consumer warps
+constexpr int kSpConsumers = 512;               // 16 consumer warps
 constexpr int kSpBlock = kSpConsumers + 64;     // + producer warp + MMA warp
 constexpr uint32_t kSpTmemCols = 512;
 constexpr int kSpAtile = kSpRows * kSpK * 2;    // bytes of one R~ digit tile
@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
     return;
   }
 
-  // ---- consumers: 8 warps ----
+  // ---- consumers: 16 warps ----
   uint32_t cbphase = 0;
   bool failed = false;
   auto give_up = [&](bool ok) -> bool {
@@ -483,30 +483,25 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
   };
   const long long ld = A.ld;
   const unsigned long long* Ub = reinterpret_cast<const unsigned long long*>(A.U);
-  // split: thread t owns point n = t & 63 of the tile and 16 time levels (t >> 6) * 16 .. of a K-block
-  const int sn = t & 63, sk = (t >> 6) * 16;
-  // epilogue: lane quarter (time rows) and column half
+  // split: thread t owns point n = t & 63 of the tile and 8 time levels (t >> 6) * 8 .. of a K-block
+  const int sn = t & 63, sk = (t >> 6) * 8;
+  // epilogue: lane quarter (time rows) and column quarter
   const int wq = w & 3, ch = w >> 2;
   const uint32_t lane_base = (uint32_t)(32 * wq) << 16;
   unsigned long long nmax = 0;
   long long q = 0, nblk = 0;
   const int npairs = nI * (nI + 1);
 
-  // L2 prefetch of the B rows that block I's epilogue reads (this thread's time row, its 32 points):
+  // L2 prefetch of the B rows that block I's epilogue reads (this thread's time row, its 16 points):
   // issued when the block's first pair is split, so that their latency overlaps the block's MMAs
   auto prefetch_block = [&](long long p0, int I) {
     const int m = I * kSpRows + wq * 32 + lane;
-    const long long pc = p0 + ch * 32;
-    const double* orow = A.OUT + (long long)m * ld;
-#pragma unroll
-    for (int o = 0; o < 32; o += 16) {
-      const long long i = pc + o < ld ? pc + o : ld - 1;
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(orow + i));
-    }
+    const long long pc = min(p0 + ch * 16, ld - 1);
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(A.OUT + (long long)m * ld + pc));
   };
 
   // epilogue of output block I of the tile at p0 (its accumulators complete: accdone waited).  Phase
-  // 1: all eight warps fold the seven groups of their 32 time rows x 32 points into double-float sums
+  // 1: all sixteen warps fold the seven groups of their 32 time rows x 16 points into double-float sums
   // and write them transposed into the two pieces (points 0..31 in the staging bytes, points 32..63
   // in digit buffer bfree, whose pair's MMAs completed with the block's), then release tensor memory,
   // so that the next block's MMAs start while phase 2 runs.  Phase 2: thread per grid point, so that
@@ -517,11 +512,11 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
     float2* const piece1 = reinterpret_cast<float2*>(xbuf + (size_t)bfree * kSpG * kSpBtile);
     if (!consumer_meet()) return false;  // every warp has read its staged values (piece 0 reuses them)
     {
-      float2* const pc = ch ? piece1 : piece0;
+      float2* const pc = (ch >> 1 ? piece1 : piece0) + (size_t)(ch & 1) * 16 * kSpPieceLd;
       const int ml = wq * 32 + lane;
 #pragma unroll 1
-      for (int c8 = 0; c8 < 4; ++c8) {
-        const uint32_t n0 = (uint32_t)(ch * 32 + c8 * 8);
+      for (int c8 = 0; c8 < 2; ++c8) {
+        const uint32_t n0 = (uint32_t)(ch * 16 + c8 * 8);
         uint32_t r[kSpG][8];
 #pragma unroll
         for (int gg = 0; gg < kSpG; ++gg)
@@ -555,41 +550,34 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
       if (lane == 0) mbar_arrive(accfree);  // this warp is done with block I's accumulators
     }
     if (!consumer_meet()) return false;  // the pieces are complete
-    // thread: point n = half * 32 + lane, time rows w * 16 .. + 15 of the block, half 0 first:
-    // r = B - (R~ u), B = F - A_h u from the pre-pass (in OUT).  Once every thread is done with piece
-    // 0, mid() may reuse the staging bytes (the next K-block's copies overlap half 1)
-#pragma unroll 1
-    for (int half = 0; half < 2; ++half) {
-      const int n = half * 32 + lane;
-      const float2* const pc = half ? piece1 : piece0;
+    // thread: point n = (w / 8) * 32 + lane, time rows (w % 8) * 16 .. + 15 of the block:
+    // r = B - (R~ u), B = F - A_h u from the pre-pass (in OUT)
+    {
+      const int n = (w >> 3) * 32 + lane, m0 = (w & 7) * 16;
+      const float2* const pc = (w >> 3 ? piece1 : piece0) + (size_t)lane * kSpPieceLd + m0;
       const SpCol c = col[n];
       const long long p = p0 + n;
-      const long long pa = c.valid ? p : 0;
+      double* const out = A.OUT + (long long)(I * kSpRows + m0) * ld + (c.valid ? p : 0);
       double bv[16];
-      const double* bsrc = A.OUT + (long long)(I * kSpRows + w * 16) * ld + pa;
 #pragma unroll
-      for (int rr = 0; rr < 16; ++rr) bv[rr] = __ldcg(bsrc + (long long)rr * ld);
+      for (int rr = 0; rr < 16; ++rr) bv[rr] = __ldcg(out + (long long)rr * ld);
 #pragma unroll
       for (int rr = 0; rr < 16; ++rr) {
-        const int ml = w * 16 + rr;
-        const int m = I * kSpRows + ml;
-        const int Em = __ldg(A.rexp + m);
-        const float2 P = pc[(size_t)lane * kSpPieceLd + ml];
+        const int Em = __ldg(A.rexp + I * kSpRows + m0 + rr);
+        const float2 P = pc[rr];
         // (R~ u)_{m,c} = 2^{E_m + F_c - 14} P, F_c = fe - 1022
         const double y = sp_join(P.x, P.y, Em + c.fe - 1036);
         const double r = c.fe == 2047 ? __longlong_as_double(0x7FF8000000000000LL) : bv[rr] - y;
         if (c.valid) {
-          A.OUT[(long long)m * ld + p] = r;
+          out[(long long)rr * ld] = r;
           const unsigned long long ab = (unsigned long long)__double_as_longlong(r) & 0x7FFFFFFFFFFFFFFFULL;
           nmax = ab > nmax ? ab : nmax;
         }
       }
-      if (half == 0) {
-        if (!consumer_meet()) return false;  // every thread is done with piece 0
-        mid();
-      }
     }
-    return consumer_meet();  // every thread is done with the pieces
+    if (!consumer_meet()) return false;  // every thread is done with the pieces
+    mid();
+    return true;
   };
 
   for (long long g = blockIdx.x; g < A.ntiles && !failed; g += gridDim.x) {
@@ -613,19 +601,19 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
     }
     const SpCol mine = col[sn];
     const long long ps = mine.valid ? p0 + sn : 0;
-    // this thread's 16 values of K-block J, staged in shared memory by cp.async (the next block's
+    // this thread's 8 values of K-block J, staged in shared memory by cp.async (the next block's
     // copies are issued once this one's digits are published); each thread reads back only its own
     unsigned long long* mystage = stage + (size_t)sk * kSpCols + sn;
-    auto stage16 = [&](int J) {
+    auto stage8 = [&](int J) {
       const unsigned long long* src = Ub + (long long)(J * kSpK + sk) * ld + ps;
 #pragma unroll
-      for (int j = 0; j < 16; ++j)
+      for (int j = 0; j < 8; ++j)
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(mystage + (size_t)j * kSpCols)),
                      "l"(src + (long long)j * ld)
                      : "memory");
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    stage16(0);
+    stage8(0);
     // the tile's pairs in order; block I's epilogue runs after the first pair of block I + 1 is
     // split (so that block I's last MMAs overlap that work), the last block's at the tile's end
     int I = 0, J = 0;
@@ -638,21 +626,17 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
       const int In = J + 1 <= 2 * I + 1 ? I : I + 1;
       const int Jn = J + 1 <= 2 * I + 1 ? J + 1 : 0;
       asm volatile("cp.async.wait_group 0;" ::: "memory");
-      unsigned long long v[16];
+      unsigned long long v[8];
 #pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = mine.valid ? mystage[(size_t)j * kSpCols] : 0ULL;
+      for (int j = 0; j < 8; ++j) v[j] = mine.valid ? mystage[(size_t)j * kSpCols] : 0ULL;
       unsigned char* xb = xbuf + (size_t)b * kSpG * kSpBtile;
+      uint32_t pk[4][kSpG];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        uint32_t pk[4][kSpG];
+      for (int j = 0; j < 4; ++j) sp_digit_pairs(sp_biased(v[2 * j], mine.fe), sp_biased(v[2 * j + 1], mine.fe), pk[j]);
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          sp_digit_pairs(sp_biased(v[8 * h + 2 * j], mine.fe), sp_biased(v[8 * h + 2 * j + 1], mine.fe), pk[j]);
-#pragma unroll
-        for (int a = 0; a < kSpG; ++a)
-          *reinterpret_cast<uint4*>(xb + (size_t)a * kSpBtile + sp_sw128_off(sn, sk + 8 * h)) =
-              make_uint4(pk[0][a], pk[1][a], pk[2][a], pk[3][a]);
-      }
+      for (int a = 0; a < kSpG; ++a)
+        *reinterpret_cast<uint4*>(xb + (size_t)a * kSpBtile + sp_sw128_off(sn, sk)) =
+            make_uint4(pk[0][a], pk[1][a], pk[2][a], pk[3][a]);
       async_proxy_fence();
       __syncwarp();
       if (lane == 0) mbar_arrive(xready + b);
@@ -661,7 +645,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
       const bool epi = (J == 0 && I > 0) || last;
       // the next pair's copies only now (the proxy fence above waits for this thread's outstanding
       // memory operations) and, when an epilogue runs here, once it is done with the staging bytes
-      if (!epi && s + 1 < npairs) stage16(Jn);
+      if (!epi && s + 1 < npairs) stage8(Jn);
       if (epi) {
         // epilogue of block I - 1 (or, at the tile's end, of the last block)
         const int Ie = last ? I : I - 1;
@@ -673,7 +657,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
         }
         tc_after_sync();
         if (!epilogue(p0, Ie, bfree, [&]() {
-              if (s + 1 < npairs) stage16(Jn);
+              if (s + 1 < npairs) stage8(Jn);
             })) {
           failed = true;
           break;
