@@ -44,30 +44,25 @@ constexpr int kSpG = 7;                         // digits per factor = group acc
 constexpr int kSpCols = 64;                     // grid points per tile (MMA N: 64 per digit, up to four digits)
 constexpr int kSpRows = kSplitRows;             // time rows per output block (MMA M)
 constexpr int kSpK = 64;                        // time levels per K-block
-constexpr int kSpConsumers = 512;               // 16 consumer warps
-constexpr int kSpBlock = kSpConsumers + 64;     // + producer warp + MMA warp
+constexpr int kSpSplit = 256;                   // 8 warps that split u into digit tiles
+constexpr int kSpEpi = 256;                     // 8 epilogue warps
+constexpr int kSpBlock = kSpSplit + kSpEpi + 64;  // + producer warp + MMA warp
 constexpr uint32_t kSpTmemCols = 512;
 constexpr int kSpAtile = kSpRows * kSpK * 2;    // bytes of one R~ digit tile
 constexpr int kSpBtile = kSpCols * kSpK * 2;    // bytes of one u digit tile
 constexpr int kSpPieceLd = kSpRows + 1;         // float pairs per point of the epilogue's piece (odd: no bank conflicts)
-static_assert((size_t)32 * kSpPieceLd * 8 <= (size_t)kSpG * kSpBtile, "a piece fits a digit buffer");
 
 struct SplitSmem {
-  size_t ring, xbuf, stage, col, bar, total;
+  size_t ring, xbuf, piece, bar, total;
 };
 __host__ __device__ inline SplitSmem split_smem(int ns) {
   SplitSmem s;
   s.ring = 0;
   s.xbuf = (size_t)ns * kSpAtile;
-  // the next K-block's u values ([64 levels][64 points] doubles); during an epilogue the same bytes hold
-  // the transposed piece of points 0..31 ([32 points][kSpPieceLd] float pairs; points 32..63 go to
-  // the free digit buffer, kSpG * kSpBtile bytes)
-  s.stage = s.xbuf + 2 * (size_t)kSpG * kSpBtile;
-  const size_t stage_bytes = (size_t)kSpK * kSpCols * 8, piece_bytes = (size_t)32 * kSpPieceLd * 8;
-  s.col = s.stage + (stage_bytes > piece_bytes ? stage_bytes : piece_bytes);
-  s.bar = s.col + (size_t)kSpCols * 16;
+  s.piece = s.xbuf + 2 * (size_t)kSpG * kSpBtile;  // epilogue: [32 points][kSpPieceLd] float pairs
+  s.bar = s.piece + (size_t)32 * kSpPieceLd * 8;
   // full[ns], empty[ns], xready[2], xfree[2], accdone, accfree, cbar, exitbar, donebar, then the
-  // abort flag, the group mask and the TMEM address
+  // abort flag, the lowest group written and the TMEM address
   s.total = s.bar + 8 * ((size_t)2 * ns + 9) + 16;
   return s;
 }
@@ -111,70 +106,43 @@ __device__ __forceinline__ float sp_pow2f(int k) {
   return k < -126 ? 0.f : __int_as_float((min(k, 127) + 127) << 23);
 }
 
-// FP64 value of float f times 2^k, exactly (integer operations; f normal or zero)
+// FP64 value of float f times 2^k, exactly, by integer operations (a conversion runs on the 1/64-rate
+// FP64 pipe); f subnormal and results below the FP64 normal range: 0, above it: Inf
 __device__ __forceinline__ double sp_f2d_scaled(float f, int k) {
-  const uint32_t b = __float_as_uint(f);
-  const int ef = (int)((b >> 23) & 0xFF);
-  if (ef == 0) return 0.0;
-  const unsigned long long sign = (unsigned long long)(b >> 31) << 63;
-  const long long ed = (long long)ef - 127 + 1023 + k;
-  if (ed <= 0) return 0.0;  // below the FP64 normal range
-  if (ed >= 2047) return __longlong_as_double((long long)(sign | 0x7FF0000000000000ULL));
-  const unsigned long long mant = (unsigned long long)(b & 0x7FFFFF) << 29;
-  return __longlong_as_double((long long)(sign | ((unsigned long long)ed << 52) | mant));
+  const uint32_t b = __float_as_uint(f), m = b & 0x7FFFFFFFu;
+  const int e = (int)(m >> 23) + 896 + k;
+  uint32_t hi = (m >> 3) + ((uint32_t)(896 + k) << 20), lo = b << 29;
+  if (m < 0x00800000u || (unsigned)(e - 1) >= 2046u) {
+    hi = m < 0x00800000u || e <= 0 ? 0u : 0x7FF00000u;
+    lo = 0u;
+  }
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)lo);
 }
 
-// FP64 nearest (up to one rounding of the smaller part) to (h + l) 2^k for a float pair, by integer
-// operations: the 24-bit significand of the part with the larger exponent is widened to 53 bits and
-// the other one's added at its offset (dropped below 2^-25 of its last place); zero: the other alone.
-__device__ __forceinline__ double sp_join(float h, float l, int k) {
-  uint32_t hb = __float_as_uint(h), lb = __float_as_uint(l);
-  if (((lb >> 23) & 0xFF) > ((hb >> 23) & 0xFF)) {  // the larger exponent leads (then d <= 29 below)
-    const uint32_t x = hb;
-    hb = lb;
-    lb = x;
-  }
-  const int eh = (int)((hb >> 23) & 0xFF), el = (int)((lb >> 23) & 0xFF);
-  if (eh == 0) return sp_f2d_scaled(l, k);
-  long long Mh = (long long)((hb & 0x7FFFFF) | 0x800000) << 29;  // units 2^{eh - 127 - 52}
-  if (hb >> 31) Mh = -Mh;
-  if (el != 0) {
-    const int d = el - eh + 29;  // l's significand in units of Mh's last place: shift by d
-    const long long ml = (long long)((lb & 0x7FFFFF) | 0x800000);
-    long long Ml = d >= 0 ? (ml << d) : (d > -25 ? ((ml + (1LL << (-d - 1))) >> (-d)) : 0);
-    if (lb >> 31) Ml = -Ml;
-    Mh += Ml;
-  }
-  if (Mh == 0) return 0.0;
-  const unsigned long long sign = Mh < 0 ? (1ULL << 63) : 0ULL;
-  unsigned long long a = (unsigned long long)(Mh < 0 ? -Mh : Mh);
-  int e = eh - 127 - 52 + k;  // value = a 2^e
-  const int lz = __clzll((long long)a);  // normalise to 53 bits (bit 52 set)
-  if (lz > 11) {
-    a <<= (lz - 11);
-    e -= lz - 11;
-  } else if (lz < 11) {
-    const int sh = 11 - lz;
-    a = (a + (1ULL << (sh - 1))) >> sh;
-    e += sh;
-    if (a >> 53) {
-      a >>= 1;
-      ++e;
-    }
-  }
-  const long long ed = (long long)e + 52 + 1023;
-  if (ed <= 0) return 0.0;
-  if (ed >= 2047) return __longlong_as_double((long long)(sign | 0x7FF0000000000000ULL));
-  return __longlong_as_double((long long)(sign | ((unsigned long long)ed << 52) | (a & 0xFFFFFFFFFFFFFULL)));
+// two FP32 values in one register pair: sums and products of both with one instruction
+typedef unsigned long long sp_f2;
+__device__ __forceinline__ sp_f2 sp_pack2(uint32_t a, uint32_t b) { return (sp_f2)a | ((sp_f2)b << 32); }
+__device__ __forceinline__ sp_f2 sp_add2(sp_f2 a, sp_f2 b) {
+  sp_f2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
 }
-
-// (h, l) = a + b exactly
-__device__ __forceinline__ void sp_two_sum(float a, float b, float& h, float& l) {
-  h = __fadd_rn(a, b);
-  const float bb = __fsub_rn(h, a);
-  l = __fadd_rn(__fsub_rn(a, __fsub_rn(h, bb)), __fsub_rn(b, bb));
+__device__ __forceinline__ sp_f2 sp_sub2(sp_f2 a, sp_f2 b) {
+  sp_f2 d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
 }
-
+__device__ __forceinline__ sp_f2 sp_mul2(sp_f2 a, sp_f2 b) {
+  sp_f2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// (h, l) = a + b exactly (both halves)
+__device__ __forceinline__ void sp_two_sum2(sp_f2 a, sp_f2 b, sp_f2& h, sp_f2& l) {
+  h = sp_add2(a, b);
+  const sp_f2 bb = sp_sub2(h, a);
+  l = sp_add2(sp_sub2(a, sp_sub2(h, bb)), sp_sub2(b, bb));
+}
 
 // The balanced base-2^7 digits of an integer |X| <= 2^49, X = sum_b d_b 2^{7(G-1-b)}, d_1..d_6 in
 // [-64, 63] and |d_0| <= 129, are the 7-bit fields of Y = X + kSpBias less 64 (d_0: the bits above
@@ -286,12 +254,6 @@ __global__ void __launch_bounds__(256) split_prep_kernel(const double* __restric
   }
 }
 
-struct SpCol {
-  int fe;     // the point's exponent (biased; 2047: an Inf or NaN in u at the point, r := NaN)
-  int valid;
-  int pad0, pad1;
-};
-
 __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_constant__ SplitArgs A) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   // the swizzled operand tiles need 1024-byte aligned addresses (the launcher adds 1 KB)
@@ -300,8 +262,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
   const int ns = A.ns;
   unsigned char* ring = sm + lay.ring;
   unsigned char* xbuf = sm + lay.xbuf;
-  SpCol* col = reinterpret_cast<SpCol*>(sm + lay.col);
-  unsigned long long* stage = reinterpret_cast<unsigned long long*>(sm + lay.stage);
+  float2* const piece = reinterpret_cast<float2*>(sm + lay.piece);
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + lay.bar);
   uint64_t* empty = full + ns;
   uint64_t* xready = empty + ns;  // [2]
@@ -312,7 +273,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
   uint64_t* exitbar = accdone + 3;
   uint64_t* donebar = accdone + 4;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(accdone + 5);
-  volatile int* gmask = abort_flag + 1;
+  volatile int* gfirst_s = abort_flag + 1;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(accdone + 5) + 2;
 
   const int t = threadIdx.x;
@@ -326,16 +287,16 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
       mbar_init(empty + s, 1);  // the MMAs' commit
     }
     for (int b = 0; b < 2; ++b) {
-      mbar_init(xready + b, kSpConsumers / 32);
+      mbar_init(xready + b, kSpSplit / 32);
       mbar_init(xfree + b, 1);
     }
-    mbar_init(accdone, 2);  // the MMAs' commit + the MMA thread's arrive after publishing the group mask
-    mbar_init(accfree, kSpConsumers / 32);
-    mbar_init(cbar, kSpConsumers / 32);
-    mbar_init(exitbar, kSpConsumers / 32 + 1);
+    mbar_init(accdone, 2);  // the MMAs' commit + the MMA thread's arrive after publishing the lowest group
+    mbar_init(accfree, kSpEpi / 32);
+    mbar_init(cbar, kSpEpi / 32);
+    mbar_init(exitbar, (kSpSplit + kSpEpi) / 32 + 1);
     mbar_init(donebar, 1);
     *abort_flag = 0;
-    *gmask = 0;
+    *gfirst_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (w == 0) {
@@ -355,7 +316,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
     }
   };
 
-  if (w == kSpConsumers / 32) {
+  if (w == (kSpSplit + kSpEpi) / 32) {
     // ---- producer: R~ digit tiles of every pair of every tile of this CTA, in order ----
     if (lane != 0) return;
     long long k = 0;
@@ -391,7 +352,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
     return;
   }
 
-  if (w == kSpConsumers / 32 + 1) {
+  if (w == (kSpSplit + kSpEpi) / 32 + 1) {
     // ---- MMA thread ----
     if (lane == 0) {
       long long k = 0, q = 0, nblk = 0;
@@ -453,9 +414,9 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
             umma_commit(xfree + b);
           }
           if (failed) break;
-          *gmask = 0x7f & (0x7f << gfirst);
+          *gfirst_s = gfirst;
           umma_commit(accdone);
-          mbar_arrive(accdone);  // release: the group mask is visible to the consumers after their wait
+          mbar_arrive(accdone);  // release: the lowest group is visible to the epilogue after its wait
         }
       if (failed) raise();
       umma_commit(donebar);  // completes when every MMA issued above has completed
@@ -466,217 +427,220 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
     return;
   }
 
-  // ---- consumers: 16 warps ----
-  uint32_t cbphase = 0;
+  // ---- split and epilogue warps ----
   bool failed = false;
   auto give_up = [&](bool ok) -> bool {
     if (__all_sync(0xffffffffu, ok)) return false;
     if (lane == 0) raise();
     return true;
   };
-  auto consumer_meet = [&]() -> bool {
-    __syncwarp();
-    if (lane == 0) mbar_arrive(cbar);
-    const bool ok = mbar_wait_or_abort(cbar, cbphase, abort_flag, A.spin);
-    cbphase ^= 1;
-    return !give_up(ok);
-  };
   const long long ld = A.ld;
-  const unsigned long long* Ub = reinterpret_cast<const unsigned long long*>(A.U);
-  // split: thread t owns point n = t & 63 of the tile and 8 time levels (t >> 6) * 8 .. of a K-block
-  const int sn = t & 63, sk = (t >> 6) * 8;
-  // epilogue: lane quarter (time rows) and column quarter
-  const int wq = w & 3, ch = w >> 2;
-  const uint32_t lane_base = (uint32_t)(32 * wq) << 16;
-  unsigned long long nmax = 0;
-  long long q = 0, nblk = 0;
-  const int npairs = nI * (nI + 1);
 
-  // L2 prefetch of the B rows that block I's epilogue reads (this thread's time row, its 16 points):
-  // issued when the block's first pair is split, so that their latency overlaps the block's MMAs
-  auto prefetch_block = [&](long long p0, int I) {
-    const int m = I * kSpRows + wq * 32 + lane;
-    const long long pc = min(p0 + ch * 16, ld - 1);
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(A.OUT + (long long)m * ld + pc));
-  };
-
-  // epilogue of output block I of the tile at p0 (its accumulators complete: accdone waited).  Phase
-  // 1: all sixteen warps fold the seven groups of their 32 time rows x 16 points into double-float sums
-  // and write them transposed into the two pieces (points 0..31 in the staging bytes, points 32..63
-  // in digit buffer bfree, whose pair's MMAs completed with the block's), then release tensor memory,
-  // so that the next block's MMAs start while phase 2 runs.  Phase 2: thread per grid point, so that
-  // every global access is a contiguous row segment.
-  auto epilogue = [&](long long p0, int I, int bfree, auto&& mid) -> bool {
-    const int mask = *gmask;
-    float2* const piece0 = reinterpret_cast<float2*>(stage);
-    float2* const piece1 = reinterpret_cast<float2*>(xbuf + (size_t)bfree * kSpG * kSpBtile);
-    if (!consumer_meet()) return false;  // every warp has read its staged values (piece 0 reuses them)
-    {
-      float2* const pc = (ch >> 1 ? piece1 : piece0) + (size_t)(ch & 1) * 16 * kSpPieceLd;
-      const int ml = wq * 32 + lane;
-#pragma unroll 1
-      for (int c8 = 0; c8 < 2; ++c8) {
-        const uint32_t n0 = (uint32_t)(ch * 16 + c8 * 8);
-        uint32_t r[kSpG][8];
+  if (w < kSpSplit / 32) {
+    // ---- split: thread t owns point n = t & 63 of the tile and 16 time levels (t >> 6) * 16 .. of a
+    // K-block; the next block's values are loaded into registers once this one's digits are published
+    const int sn = t & 63, sk = (t >> 6) * 16;
+    const unsigned long long* Ub = reinterpret_cast<const unsigned long long*>(A.U);
+    unsigned long long v[16];
+    int fe = 0;
+    auto load16 = [&](long long g, int J) {
+      const long long p = g * kSpCols + sn;
+      const bool ok = p < ld;
+      const unsigned long long* src = Ub + (long long)(J * kSpK + sk) * ld + (ok ? p : 0);
 #pragma unroll
-        for (int gg = 0; gg < kSpG; ++gg)
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-              : "=r"(r[gg][0]), "=r"(r[gg][1]), "=r"(r[gg][2]), "=r"(r[gg][3]), "=r"(r[gg][4]), "=r"(r[gg][5]),
-                "=r"(r[gg][6]), "=r"(r[gg][7])
-              : "r"(tmem + lane_base + 64u * gg + n0));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        // the loaded registers are read only after the wait
-#pragma unroll
-        for (int gg = 0; gg < kSpG; ++gg)
-          asm volatile("" : "+r"(r[gg][0]), "+r"(r[gg][1]), "+r"(r[gg][2]), "+r"(r[gg][3]), "+r"(r[gg][4]),
-                       "+r"(r[gg][5]), "+r"(r[gg][6]), "+r"(r[gg][7]));
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          float ph = (mask & 1) ? __uint_as_float(r[0][j]) : 0.f, pl = 0.f;
-#pragma unroll
-          for (int gg = 1; gg < kSpG; ++gg) {
-            const float a = ((mask >> gg) & 1) ? __uint_as_float(r[gg][j]) : 0.f;
-            float s2, e;
-            sp_two_sum(ph, a * sp_pow2f(-7 * gg), s2, e);
-            ph = s2;
-            pl = __fadd_rn(pl, e);
+      for (int j = 0; j < 16; ++j) v[j] = ok ? __ldg(src + (long long)j * ld) : 0ULL;
+      if (J == 0) fe = ok ? __ldg(A.fe + p) : 0;
+    };
+    // L2 prefetch of 128 time rows from row m0 on of tile g of u (two lines per thread)
+    auto prefetch_u = [&](long long g, int m0) {
+      const unsigned long long* row = Ub + (long long)(m0 + (t >> 1)) * ld;
+      const long long p = g * kSpCols + (t & 1) * 32;
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(row + min(p, ld - 1)));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(row + min(p + 16, ld - 1)));
+    };
+    long long q = 0;
+    load16(blockIdx.x, 0);
+    for (long long g = blockIdx.x; g < A.ntiles && !failed; g += gridDim.x)
+      for (int I = 0; I < nI && !failed; ++I)
+        for (int J = 0; J <= 2 * I + 1; ++J, ++q) {
+          const int b = (int)(q & 1);
+          if (q >= 2 && give_up(mbar_wait_or_abort(xfree + b, (uint32_t)(((q >> 1) - 1) & 1), abort_flag, A.spin))) {
+            failed = true;
+            break;
           }
-          pc[(size_t)(c8 * 8 + j) * kSpPieceLd + ml] = make_float2(ph, pl);
+          unsigned char* xb = xbuf + (size_t)b * kSpG * kSpBtile;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            uint32_t pk[4][kSpG];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              sp_digit_pairs(sp_biased(v[8 * h + 2 * j], fe), sp_biased(v[8 * h + 2 * j + 1], fe), pk[j]);
+#pragma unroll
+            for (int a = 0; a < kSpG; ++a)
+              *reinterpret_cast<uint4*>(xb + (size_t)a * kSpBtile + sp_sw128_off(sn, sk + 8 * h)) =
+                  make_uint4(pk[0][a], pk[1][a], pk[2][a], pk[3][a]);
+          }
+          async_proxy_fence();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(xready + b);
+          // the next block's loads only now: the proxy fence waits for this thread's outstanding
+          // memory operations.  K-blocks 2 I + 2, 2 I + 3 (the next tile's 0, 1) are new to this CTA
+          // when block I is done: their lines are fetched into L2 meanwhile
+          if (J == 0) {
+            if (I + 1 < nI)
+              prefetch_u(g, 2 * (I + 1) * kSpK);
+            else if (g + gridDim.x < A.ntiles)
+              prefetch_u(g + gridDim.x, 0);
+          }
+          const int Jn = J < 2 * I + 1 ? J + 1 : 0;
+          const long long gn = Jn == 0 && I + 1 == nI ? g + gridDim.x : g;
+          if (gn < A.ntiles) load16(gn, Jn);
+        }
+  } else {
+    // ---- epilogue: r = B - R~ u for a block of 128 time rows x 64 points, B = F - A_h u from the
+    // pre-pass (in OUT).  Drain: thread (lane quarter wq: 32 time rows; ch: column half of each 32
+    // points) folds the seven groups into double-float sums, points 0..31 straight into the piece,
+    // points 32..63 kept in registers, and releases tensor memory, so that the next block's MMAs
+    // run during the rest.  Write-back, 32 points at a time: transposed through the piece, thread
+    // per grid point, so that every global access runs along a row.
+    const int e = t - kSpSplit, ew = e >> 5;
+    const int wq = ew & 3, ch = ew >> 2;
+    const uint32_t lane_base = (uint32_t)(32 * wq) << 16;
+    uint32_t cbphase = 0;
+    auto meet = [&]() -> bool {  // all epilogue warps (bounded)
+      __syncwarp();
+      if (lane == 0) mbar_arrive(cbar);
+      const bool ok = mbar_wait_or_abort(cbar, cbphase, abort_flag, A.spin);
+      cbphase ^= 1;
+      return !give_up(ok);
+    };
+    unsigned long long nmax = 0;
+    float2* const mine = piece + (size_t)(ch * 16) * kSpPieceLd + wq * 32 + lane;
+    // the double-float sums of this thread's time row at points pbase + 8 c8 + 0..7
+    auto fold8 = [&](uint32_t col, int gfirst, sp_f2 (&h)[4], sp_f2 (&l)[4]) {
+      uint32_t r[kSpG][8];
+#pragma unroll
+      for (int gg = 0; gg < kSpG; ++gg)
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+            : "=r"(r[gg][0]), "=r"(r[gg][1]), "=r"(r[gg][2]), "=r"(r[gg][3]), "=r"(r[gg][4]), "=r"(r[gg][5]),
+              "=r"(r[gg][6]), "=r"(r[gg][7])
+            : "r"(tmem + lane_base + 64u * gg + col));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      // the loaded registers are read only after the wait
+#pragma unroll
+      for (int gg = 0; gg < kSpG; ++gg) {
+        asm volatile("" : "+r"(r[gg][0]), "+r"(r[gg][1]), "+r"(r[gg][2]), "+r"(r[gg][3]), "+r"(r[gg][4]),
+                     "+r"(r[gg][5]), "+r"(r[gg][6]), "+r"(r[gg][7]));
+        if (gg < gfirst) {  // a group no MMA wrote (none of R~'s digits a <= gg in the block)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) r[gg][j] = 0;
         }
       }
-      tc_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(accfree);  // this warp is done with block I's accumulators
-    }
-    if (!consumer_meet()) return false;  // the pieces are complete
-    // thread: point n = (w / 8) * 32 + lane, time rows (w % 8) * 16 .. + 15 of the block:
-    // r = B - (R~ u), B = F - A_h u from the pre-pass (in OUT)
-    {
-      const int n = (w >> 3) * 32 + lane, m0 = (w & 7) * 16;
-      const float2* const pc = (w >> 3 ? piece1 : piece0) + (size_t)lane * kSpPieceLd + m0;
-      const SpCol c = col[n];
-      const long long p = p0 + n;
-      double* const out = A.OUT + (long long)(I * kSpRows + m0) * ld + (c.valid ? p : 0);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        h[j] = sp_pack2(r[0][2 * j], r[0][2 * j + 1]);
+        l[j] = 0;
+#pragma unroll
+        for (int gg = 1; gg < kSpG; ++gg) {
+          const uint32_t sc = __float_as_uint(1.f / (float)(1ULL << (7 * gg)));
+          sp_f2 s2, er;
+          sp_two_sum2(h[j], sp_mul2(sp_pack2(r[gg][2 * j], r[gg][2 * j + 1]), sp_pack2(sc, sc)), s2, er);
+          h[j] = s2;
+          l[j] = sp_add2(l[j], er);
+        }
+      }
+    };
+    auto put8 = [&](int c8, const sp_f2 (&h)[4], const sp_f2 (&l)[4]) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        mine[(size_t)(c8 * 8 + 2 * j) * kSpPieceLd] =
+            make_float2(__uint_as_float((uint32_t)h[j]), __uint_as_float((uint32_t)l[j]));
+        mine[(size_t)(c8 * 8 + 2 * j + 1) * kSpPieceLd] =
+            make_float2(__uint_as_float((uint32_t)(h[j] >> 32)), __uint_as_float((uint32_t)(l[j] >> 32)));
+      }
+    };
+    // write-back of the piece: thread = point p, time rows m0 .. m0 + 15
+    auto write16 = [&](long long p, int fe, int m0) {
+      const float2* const pc = piece + (size_t)lane * kSpPieceLd + ew * 16;
+      const bool ok = p < ld;
+      double* const out = A.OUT + (long long)m0 * ld + (ok ? p : 0);
       double bv[16];
 #pragma unroll
       for (int rr = 0; rr < 16; ++rr) bv[rr] = __ldcg(out + (long long)rr * ld);
 #pragma unroll
       for (int rr = 0; rr < 16; ++rr) {
-        const int Em = __ldg(A.rexp + I * kSpRows + m0 + rr);
         const float2 P = pc[rr];
-        // (R~ u)_{m,c} = 2^{E_m + F_c - 14} P, F_c = fe - 1022
-        const double y = sp_join(P.x, P.y, Em + c.fe - 1036);
-        const double r = c.fe == 2047 ? __longlong_as_double(0x7FF8000000000000LL) : bv[rr] - y;
-        if (c.valid) {
+        const int k = __ldg(A.rexp + m0 + rr) + fe - 1036;  // (R~ u)_{m,c} = 2^{E_m + F_c - 14} P, F_c = fe - 1022
+        double r = (bv[rr] - sp_f2d_scaled(P.x, k)) - sp_f2d_scaled(P.y, k);
+        if (fe == 2047) r = __longlong_as_double(0x7FF8000000000000LL);  // an Inf or NaN in u at the point
+        if (ok) {
           out[(long long)rr * ld] = r;
           const unsigned long long ab = (unsigned long long)__double_as_longlong(r) & 0x7FFFFFFFFFFFFFFFULL;
           nmax = ab > nmax ? ab : nmax;
         }
       }
-    }
-    if (!consumer_meet()) return false;  // every thread is done with the pieces
-    mid();
-    return true;
-  };
-
-  for (long long g = blockIdx.x; g < A.ntiles && !failed; g += gridDim.x) {
-    const long long p0 = g * kSpCols;
-    if (!consumer_meet()) {  // the previous tile's epilogue is done with col[]
-      failed = true;
-      break;
-    }
-    if (t < kSpCols) {
-      const long long p = p0 + t;
-      SpCol c{0, 0, 0, 0};
-      if (p < ld) {
-        c.valid = 1;
-        c.fe = __ldg(A.fe + p);
-      }
-      col[t] = c;
-    }
-    if (!consumer_meet()) {
-      failed = true;
-      break;
-    }
-    const SpCol mine = col[sn];
-    const long long ps = mine.valid ? p0 + sn : 0;
-    // this thread's 8 values of K-block J, staged in shared memory by cp.async (the next block's
-    // copies are issued once this one's digits are published); each thread reads back only its own
-    unsigned long long* mystage = stage + (size_t)sk * kSpCols + sn;
-    auto stage8 = [&](int J) {
-      const unsigned long long* src = Ub + (long long)(J * kSpK + sk) * ld + ps;
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(mystage + (size_t)j * kSpCols)),
-                     "l"(src + (long long)j * ld)
-                     : "memory");
-      asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    stage8(0);
-    // the tile's pairs in order; block I's epilogue runs after the first pair of block I + 1 is
-    // split (so that block I's last MMAs overlap that work), the last block's at the tile's end
-    int I = 0, J = 0;
-    for (int s = 0; s < npairs && !failed; ++s, ++q) {
-      const int b = (int)(q & 1);
-      if (q >= 2 && give_up(mbar_wait_or_abort(xfree + b, (uint32_t)(((q >> 1) - 1) & 1), abort_flag, A.spin))) {
-        failed = true;
-        break;
-      }
-      const int In = J + 1 <= 2 * I + 1 ? I : I + 1;
-      const int Jn = J + 1 <= 2 * I + 1 ? J + 1 : 0;
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      unsigned long long v[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = mine.valid ? mystage[(size_t)j * kSpCols] : 0ULL;
-      unsigned char* xb = xbuf + (size_t)b * kSpG * kSpBtile;
-      uint32_t pk[4][kSpG];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) sp_digit_pairs(sp_biased(v[2 * j], mine.fe), sp_biased(v[2 * j + 1], mine.fe), pk[j]);
-#pragma unroll
-      for (int a = 0; a < kSpG; ++a)
-        *reinterpret_cast<uint4*>(xb + (size_t)a * kSpBtile + sp_sw128_off(sn, sk)) =
-            make_uint4(pk[0][a], pk[1][a], pk[2][a], pk[3][a]);
-      async_proxy_fence();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(xready + b);
-      if (J == 0) prefetch_block(p0, I);
-      const bool last = s + 1 == npairs;
-      const bool epi = (J == 0 && I > 0) || last;
-      // the next pair's copies only now (the proxy fence above waits for this thread's outstanding
-      // memory operations) and, when an epilogue runs here, once it is done with the staging bytes
-      if (!epi && s + 1 < npairs) stage8(Jn);
-      if (epi) {
-        // epilogue of block I - 1 (or, at the tile's end, of the last block)
-        const int Ie = last ? I : I - 1;
-        // the digit buffer of the pair split before this one: its MMAs completed with block Ie's
-        const int bfree = b ^ 1;
+    long long nblk = 0;
+    for (long long g = blockIdx.x; g < A.ntiles && !failed; g += gridDim.x) {
+      const long long p = g * kSpCols + lane;
+      const int fe0 = p < ld ? __ldg(A.fe + p) : 0, fe1 = p + 32 < ld ? __ldg(A.fe + p + 32) : 0;
+      for (int I = 0; I < nI; ++I, ++nblk) {
+        {  // L2 prefetch of the rows of B that this block's write-back reads, two lines per thread
+          const double* row = A.OUT + (long long)(I * kSpRows + (e >> 1)) * ld;
+          const long long pb = g * kSpCols + (e & 1) * 32;
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(row + min(pb, ld - 1)));
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(row + min(pb + 16, ld - 1)));
+        }
         if (give_up(mbar_wait_or_abort(accdone, (uint32_t)(nblk & 1), abort_flag, A.spin))) {
           failed = true;
           break;
         }
         tc_after_sync();
-        if (!epilogue(p0, Ie, bfree, [&]() {
-              if (s + 1 < npairs) stage8(Jn);
-            })) {
+        const int gfirst = *gfirst_s;
+        sp_f2 h[2][4], l[2][4];
+#pragma unroll
+        for (int c8 = 0; c8 < 2; ++c8) {
+          fold8(ch * 16 + c8 * 8, gfirst, h[0], l[0]);
+          put8(c8, h[0], l[0]);
+        }
+#pragma unroll
+        for (int c8 = 0; c8 < 2; ++c8) fold8(32 + ch * 16 + c8 * 8, gfirst, h[c8], l[c8]);
+        tc_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(accfree);  // this warp is done with the block's accumulators
+        const int m0 = I * kSpRows + ew * 16;
+        if (!meet()) {  // points 0..31 are in the piece
           failed = true;
           break;
         }
-        ++nblk;
+        write16(p, fe0, m0);
+        if (!meet()) {  // every thread is done with them
+          failed = true;
+          break;
+        }
+#pragma unroll
+        for (int c8 = 0; c8 < 2; ++c8) put8(c8, h[c8], l[c8]);
+        if (!meet()) {
+          failed = true;
+          break;
+        }
+        write16(p + 32, fe1, m0);
+        if (!meet()) {  // every thread is done with the piece
+          failed = true;
+          break;
+        }
       }
-      I = In;
-      J = Jn;
+    }
+    if (A.norm != nullptr && !failed) {
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long other = __shfl_xor_sync(0xffffffffu, nmax, o);
+        nmax = other > nmax ? other : nmax;
+      }
+      if (lane == 0) atomicMax(A.norm, nmax);
     }
   }
-  if (A.norm != nullptr && !failed) {
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long other = __shfl_xor_sync(0xffffffffu, nmax, o);
-      nmax = other > nmax ? other : nmax;
-    }
-    if (lane == 0) atomicMax(A.norm, nmax);
-  }
-  asm volatile("cp.async.wait_all;" ::: "memory");  // no staging copy outlives the thread
-  // exit: every consumer warp and the MMA warp arrive (bounded waits everywhere, so all do), the
+  // exit: every split and epilogue warp and the MMA warp arrive (bounded waits everywhere, so all do), the
   // MMA thread's last commit signals that every issued MMA completed, then warp 0 frees TMEM
   tc_before_sync();
   __syncwarp();

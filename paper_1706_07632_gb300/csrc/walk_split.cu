@@ -28,7 +28,7 @@ int split_defect_launch(cudaStream_t st, const SplitArgs& a0, std::string* err) 
     if (err) *err = std::string("split_prep_kernel: ") + cudaGetErrorString(e);
     return 1;
   }
-  a.ns = 4;
+  a.ns = 5;
   const size_t smem = split_smem(a.ns).total + 1024;  // + the alignment of the swizzled tiles
   int occ = 1;
   e = prepare_launch(split_defect_kernel, kSpBlock, smem, g_split_cache, &occ);
