@@ -52,8 +52,10 @@ constexpr int kSpAtile = kSpRows * kSpK * 2;    // bytes of one R~ digit tile
 constexpr int kSpBtile = kSpCols * kSpK * 2;    // bytes of one u digit tile
 constexpr int kSpPieceLd = kSpRows + 1;         // float pairs per point of the epilogue's piece (odd: no bank conflicts)
 
+constexpr int kSpMaxPairs = (kSplitMaxM / kSpRows) * (kSplitMaxM / kSpRows + 1);  // (I, J) blocks at the largest M
+
 struct SplitSmem {
-  size_t ring, xbuf, piece, bar, total;
+  size_t ring, xbuf, piece, bar, pairs, total;
 };
 __host__ __device__ inline SplitSmem split_smem(int ns) {
   SplitSmem s;
@@ -62,8 +64,9 @@ __host__ __device__ inline SplitSmem split_smem(int ns) {
   s.piece = s.xbuf + 2 * (size_t)kSpG * kSpBtile;  // epilogue: [32 points][kSpPieceLd] float pairs
   s.bar = s.piece + (size_t)32 * kSpPieceLd * 8;
   // full[ns], empty[ns], xready[2], xfree[2], accdone, accfree, cbar, exitbar, donebar, then the
-  // abort flag, the lowest group written and the TMEM address
-  s.total = s.bar + 8 * ((size_t)2 * ns + 9) + 16;
+  // abort flag, the lowest group written and the TMEM address; then the pair table
+  s.pairs = s.bar + 8 * ((size_t)2 * ns + 9) + 16;
+  s.total = s.pairs + 8 * (size_t)kSpMaxPairs;
   return s;
 }
 
@@ -132,16 +135,16 @@ __device__ __forceinline__ sp_f2 sp_sub2(sp_f2 a, sp_f2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
-__device__ __forceinline__ sp_f2 sp_mul2(sp_f2 a, sp_f2 b) {
+__device__ __forceinline__ sp_f2 sp_fma2(sp_f2 a, sp_f2 b, sp_f2 c) {
   sp_f2 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
-// (h, l) = a + b exactly (both halves)
-__device__ __forceinline__ void sp_two_sum2(sp_f2 a, sp_f2 b, sp_f2& h, sp_f2& l) {
-  h = sp_add2(a, b);
-  const sp_f2 bb = sp_sub2(h, a);
-  l = sp_add2(sp_sub2(a, sp_sub2(h, bb)), sp_sub2(b, bb));
+// h += a s, its rounding error (exact, s a power of two: TwoSum after Knuth) added to l (both halves)
+__device__ __forceinline__ void sp_two_sum2(sp_f2& h, sp_f2& l, sp_f2 a, sp_f2 s) {
+  const sp_f2 t = sp_fma2(a, s, h), nb = sp_sub2(h, t);  // nb: less what t gained of a s
+  l = sp_add2(l, sp_add2(sp_sub2(h, sp_add2(t, nb)), sp_fma2(a, s, nb)));
+  h = t;
 }
 
 // The balanced base-2^7 digits of an integer |X| <= 2^49, X = sum_b d_b 2^{7(G-1-b)}, d_1..d_6 in
@@ -254,6 +257,10 @@ __global__ void __launch_bounds__(256) split_prep_kernel(const double* __restric
   }
 }
 
+// Order of R~'s digits within a block: digit a takes part in 7 - a products, so long and short ones
+// alternate (0, 6, 1, 5, ...) and any two successive ring slots are held for about the same time.
+__host__ __device__ constexpr int sp_digit_at(int i) { return i & 1 ? kSpG - 1 - i / 2 : i / 2; }
+
 __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_constant__ SplitArgs A) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   // the swizzled operand tiles need 1024-byte aligned addresses (the launcher adds 1 KB)
@@ -275,12 +282,18 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
   volatile int* abort_flag = reinterpret_cast<volatile int*>(accdone + 5);
   volatile int* gfirst_s = abort_flag + 1;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(accdone + 5) + 2;
+  int2* pairs = reinterpret_cast<int2*>(sm + lay.pairs);  // digit mask, first tile
 
   const int t = threadIdx.x;
   const int w = t >> 5;
   const int lane = t & 31;
   const int nI = A.M / kSpRows;
+  const int npairs = nI * (nI + 1);
 
+  for (int i = t; i < npairs; i += kSpBlock) {
+    const int4 pd = __ldg(A.pairs + i);
+    pairs[i] = make_int2(pd.x, pd.y);
+  }
   if (t == 0) {
     for (int s = 0; s < ns; ++s) {
       mbar_init(full + s, 1);
@@ -317,31 +330,34 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
   };
 
   if (w == (kSpSplit + kSpEpi) / 32) {
-    // ---- producer: R~ digit tiles of every pair of every tile of this CTA, in order ----
+    // ---- producer: R~ digit tiles of every pair of every tile of this CTA, in the MMA thread's order ----
     if (lane != 0) return;
     long long k = 0;
     int slot = 0;
+    uint32_t phase = 1;  // of the slot's previous release (the first round finds every slot free)
     bool ok = true, stop = false;
-    const int npairs = nI * (nI + 1);
     for (long long g = blockIdx.x; g < A.ntiles && ok && !stop; g += gridDim.x)
       for (int q = 0; q < npairs && ok && !stop; ++q) {
-        const int4 pd = __ldg(A.pairs + q);
-        int ti = pd.y;
-        for (int a = 0; a < kSpG; ++a) {
+        const int2 pd = pairs[q];
+        for (int ia = 0; ia < kSpG; ++ia) {
+          const int a = sp_digit_at(ia);
           if (!((pd.x >> a) & 1)) continue;
           if (k + 1 == A.withhold) {
             stop = true;
             break;
           }
-          if (k >= ns && !mbar_wait_or_abort(empty + slot, (uint32_t)(((k / ns) - 1) & 1), abort_flag)) {
+          if (!mbar_wait_or_abort(empty + slot, phase, abort_flag)) {
             ok = false;
             break;
           }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          bulk_load(ring + (size_t)slot * kSpAtile, A.At + (size_t)ti * kSpAtile, kSpAtile, full + slot);
-          ++ti;
+          bulk_load(ring + (size_t)slot * kSpAtile, A.At + (size_t)(pd.y + __popc(pd.x & ((1 << a) - 1))) * kSpAtile,
+                    kSpAtile, full + slot);
           ++k;
-          if (++slot == ns) slot = 0;
+          if (++slot == ns) {
+            slot = 0;
+            phase ^= 1;
+          }
         }
       }
     if (!ok) raise();
@@ -355,63 +371,98 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
   if (w == (kSpSplit + kSpEpi) / 32 + 1) {
     // ---- MMA thread ----
     if (lane == 0) {
-      long long k = 0, q = 0, nblk = 0;
+      // descriptors: K-major, 128-byte swizzle; a K step of 16 adds 2 to the address field
+      const uint64_t dbase = sp_desc_sw128(0);
+      const uint32_t ring16 = smem_u32(ring) >> 4, xbuf16 = smem_u32(xbuf) >> 4;
       int slot = 0;
+      uint32_t fphase = 0, accphase = 1, xphase = 0;  // accfree: the first block finds tensor memory free
+      int b = 0;
       bool failed = false;
+      // ng u digits from digit b0 on times the R~ digit in the slot, into the groups from g0 on
+      auto mma = [&](uint32_t bbuf16, int g0, int b0, int ng, bool fresh) {
+        const uint64_t ad = dbase | (uint64_t)(ring16 + (uint32_t)slot * (kSpAtile >> 4));
+        const uint64_t bd = dbase | (uint64_t)(bbuf16 + (uint32_t)b0 * (kSpBtile >> 4));
+        const uint32_t idesc = umma_idesc(ng * kSpCols), d = tmem + 64u * g0;
+#pragma unroll
+        for (int st = 0; st < kSpK / 16; ++st)
+          asm volatile(
+              "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+              " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+              "l"(ad + 2ULL * st), "l"(bd + 2ULL * st), "r"(idesc), "r"(st > 0 || !fresh ? 1u : 0u)
+              : "memory");
+      };
+      auto slot_full = [&]() -> bool {
+        if (!mbar_wait_or_abort(full + slot, fphase, abort_flag, A.spin)) return false;
+        tc_after_sync();
+        return true;
+      };
+      auto slot_done = [&]() {
+        umma_commit(empty + slot);
+        if (++slot == ns) {
+          slot = 0;
+          fphase ^= 1;
+        }
+      };
       for (long long g = blockIdx.x; g < A.ntiles && !failed; g += gridDim.x)
-        for (int I = 0; I < nI && !failed; ++I, ++nblk) {
-          if (nblk > 0 && !mbar_wait_or_abort(accfree, (uint32_t)((nblk - 1) & 1), abort_flag, A.spin)) {
+        for (int I = 0; I < nI && !failed; ++I) {
+          if (!mbar_wait_or_abort(accfree, accphase, abort_flag, A.spin)) {
             failed = true;
             break;
           }
-          tc_after_sync();
+          accphase ^= 1;
           int gfirst = kSpG;  // lowest group this block has written
-          for (int J = 0; J <= 2 * I + 1 && !failed; ++J, ++q) {
-            const int b = (int)(q & 1);
-            if (!mbar_wait_or_abort(xready + b, (uint32_t)((q >> 1) & 1), abort_flag, A.spin)) {
+          for (int J = 0; J <= 2 * I + 1 && !failed; ++J) {
+            const int mask = pairs[I * (I + 1) + J].x;
+            const uint32_t bbuf16 = xbuf16 + (uint32_t)b * (kSpG * kSpBtile >> 4);
+            if (!mbar_wait_or_abort(xready + b, xphase, abort_flag, A.spin)) {
               failed = true;
               break;
             }
             tc_after_sync();
-            const int4 pd = __ldg(A.pairs + I * (I + 1) + J);
-            const uint32_t xb = smem_u32(xbuf + (size_t)b * kSpG * kSpBtile);
-            // operand descriptors: K-major, 128-byte swizzle; a K step of 16 adds 2
-            for (int a = 0; a < kSpG; ++a) {
-              if (!((pd.x >> a) & 1)) continue;
-              if (!mbar_wait_or_abort(full + slot, (uint32_t)((k / ns) & 1), abort_flag, A.spin)) {
-                failed = true;
-                break;
-              }
-              tc_after_sync();
-              const uint64_t adesc = sp_desc_sw128(smem_u32(ring + (size_t)slot * kSpAtile));
-              // digit a meets the u digits 0..6-a in the groups a..6: their tiles are consecutive in
-              // shared memory and the groups in tensor memory, so one MMA covers up to four of them
-              // (N = 256).  The groups touched so far are a suffix gfirst..6, which is accumulated
-              // into; the groups a..gfirst-1 are written afresh.  A 128 x 64 x 16 MMA is bound by its
-              // operand reads (48 cycles for 32 of tensor work) and by its issue (95 cycles seen); ten
-              // wide ones replace 28 per K step, and the sums keep their order (same bits): the defect
-              // of a 511^2 x 512 grid, pre-pass included, 6.47 -> 5.41 ms.
-              for (int g0 = a; g0 < kSpG;) {
-                const bool fresh = g0 < gfirst;
-                const int ng = min(fresh ? gfirst - g0 : kSpG - g0, 4);
-                const uint64_t bdesc = sp_desc_sw128(xb + (uint32_t)(g0 - a) * kSpBtile);
-                const uint32_t idesc = umma_idesc(ng * kSpCols), d = tmem + 64u * g0;
+            // R~ digit a meets the u digits 0..6-a in the groups a..6: their tiles are consecutive in
+            // shared memory and the groups in tensor memory, so one MMA covers up to four of them
+            // (N = 256).  A 128 x 64 x 16 MMA is bound by its operand reads (48 cycles for 32 of tensor
+            // work) and by its issue (95 cycles seen); ten wide ones replace 28 per K step: the defect
+            // of a 511^2 x 512 grid, pre-pass included, 6.47 -> 5.41 ms.
+            if (gfirst == 0) {
+              // every group is written already: all MMAs accumulate, shapes known at compile time
 #pragma unroll
-                for (int st = 0; st < kSpK / 16; ++st)
-                  asm volatile(
-                      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-                      "l"(adesc + 2ULL * st), "l"(bdesc + 2ULL * st), "r"(idesc), "r"(st > 0 || !fresh ? 1u : 0u)
-                      : "memory");
-                g0 += ng;
+              for (int ia = 0; ia < kSpG; ++ia) {
+                const int a = sp_digit_at(ia);
+                if (!((mask >> a) & 1)) continue;
+                if (!slot_full()) {
+                  failed = true;
+                  break;
+                }
+                mma(bbuf16, a, 0, a < 3 ? 4 : kSpG - a, false);
+                if (a < 3) mma(bbuf16, a + 4, 4, 3 - a, false);
+                slot_done();
               }
-              gfirst = min(gfirst, a);
-              umma_commit(empty + slot);
-              ++k;
-              if (++slot == ns) slot = 0;
+            } else {
+              // the groups written so far are a suffix gfirst..6, which is accumulated into; the
+              // groups a..gfirst-1 are written afresh
+#pragma unroll 1
+              for (int ia = 0; ia < kSpG; ++ia) {
+                const int a = sp_digit_at(ia);
+                if (!((mask >> a) & 1)) continue;
+                if (!slot_full()) {
+                  failed = true;
+                  break;
+                }
+                for (int g0 = a; g0 < kSpG;) {
+                  const bool fresh = g0 < gfirst;
+                  const int ng = min(fresh ? gfirst - g0 : kSpG - g0, 4);
+                  mma(bbuf16, g0, g0 - a, ng, fresh);
+                  g0 += ng;
+                }
+                gfirst = min(gfirst, a);
+                slot_done();
+              }
             }
             if (failed) break;
             umma_commit(xfree + b);
+            b ^= 1;
+            xphase ^= b ^ 1;
           }
           if (failed) break;
           *gfirst_s = gfirst;
@@ -544,10 +595,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
 #pragma unroll
         for (int gg = 1; gg < kSpG; ++gg) {
           const uint32_t sc = __float_as_uint(1.f / (float)(1ULL << (7 * gg)));
-          sp_f2 s2, er;
-          sp_two_sum2(h[j], sp_mul2(sp_pack2(r[gg][2 * j], r[gg][2 * j + 1]), sp_pack2(sc, sc)), s2, er);
-          h[j] = s2;
-          l[j] = sp_add2(l[j], er);
+          sp_two_sum2(h[j], l[j], sp_pack2(r[gg][2 * j], r[gg][2 * j + 1]), sp_pack2(sc, sc));
         }
       }
     };
