@@ -140,10 +140,14 @@ __device__ __forceinline__ sp_f2 sp_fma2(sp_f2 a, sp_f2 b, sp_f2 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
-// h += a s, its rounding error (exact, s a power of two: TwoSum after Knuth) added to l (both halves)
-__device__ __forceinline__ void sp_two_sum2(sp_f2& h, sp_f2& l, sp_f2 a, sp_f2 s) {
+// h += a s, its rounding error added to l (both halves), for s = 2^{-7 g}, a an integer of at most 24
+// bits and h a multiple of 2^{-7 (g - 1)}, the groups' sums before g.  Fast2Sum (Dekker) without its
+// condition |h| >= |a s|: with u = ulp(a s) <= 2^{-7 g}, h is a multiple of u, so where |h| < |a s| the
+// sum is a multiple of u below 2^25 u, its error is 0 or u, t - h = a s + error fits 24 bits and both
+// subtractions are exact.
+__device__ __forceinline__ void sp_accum2(sp_f2& h, sp_f2& l, sp_f2 a, sp_f2 s) {
   const sp_f2 t = sp_fma2(a, s, h), nb = sp_sub2(h, t);  // nb: less what t gained of a s
-  l = sp_add2(l, sp_add2(sp_sub2(h, sp_add2(t, nb)), sp_fma2(a, s, nb)));
+  l = sp_add2(l, sp_fma2(a, s, nb));
   h = t;
 }
 
@@ -330,7 +334,8 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
   };
 
   if (w == (kSpSplit + kSpEpi) / 32) {
-    // ---- producer: R~ digit tiles of every pair of every tile of this CTA, in the MMA thread's order ----
+    // ---- producer: R~ digit tiles of every pair of every tile of this CTA, in the MMA thread's order
+    // (a slot is only ever read by MMAs and written by bulk copies, both of the async proxy) ----
     if (lane != 0) return;
     long long k = 0;
     int slot = 0;
@@ -350,7 +355,6 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
             ok = false;
             break;
           }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           bulk_load(ring + (size_t)slot * kSpAtile, A.At + (size_t)(pd.y + __popc(pd.x & ((1 << a) - 1))) * kSpAtile,
                     kSpAtile, full + slot);
           ++k;
@@ -595,7 +599,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
 #pragma unroll
         for (int gg = 1; gg < kSpG; ++gg) {
           const uint32_t sc = __float_as_uint(1.f / (float)(1ULL << (7 * gg)));
-          sp_two_sum2(h[j], l[j], sp_pack2(r[gg][2 * j], r[gg][2 * j + 1]), sp_pack2(sc, sc));
+          sp_accum2(h[j], l[j], sp_pack2(r[gg][2 * j], r[gg][2 * j + 1]), sp_pack2(sc, sc));
         }
       }
     };
