@@ -261,6 +261,13 @@ __global__ void __launch_bounds__(256) split_prep_kernel(const double* __restric
   }
 }
 
+// one lane of a converged warp
+__device__ __forceinline__ bool sp_elect() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+
 // Order of R~'s digits within a block: digit a takes part in 7 - a products, so long and short ones
 // alternate (0, 6, 1, 5, ...) and any two successive ring slots are held for about the same time.
 __host__ __device__ constexpr int sp_digit_at(int i) { return i & 1 ? kSpG - 1 - i / 2 : i / 2; }
@@ -373,8 +380,11 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
   }
 
   if (w == (kSpSplit + kSpEpi) / 32 + 1) {
-    // ---- MMA thread ----
-    if (lane == 0) {
+    // ---- MMA warp: every lane runs the loop, so that the descriptors stay in uniform registers; one
+    // elected lane issues ----
+    {
+      const bool leader = sp_elect();
+      const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
       // descriptors: K-major, 128-byte swizzle; a K step of 16 adds 2 to the address field
       const uint64_t dbase = sp_desc_sw128(0);
       const uint32_t ring16 = smem_u32(ring) >> 4, xbuf16 = smem_u32(xbuf) >> 4;
@@ -386,7 +396,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
       auto mma = [&](uint32_t bbuf16, int g0, int b0, int ng, bool fresh) {
         const uint64_t ad = dbase | (uint64_t)(ring16 + (uint32_t)slot * (kSpAtile >> 4));
         const uint64_t bd = dbase | (uint64_t)(bbuf16 + (uint32_t)b0 * (kSpBtile >> 4));
-        const uint32_t idesc = umma_idesc(ng * kSpCols), d = tmem + 64u * g0;
+        const uint32_t idesc = umma_idesc(ng * kSpCols), d = tm + 64u * g0;
 #pragma unroll
         for (int st = 0; st < kSpK / 16; ++st)
           asm volatile(
@@ -396,12 +406,12 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
               : "memory");
       };
       auto slot_full = [&]() -> bool {
-        if (!mbar_wait_or_abort(full + slot, fphase, abort_flag, A.spin)) return false;
+        if (!__all_sync(0xffffffffu, mbar_wait_or_abort(full + slot, fphase, abort_flag, A.spin))) return false;
         tc_after_sync();
         return true;
       };
       auto slot_done = [&]() {
-        umma_commit(empty + slot);
+        if (leader) umma_commit(empty + slot);
         if (++slot == ns) {
           slot = 0;
           fphase ^= 1;
@@ -409,7 +419,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
       };
       for (long long g = blockIdx.x; g < A.ntiles && !failed; g += gridDim.x)
         for (int I = 0; I < nI && !failed; ++I) {
-          if (!mbar_wait_or_abort(accfree, accphase, abort_flag, A.spin)) {
+          if (!__all_sync(0xffffffffu, mbar_wait_or_abort(accfree, accphase, abort_flag, A.spin))) {
             failed = true;
             break;
           }
@@ -418,7 +428,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
           for (int J = 0; J <= 2 * I + 1 && !failed; ++J) {
             const int mask = pairs[I * (I + 1) + J].x;
             const uint32_t bbuf16 = xbuf16 + (uint32_t)b * (kSpG * kSpBtile >> 4);
-            if (!mbar_wait_or_abort(xready + b, xphase, abort_flag, A.spin)) {
+            if (!__all_sync(0xffffffffu, mbar_wait_or_abort(xready + b, xphase, abort_flag, A.spin))) {
               failed = true;
               break;
             }
@@ -438,8 +448,10 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
                   failed = true;
                   break;
                 }
-                mma(bbuf16, a, 0, a < 3 ? 4 : kSpG - a, false);
-                if (a < 3) mma(bbuf16, a + 4, 4, 3 - a, false);
+                if (leader) {
+                  mma(bbuf16, a, 0, a < 3 ? 4 : kSpG - a, false);
+                  if (a < 3) mma(bbuf16, a + 4, 4, 3 - a, false);
+                }
                 slot_done();
               }
             } else {
@@ -456,7 +468,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
                 for (int g0 = a; g0 < kSpG;) {
                   const bool fresh = g0 < gfirst;
                   const int ng = min(fresh ? gfirst - g0 : kSpG - g0, 4);
-                  mma(bbuf16, g0, g0 - a, ng, fresh);
+                  if (leader) mma(bbuf16, g0, g0 - a, ng, fresh);
                   g0 += ng;
                 }
                 gfirst = min(gfirst, a);
@@ -464,17 +476,21 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
               }
             }
             if (failed) break;
-            umma_commit(xfree + b);
+            if (leader) umma_commit(xfree + b);
             b ^= 1;
             xphase ^= b ^ 1;
           }
           if (failed) break;
-          *gfirst_s = gfirst;
-          umma_commit(accdone);
-          mbar_arrive(accdone);  // release: the lowest group is visible to the epilogue after its wait
+          if (leader) {
+            *gfirst_s = gfirst;
+            umma_commit(accdone);
+            mbar_arrive(accdone);  // release: the lowest group is visible to the epilogue after its wait
+          }
         }
-      if (failed) raise();
-      umma_commit(donebar);  // completes when every MMA issued above has completed
+      if (leader) {
+        if (failed) raise();
+        umma_commit(donebar);  // completes when every MMA issued above has completed
+      }
     }
     __syncwarp();
     tc_before_sync();
