@@ -87,28 +87,6 @@ __device__ __forceinline__ uint64_t sp_desc_sw128(uint32_t addr) {
 
 // ---- integer views of FP64 values (no FP64 arithmetic) ----
 
-// round(|x| * 2^-s) for the 53-bit significand mt of x, s >= -7 (left shift) .. (>= 64: 0)
-__device__ __forceinline__ long long sp_shift_round(unsigned long long mt, int s) {
-  if (s <= 0) return (long long)(mt << (-s));
-  if (s >= 64) return 0;
-  return (long long)((mt + (1ULL << (s - 1))) >> s);
-}
-
-// round(x 2^{1075 - shift_base}) for the FP64 value x given by its bits (biased exponent e,
-// significand mt: x = mt 2^{e - 1075}, so the result is round(mt 2^{e - shift_base})); subnormals as 0
-__device__ __forceinline__ long long sp_fixed(unsigned long long bits, int shift_base) {
-  const int e = (int)((bits >> 52) & 0x7FF);
-  if (e == 0) return 0;
-  const unsigned long long mt = (bits & 0xFFFFFFFFFFFFFULL) | (1ULL << 52);
-  const long long v = sp_shift_round(mt, shift_base - e);
-  return (bits >> 63) ? -v : v;
-}
-
-// float 2^k (0 below the normal range, clamped at 2^127)
-__device__ __forceinline__ float sp_pow2f(int k) {
-  return k < -126 ? 0.f : __int_as_float((min(k, 127) + 127) << 23);
-}
-
 // FP64 value of float f times 2^k, exactly, by integer operations (a conversion runs on the 1/64-rate
 // FP64 pipe); f subnormal and results below the FP64 normal range: 0, above it: Inf
 __device__ __forceinline__ double sp_f2d_scaled(float f, int k) {
@@ -191,74 +169,96 @@ __device__ __forceinline__ void sp_digit_pairs(long long y0, long long y1, uint3
   pk[0] = __byte_perm(f0, f1, 0x7632);
 }
 
-// FP64 value of the integer D times 2^k (D exact up to 53 bits, else rounded half up), by integer
-// operations; 0 below the FP64 normal range
-__device__ __forceinline__ double sp_ll2d(long long D, int k) {
-  if (D == 0) return 0.0;
-  const unsigned long long sign = D < 0 ? (1ULL << 63) : 0ULL;
-  unsigned long long a = (unsigned long long)(D < 0 ? -D : D);
-  int msb = 63 - __clzll((long long)a);
-  if (msb <= 52) {
-    a <<= (52 - msb);
-  } else {
-    const int sh = msb - 52;
-    a = (a + (1ULL << (sh - 1))) >> sh;
-    if (a >> 53) {
-      a >>= 1;
-      ++msb;
-    }
+// S = cd c - x0 - x1 (- x2 - x3) (cd = 2 NX), the undivided stencil of FP64 values, in 64-bit fixed
+// point relative to the largest of them: each value's significand, 6 bits up, shifted right by its
+// distance from the largest exponent (truncated towards -inf within 2^-59 of the largest value, so
+// S is within 2^-55 of it; the FP64 subtractions would be within a few 2^-53), the sum widened to FP64
+// by one conversion.  Zeros and negligible values shift out.  Outside the middle of the exponent
+// range, and for Inf and NaN, the FP64 subtractions themselves.
+template <int NX>
+__device__ __forceinline__ double sp_stencil(unsigned long long c, const unsigned long long (&x)[NX]) {
+  auto ex = [](unsigned long long b) { return (uint32_t)(b >> 32) & 0x7FF00000u; };
+  uint32_t q = ex(c);
+#pragma unroll
+  for (int i = 0; i < NX; ++i) q = max(q, ex(x[i]));
+  if (q - (64u << 20) >= (1976u << 20)) {
+    auto d = [](unsigned long long b) { return __longlong_as_double((long long)b); };
+    const double t = fma((double)NX, d(c), -d(x[0])) - d(x[1]);
+    return NX == 4 ? t - (d(x[NX - 2]) + d(x[NX - 1])) : t;
   }
-  const long long ed = (long long)msb + k + 1023;
-  if (ed <= 0) return 0.0;
-  if (ed >= 2047) return __longlong_as_double((long long)(sign | 0x7FF0000000000000ULL));
-  return __longlong_as_double((long long)(sign | ((unsigned long long)ed << 52) | (a & 0xFFFFFFFFFFFFFULL)));
+  auto fixed = [&](unsigned long long b, int up) -> long long {
+    unsigned long long m = ((b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52)) << up;
+    asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"((q - ex(b)) >> 20));  // shifts past 63 give 0
+    return (long long)m ^ ((long long)b >> 63);
+  };
+  long long D = fixed(c, NX == 4 ? 8 : 7);
+#pragma unroll
+  for (int i = 0; i < NX; ++i) D -= fixed(x[i], 6);
+  const double s = (double)D;  // times 2^{q - 1081}: exponent field added
+  const int hi = __double2hiint(s);
+  return __hiloint2double(hi == 0 ? 0 : hi + (int)(q - (1081u << 20)), __double2loint(s));
 }
 
-// Pre-pass, one thread per grid point (grid-stride), over the M time levels: fe[p] = the largest
-// biased exponent of u at p, and B = F - A_h u written to B -- the defect kernel then subtracts R~ u
-// in place.  The stencil needs FP64 accuracy (at N = 4095 it cancels 2^24-fold).  Two time levels in
-// three form it with FP64 FMAs and subtractions (a few 2^-53 of |A_h| |u|); the third exactly in
-// 64-bit fixed point relative to the largest of its five values (59 bits), converted by integer
-// operations -- so the FP64 pipe (1/64 of the FP32 rate on GB300) and the integer pipe share the work
-// -- and both end with one FMA, B = F - S / h^2.  An Inf or NaN in u or F propagates.
-__global__ void __launch_bounds__(256) split_prep_kernel(const double* __restrict__ U, const double* __restrict__ F,
-                                                         double* __restrict__ B, int* __restrict__ fe, long long ld,
-                                                         int M, int dim, int N, double ih) {
-  const unsigned long long* u = reinterpret_cast<const unsigned long long*>(U);
-  const double cdiag = dim == 2 ? 4.0 : 2.0;
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < ld; p += (long long)gridDim.x * blockDim.x) {
-    const int ix = dim == 2 ? (int)(p % N) : (int)p;
-    const int iy = dim == 2 ? (int)(p / N) : 0;
-    const long long o0 = ix > 0 ? p - 1 : p, o1 = ix < N - 1 ? p + 1 : p;
-    const long long o2 = (dim == 2 && iy > 0) ? p - N : p, o3 = (dim == 2 && iy < N - 1) ? p + N : p;
-    const unsigned long long k0 = ix > 0 ? ~0ULL : 0ULL, k1 = ix < N - 1 ? ~0ULL : 0ULL;
-    const unsigned long long k2 = (dim == 2 && iy > 0) ? ~0ULL : 0ULL, k3 = (dim == 2 && iy < N - 1) ? ~0ULL : 0ULL;
-    unsigned int mx = 0;
-#pragma unroll 3
-    for (int m = 0; m < M; ++m) {
-      const long long r = (long long)m * ld;
-      const unsigned long long bc = __ldg(u + r + p);
-      const unsigned long long x0 = __ldg(u + r + o0) & k0, x1 = __ldg(u + r + o1) & k1;
-      const unsigned long long x2 = __ldg(u + r + o2) & k2, x3 = __ldg(u + r + o3) & k3;
-      auto ex = [](unsigned long long b) { return (int)((b >> 52) & 0x7FF); };
-      mx = max(mx, (unsigned int)ex(bc));
-      double S;
-      if (m % 3 != 2) {
-        auto d = [](unsigned long long b) { return __longlong_as_double((long long)b); };
-        const double t = fma(cdiag, d(bc), -d(x0));
-        S = (t - d(x1)) - (d(x2) + d(x3));
-      } else {
-        // X = round(u 2^{59 - (ql - 1022)}) = round(mt 2^{e - ql + 6}); |D| < 2^62
-        const int ql = max(max(ex(bc), ex(x0)), max(max(ex(x1), ex(x2)), ex(x3)));
-        const int sb = ql - 6;
-        const long long D = (dim == 2 ? 4 : 2) * sp_fixed(bc, sb) - sp_fixed(x0, sb) - sp_fixed(x1, sb) -
-                            sp_fixed(x2, sb) - sp_fixed(x3, sb);
-        S = ql == 2047 ? __longlong_as_double(0x7FF8000000000000LL) : sp_ll2d(D, ql - 1022 - 59);
-      }
-      B[r + p] = fma(-ih, S, __ldg(F + r + p));
+constexpr int kPrepThreads = 256, kPrepM = 32;  // threads along a grid row; time levels per block
+
+// Pre-pass: fe[p] = the largest biased exponent of u at p (zeroed by the launcher), and B = F - A_h u
+// written to B -- the defect kernel then subtracts R~ u in place.  The stencil needs FP64 accuracy (at
+// N = 4095 it cancels 2^24-fold), but FP64 runs at 1/64 of the FP32 rate: it is formed in integers
+// (sp_stencil) and costs a conversion and a multiply-add of that pipe instead of five operations.  A
+// thread takes RY points of a column of the grid (their rows are loaded once) and kPrepM time levels.
+// Bound by HBM (24 bytes per value) and the issue of ~90 instructions per value; 511^2 x 512: 1.17 ms
+// with one thread per grid point and two thirds of the levels in FP64, 0.70 ms now (0.84 with four rows).
+template <int DIM, int RY>
+__global__ void __launch_bounds__(kPrepThreads) split_prep_kernel(const double* __restrict__ U,
+                                                                  const double* __restrict__ F, double* __restrict__ B,
+                                                                  int* __restrict__ fe, long long ld, int M, int N,
+                                                                  double ih) {
+  const int x = blockIdx.x * kPrepThreads + threadIdx.x, y0 = blockIdx.y * RY;
+  if (x >= N) return;
+  const unsigned long long kl = x > 0 ? ~0ULL : 0ULL, kr = x < N - 1 ? ~0ULL : 0ULL;
+  const int ol = x > 0 ? -1 : 0, orr = x < N - 1 ? 1 : 0;
+  const int ny = DIM == 2 ? min(RY, N - y0) : 1;
+  uint32_t mx[RY];
+#pragma unroll
+  for (int r = 0; r < RY; ++r) mx[r] = 0;
+  const int m1 = min(M, (int)(blockIdx.z + 1) * kPrepM);
+  for (int m = blockIdx.z * kPrepM; m < m1; ++m) {
+    const long long o = (long long)m * ld + (long long)y0 * N + x;
+    const unsigned long long* u = reinterpret_cast<const unsigned long long*>(U) + o;
+    unsigned long long c[RY + 2];  // the column: rows y0 - 1 .. y0 + RY
+    unsigned long long xl[RY], xr[RY];
+    double f[RY];
+#pragma unroll
+    for (int r = 0; r < RY; ++r) {
+      const bool in = r < ny;
+      const long long q = (long long)r * N;
+      c[r + 1] = in ? __ldg(u + q) : 0ULL;
+      xl[r] = in ? __ldg(u + q + ol) & kl : 0ULL;
+      xr[r] = in ? __ldg(u + q + orr) & kr : 0ULL;
+      f[r] = in ? __ldg(F + o + q) : 0.0;
     }
-    fe[p] = (int)mx;
+    if (DIM == 2) {
+      c[0] = y0 > 0 ? __ldg(u - N) : 0ULL;
+      if (ny == RY) c[RY + 1] = y0 + RY < N ? __ldg(u + (long long)RY * N) : 0ULL;
+    }
+#pragma unroll
+    for (int r = 0; r < RY; ++r) {
+      if (r >= ny) break;
+      mx[r] = max(mx[r], (uint32_t)(c[r + 1] >> 32) & 0x7FF00000u);
+      double S;
+      if (DIM == 2) {
+        const unsigned long long nb[4] = {xl[r], xr[r], c[r], c[r + 2]};  // rows past the grid hold zeros
+        S = sp_stencil<4>(c[r + 1], nb);
+      } else {
+        const unsigned long long nb[2] = {xl[r], xr[r]};
+        S = sp_stencil<2>(c[r + 1], nb);
+      }
+      B[o + (long long)r * N] = fma(-ih, S, f[r]);
+    }
   }
+#pragma unroll
+  for (int r = 0; r < RY; ++r)
+    if (r < ny) atomicMax(fe + (long long)(y0 + r) * N + x, (int)(mx[r] >> 20));
 }
 
 // one lane of a converged warp

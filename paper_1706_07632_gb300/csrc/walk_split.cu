@@ -8,6 +8,7 @@
 namespace fhmg {
 
 namespace {
+constexpr int kPrepRows = 2;  // grid rows per thread of the pre-pass (2D)
 KernelCache g_split_cache;
 }
 
@@ -21,9 +22,17 @@ int split_defect_launch(cudaStream_t st, const SplitArgs& a0, std::string* err) 
   a.ntiles = (a.ld + kSpCols - 1) / kSpCols;
   if (a.spin <= 0) a.spin = kSpinLimit;
   const int sms = device_sms();
-  // the exponents of u per grid point and B = F - A_h u into OUT (one pass, grid-stride)
-  split_prep_kernel<<<grid_for(a.ld, 8), 256, 0, st>>>(a.U, a.F, a.OUT, a.fe, a.ld, a.M, a.dim, a.N, a.inv_h2);
-  cudaError_t e = cudaGetLastError();
+  // the exponents of u per grid point and B = F - A_h u into OUT
+  cudaError_t e = cudaMemsetAsync(a.fe, 0, sizeof(int) * a.ld, st);
+  if (e == cudaSuccess) {
+    const unsigned bx = (a.N + kPrepThreads - 1) / kPrepThreads, bz = (a.M + kPrepM - 1) / kPrepM;
+    if (a.dim == 2)
+      split_prep_kernel<2, kPrepRows><<<dim3(bx, (a.N + kPrepRows - 1) / kPrepRows, bz), kPrepThreads, 0, st>>>(
+          a.U, a.F, a.OUT, a.fe, a.ld, a.M, a.N, a.inv_h2);
+    else
+      split_prep_kernel<1, 1><<<dim3(bx, 1, bz), kPrepThreads, 0, st>>>(a.U, a.F, a.OUT, a.fe, a.ld, a.M, a.N, a.inv_h2);
+    e = cudaGetLastError();
+  }
   if (e != cudaSuccess) {
     if (err) *err = std::string("split_prep_kernel: ") + cudaGetErrorString(e);
     return 1;
