@@ -30,8 +30,8 @@
 namespace fhmg {
 
 constexpr int kUmmaCols = 128;                 // columns per tile = MMA M = TMEM lanes
-constexpr int kUmmaBlock = kUmmaCols + 32;     // consumer threads + producer warp
-constexpr uint32_t kUmmaTmemCols = 256;        // acc [0,64), res [64,128), v [128,192)
+constexpr int kUmmaBlock = 2 * kUmmaCols + 32;  // walk threads, memory threads, producer warp
+constexpr uint32_t kUmmaTmemCols = 256;        // acc / res [0,64), v [64,128), two leaf buffers [128,256)
 
 struct UmmaSmem {
   size_t ring, ystage, zstage, zpool, bar, ebar, cbar, xbar, desc, flag, tslot, total;
@@ -51,8 +51,8 @@ __host__ __device__ inline UmmaSmem umma_smem(int pool, int W, int slot_bytes, i
   s.bar = a128(s.zpool + (size_t)pool * kUmmaCols * 4);
   s.ebar = s.bar + 8 * (size_t)ns;
   s.cbar = s.ebar + 8 * (size_t)ns;  // consumer warps' barrier
-  s.xbar = s.cbar + 8;               // acc, res, v (MMA completion), exit (consumer warps), done
-  s.desc = (s.xbar + 5 * 8 + 15) & ~(size_t)15;
+  s.xbar = s.cbar + 8;               // acc, res, v (MMA completion), exit, done, leaf buffers: filled[2], walked[2]
+  s.desc = (s.xbar + 9 * 8 + 15) & ~(size_t)15;
   s.flag = s.desc + 16 * (size_t)ns;
   s.tslot = s.flag + 16;
   s.total = a128(s.tslot + 16);
@@ -111,8 +111,12 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  // the loaded registers are read only after the wait
 #pragma unroll
-  for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+  for (int j = 0; j < 16; ++j) {
+    asm volatile("" : "+r"(r[j]));
+    v[j] = __uint_as_float(r[j]);
+  }
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
@@ -136,10 +140,61 @@ __device__ __forceinline__ void put8_packed(unsigned char* tile, int c, int k0, 
   *reinterpret_cast<uint4*>(tile + umma_off(c, k0, K)) = make_uint4(q[0], q[1], q[2], q[3]);
 }
 
+// 16 consecutive TMEM columns of this thread's lane written
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) {
+  uint32_t r[16];
+#pragma unroll
+  for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(v[j]);
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};" ::"r"(r[0]),
+      "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]),
+      "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};" ::"r"(r[0]), "r"(r[1]), "r"(r[2]),
+               "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(taddr)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// a load of data that no thread writes during the launch, kept in program order with its like (so that
+// a group of loads is in flight before the first use)
+__device__ __forceinline__ float ld_nc(const float* p) {
+  float v;
+  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+
+// one lane of a converged warp
+__device__ __forceinline__ bool umma_elect() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+
+// Columns of a 2D colour in tiles of 4 grid rows x 32 points of the colour (64 grid points), thread c
+// point c % 32 of row c / 32: the rows above and below a row are then read by the same CTA, twice
+// instead of three times from L2 (20 instead of 32 bytes per value)
+__host__ __device__ inline long long umma_tiles(const Geo& g, long long ncols) {
+  if (g.dim != 2) return (ncols + kUmmaCols - 1) / kUmmaCols;
+  return (long long)((g.N + 3) / 4) * (((g.N + 1) / 2 + 31) / 32);
+}
+
 // T = float grid functions; the jobs' Dinv are the level inverses (without diagonal) in the
 // build_panel_umma layout (BF16 bits), ddiag the diagonal applied in FP32.
+//
+// Three roles: four walk warps (the chunk products), four memory warps (thread c: column c, as in the
+// walk) and a producer warp (the chunk stream).  The memory warps run ahead of the walk through two
+// leaf buffers in tensor memory (64 columns each): they load a leaf's right-hand side (smoother: F +
+// neighbour sum / h^2; product: x, as BF16 pairs) into one while the walk works on the other, and
+// write the leaf's result (x; B - d x - sum) back once the walk has left it there.  The walk then
+// never waits for DRAM, which took most of its time when its own threads loaded the next leaf
+// (2.37 ms per finest half-sweep of a 1023^2 x 512 grid, 2.31 ms now, the traffic between L2 and the SMs
+// bounding it; 214 -> 176 us for a line solve of 100003 x 512 columns).  96 registers and 112 KB of shared
+// memory: two CTAs per SM.
 template <int MODE>
-__global__ void __maxnreg__(168) humma_kernel(const __grid_constant__ WalkBatch<float, uint16_t> B) {
+__global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_constant__ WalkBatch<float, uint16_t> B) {
   constexpr int L = kUmmaL, NT = kUmmaCols;
   extern __shared__ __align__(16) unsigned char sm[];
   const UmmaSmem lay = umma_smem(B.pool, B.W, B.slot_bytes, B.ns);
@@ -156,6 +211,8 @@ __global__ void __maxnreg__(168) humma_kernel(const __grid_constant__ WalkBatch<
   uint64_t* vbar = accbar + 2;
   uint64_t* exitbar = accbar + 3;
   uint64_t* donebar = accbar + 4;
+  uint64_t* filled = accbar + 5;  // [2] a leaf buffer holds a leaf's input
+  uint64_t* walked = accbar + 7;  // [2] ... its result
   int4* sdesc = reinterpret_cast<int4*>(sm + lay.desc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + lay.flag);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + lay.tslot);
@@ -170,10 +227,10 @@ __global__ void __maxnreg__(168) humma_kernel(const __grid_constant__ WalkBatch<
   if (t == 0) {
     for (int s = 0; s < ns; ++s) {
       mbar_init(full + s, 1);
-      mbar_init(empty + s, NT / 32 + 1);  // every consumer warp + the MMAs' commit
+      mbar_init(empty + s, NT / 32 + 1);  // every walk warp + the MMAs' commit
     }
     mbar_init(cbar, NT / 32);
-    for (int b = 0; b < 5; ++b) mbar_init(accbar + b, b == 3 ? NT / 32 : 1);
+    for (int b = 0; b < 9; ++b) mbar_init(accbar + b, b == 3 ? 2 * NT / 32 : b >= 5 ? NT / 32 : 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -187,11 +244,12 @@ __global__ void __maxnreg__(168) humma_kernel(const __grid_constant__ WalkBatch<
   tc_after_sync();
   const uint32_t tmem = *tslot;
 
-  if (t >= NT) {
+  if (t >= 2 * NT) {
     // ---- producer: one lane streams every chunk of every tile of this CTA, in order ----
-    if (t != NT) return;
+    if (t != 2 * NT) return;
     long long k = 0;
     int slot = 0;
+    uint32_t phase = 1;  // of the slot's previous release (the first round finds every slot free)
     bool ok = true, stop = false;
     for (long long g = blockIdx.x; g < B.ntiles && ok && !stop; g += gridDim.x) {
       const WalkJob<float, uint16_t>& J = B.job[job_of(B, g)];
@@ -204,7 +262,7 @@ __global__ void __maxnreg__(168) humma_kernel(const __grid_constant__ WalkBatch<
           stop = true;
           break;
         }
-        if (k >= ns && !mbar_wait_or_abort(empty + slot, (uint32_t)(((k / ns) - 1) & 1), abort_flag)) {
+        if (!mbar_wait_or_abort(empty + slot, phase, abort_flag)) {
           ok = false;
           break;
         }
@@ -214,7 +272,10 @@ __global__ void __maxnreg__(168) humma_kernel(const __grid_constant__ WalkBatch<
                                                                     : (const void*)(J.P.pkg + 16LL * (long long)cd.w);
         sdesc[slot] = cd;
         bulk_load(slots + (size_t)slot * B.slot_bytes, src, (uint32_t)cd.z, full + slot);
-        if (++slot == ns) slot = 0;
+        if (++slot == ns) {
+          slot = 0;
+          phase ^= 1;
+        }
       }
     }
     if (!ok && !*abort_flag) {
@@ -228,15 +289,9 @@ __global__ void __maxnreg__(168) humma_kernel(const __grid_constant__ WalkBatch<
     return;
   }
 
-  // ---- consumers: thread c owns column c of the tile ----
-  const int c = t;
-  const bool issuer = t == 0;
-  const uint32_t t_acc = tmem, t_res = tmem + 64, t_v = tmem + 128;
-  const uint32_t lane_base = (uint32_t)(32 * w) << 16;  // this warp's TMEM lane quarter
-  uint32_t cbphase = 0, accph = 0, resph = 0, vph = 0;
-  int cslot = 0;
-  uint32_t cphase = 0;
-  bool failed = false;
+  const uint32_t lane_base = (uint32_t)(32 * (w & 3)) << 16;  // this warp's TMEM lane quarter
+  const uint32_t t_acc = tmem, t_v = tmem + 64;
+  const uint32_t t_buf = tmem + 128 + lane_base;  // + 64 * (leaf & 1)
   auto give_up = [&](bool ok) -> bool {
     if (__all_sync(0xffffffffu, ok)) return false;
     if (lane == 0) {
@@ -245,176 +300,357 @@ __global__ void __maxnreg__(168) humma_kernel(const __grid_constant__ WalkBatch<
     }
     return true;
   };
-  // all consumer warps meet (bounded); tensor-memory reads and shared writes before it are ordered
-  // before the MMAs issued after it
-  // arrive_wait: the same meeting without the fences, for callers that fenced already and issued
-  // global loads since (a proxy fence would wait for those loads to complete)
-  auto arrive_wait = [&]() -> bool {
-    __syncwarp();
-    if (lane == 0) mbar_arrive(cbar);
-    const bool ok = mbar_wait_or_abort(cbar, cbphase, abort_flag, B.spin);
-    cbphase ^= 1;
-    tc_after_sync();
-    return !give_up(ok);
-  };
-  auto consumer_sync = [&]() -> bool {
-    async_proxy_fence();
-    tc_before_sync();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(cbar);
-    const bool ok = mbar_wait_or_abort(cbar, cbphase, abort_flag, B.spin);
-    cbphase ^= 1;
-    tc_after_sync();
-    return !give_up(ok);
-  };
-  auto wait_mma = [&](uint64_t* bar, uint32_t& ph) -> bool {
-    const bool ok = mbar_wait_or_abort(bar, ph, abort_flag, B.spin);
-    ph ^= 1;
-    tc_after_sync();
-    return !give_up(ok);
-  };
 
-  for (long long g = blockIdx.x; g < B.ntiles && !failed; g += gridDim.x) {
-    const WalkJob<float, uint16_t>& J = B.job[job_of(B, g)];
-    const long long cg = (g - J.tile0) * NT + c;
-    const bool valid = cg < J.ncols;
-    const long long ld = J.geo.ld;
-    const float inv_h2 = (float)J.geo.inv_h2;
-    float* X = J.X;
-    const float* Bsrc = J.B;
-    const float* ddg = J.ddiag;
-    const int nb = J.P.nb;
-    long long p = 0;
-    long long nbr[4] = {-1, -1, -1, -1};
-    if (valid) {
-      if (MODE == MODE_SMOOTH && J.geo.dim > 0) {
-        int iy, ix;
-        p = colour_pos(J.geo.dim, J.geo.N, J.geo.colour, cg, &iy, &ix);
-        nbr[0] = ix > 0 ? p - 1 : -1;
-        nbr[1] = ix < J.geo.N - 1 ? p + 1 : -1;
-        if (J.geo.dim == 2) {
-          nbr[2] = iy > 0 ? p - J.geo.N : -1;
-          nbr[3] = iy < J.geo.N - 1 ? p + J.geo.N : -1;
-        }
-      } else {
-        p = cg;
-      }
-    }
+  if (t >= NT) {
+    // ---- memory warps ----
+    const int c = t - NT;
+    bool failed = false;
+    long long n = 0;  // leaves filled so far (over all tiles); leaf n uses buffer n & 1
     double local_max = 0.0;
-    // right-hand side of a leaf (smoother: F + neighbour sum / h^2) and, for the product, its x;
-    // loaded one leaf ahead (issued right after the previous leaf's diagonal step, the last use of
-    // these registers), so the loads overlap that leaf's V products and this leaf's first MMAs.
-    // Rows of leaf i + 1 are never written during leaf i (X, OUT alias B only row by row).
-    // b: right-hand side (product: B - d_rr x, the diagonal term folded in at load time);
-    // xq: the product's x_i as packed BF16 pairs for the ring
-    float b[L];
-    uint32_t xq[MODE == MODE_MATVEC ? L / 2 : 1];
-    // columns past the panel's end read column 0 (any valid address) and are zeroed, so that the
-    // loads carry no predicate; compact columns load their 64 values as independent loads, grid
-    // columns in groups of 8 rows (5 loads per row: the point and its neighbours), which bounds
-    // the registers the loads in flight hold
-    const long long pa = valid ? p : 0;
-    const float keep = valid ? 1.f : 0.f;
-    const bool grid = MODE == MODE_SMOOTH && J.geo.dim > 0;
-    auto load_leaf = [&](int leaf) {
-      if (leaf >= nb) return;
-      const float* Bl = Bsrc + (long long)leaf * L * ld + pa;
-      if (!grid) {
+    // where the leaves in the two buffers go (the even one and the odd one)
+    struct Dest {
+      const WalkJob<float, uint16_t>* J;
+      long long at;  // element offset of the leaf's first row
+      int leaf;
+      bool valid;
+    };
+    Dest d0{nullptr, 0, 0, false}, d1{nullptr, 0, 0, false};
+    // the result of leaf m (in buffer m & 1) to global memory
+    auto write_leaf = [&](long long m) -> bool {
+      const int buf = (int)(m & 1);
+      if (give_up(mbar_wait_or_abort(walked + buf, (uint32_t)((m >> 1) & 1), abort_flag, B.spin))) return false;
+      tc_after_sync();
+      const Dest d = buf ? d1 : d0;
+      const long long ld = d.J->geo.ld;
 #pragma unroll
-        for (int r = 0; r < L; ++r) b[r] = Bl[(long long)r * ld] * keep;
-        if (MODE == MODE_MATVEC) {
-          const float* Xl = X + (long long)leaf * L * ld + pa;
-          const float* dd = ddg + (long long)leaf * L;
+      for (int r0 = 0; r0 < L; r0 += 16) {
+        float a[16];
+        tmem_ld16(t_buf + 64 * buf + r0, a);
+        if (MODE == MODE_SMOOTH) {
+          if (d.valid) {
+            float* x = d.J->X + d.at + (long long)r0 * ld;
 #pragma unroll
-          for (int r = 0; r < L; r += 2) {
-            const float x0 = Xl[(long long)r * ld] * keep, x1 = Xl[(long long)(r + 1) * ld] * keep;
-            b[r] -= __ldg(dd + r) * x0;
-            b[r + 1] -= __ldg(dd + r + 1) * x1;
-            xq[r / 2] = pack_bf16(x0, x1);
+            for (int j = 0; j < 16; ++j) x[(long long)j * ld] = a[j];
+          }
+        } else if (d.valid) {
+          const float* bs = d.J->B + d.at + (long long)r0 * ld;
+          const float* xs = d.J->X + d.at + (long long)r0 * ld;
+          const float* dd = d.J->ddiag + (long long)d.leaf * L + r0;
+          float* o = d.J->OUT ? d.J->OUT + d.at + (long long)r0 * ld : nullptr;
+          float bv[16], xv[16];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            bv[j] = bs[(long long)j * ld];
+            xv[j] = xs[(long long)j * ld];
+          }
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const float b = bv[j] - __ldg(dd + j) * xv[j];
+            const float r = b - a[j];
+            if (o) o[(long long)j * ld] = r;
+            const double av = fabs((double)r);
+            local_max = (av > local_max || av != av) ? av : local_max;
           }
         }
-        return;
       }
-      const float* Xl = X + (long long)leaf * L * ld;
-      const long long n0 = nbr[0] >= 0 ? nbr[0] : pa, n1 = nbr[1] >= 0 ? nbr[1] : pa;
-      const long long n2 = nbr[2] >= 0 ? nbr[2] : pa, n3 = nbr[3] >= 0 ? nbr[3] : pa;
-      const float w0 = nbr[0] >= 0 ? inv_h2 : 0.f, w1 = nbr[1] >= 0 ? inv_h2 : 0.f;
-      const float w2 = nbr[2] >= 0 ? inv_h2 : 0.f, w3 = nbr[3] >= 0 ? inv_h2 : 0.f;
-#pragma unroll
-      for (int r0 = 0; r0 < L; r0 += 8) {
-        float v[8], a0[8], a1[8], a2[8], a3[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const long long o = (long long)(r0 + j) * ld;
-          v[j] = Bl[o];
-          a0[j] = Xl[o + n0];
-          a1[j] = Xl[o + n1];
-          a2[j] = Xl[o + n2];
-          a3[j] = Xl[o + n3];
+      if (MODE == MODE_MATVEC && d.J->norm != nullptr && d.leaf == d.J->P.nb - 1) {  // the tile is done
+        for (int o = 16; o > 0; o >>= 1) {
+          const double other = __shfl_xor_sync(0xffffffffu, local_max, o);
+          local_max = (other > local_max || other != other) ? other : local_max;
         }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) b[r0 + j] = keep * (v[j] + w0 * a0[j] + w1 * a1[j] + w2 * a2[j] + w3 * a3[j]);
+        if (lane == 0) atomicMax(d.J->norm, (unsigned long long)__double_as_longlong(local_max));
+        local_max = 0.0;
       }
+      tc_before_sync();  // the reads of the buffer ordered before it is filled again
+      return true;
     };
-    load_leaf(0);
-    for (int i = 0; i < nb && !failed; ++i) {
-      unsigned char* xr_i = ring + (size_t)(i % W) * tile_bytes;
-      if (MODE == MODE_MATVEC) {
-        // x_i into the ring now (its slot's previous tile, x_{i-W}, was last read by leaf i-1's MMAs,
-        // complete since this thread waited on their barriers)
-#pragma unroll
-        for (int r = 0; r < L; r += 8) put8_packed(xr_i, c, r, L, &xq[r / 2]);
+    for (long long g = blockIdx.x; g < B.ntiles && !failed; g += gridDim.x) {
+      const WalkJob<float, uint16_t>& J = B.job[job_of(B, g)];
+      const long long ld = J.geo.ld;
+      const float inv_h2 = (float)J.geo.inv_h2;
+      const int nb = J.P.nb;
+      const bool grid = MODE == MODE_SMOOTH && J.geo.dim > 0;
+      bool valid;
+      long long p = 0;
+      // columns past the panel's end read column 0 (any valid address) and are zeroed, so that the loads
+      // carry no predicate; missing neighbours read the column itself with weight 0
+      long long n0 = 0, n1 = 0, n2 = 0, n3 = 0;
+      float w0 = 0.f, w1 = 0.f, w2 = 0.f, w3 = 0.f;
+      if (grid) {
+        const int N = J.geo.N;
+        int iy = 0, ix;
+        if (J.geo.dim == 2) {
+          const int first = (N + 1) / 2, nbx = (first + 31) / 32;
+          const long long tt = g - J.tile0;
+          iy = (int)(tt / nbx) * 4 + (c >> 5);
+          ix = ((iy + J.geo.colour) & 1) + 2 * ((int)(tt % nbx) * 32 + (c & 31));
+          valid = iy < N && ix < N;
+        } else {
+          const long long cg = (g - J.tile0) * NT + c;
+          ix = (int)(2 * cg) + J.geo.colour;
+          valid = cg < J.ncols;
+        }
+        if (valid) {
+          p = (long long)iy * N + ix;
+          if (ix > 0) w0 = inv_h2;
+          if (ix < N - 1) w1 = inv_h2;
+          if (J.geo.dim == 2 && iy > 0) w2 = inv_h2;
+          if (J.geo.dim == 2 && iy < N - 1) w3 = inv_h2;
+        }
+        n0 = w0 != 0.f ? p - 1 : p;
+        n1 = w1 != 0.f ? p + 1 : p;
+        n2 = w2 != 0.f ? p - N : p;
+        n3 = w3 != 0.f ? p + N : p;
+      } else {
+        const long long cg = (g - J.tile0) * NT + c;
+        valid = cg < J.ncols;
+        p = valid ? cg : 0;
       }
-      bool acc_used = false;
-      int nu = 0;  // UPART chunks of this leaf so far
-      for (bool leaf_done = false; !leaf_done && !failed;) {
-        if (give_up(mbar_wait_or_abort(full + cslot, cphase, abort_flag, B.spin))) {
+      const float keep = valid ? 1.f : 0.f;
+      for (int i = 0; i < nb; ++i, ++n) {
+        const int buf = (int)(n & 1);
+        if (n >= 2 && !write_leaf(n - 2)) {
           failed = true;
           break;
         }
-        const int4 cd = sdesc[cslot];
-        leaf_done = ((cd.x >> 12) & 1) != 0;
-        const int type = cd.x & 15, cnt = (cd.x >> 4) & 0xff;
-        unsigned char* buf = slots + (size_t)cslot * B.slot_bytes;
-        const uint32_t b_addr = smem_u32(buf);
-        if (type == PK_DENSE) {
-          if (issuer) {
-            tc_after_sync();
-            umma_product(t_acc, smem_u32(ring + (size_t)(cd.y % W) * tile_bytes), b_addr, L, L, acc_used);
-            umma_commit(empty + cslot);
+        const long long at = (long long)i * L * ld;
+        if (grid) {
+          const float* Bl = J.B + at + p;
+          const float* Xl = J.X + at;
+#pragma unroll
+          for (int r0 = 0; r0 < L; r0 += 8) {
+            float v[8], a0[8], a1[8], a2[8], a3[8];
+            uint32_t q[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const long long o = (long long)(r0 + j) * ld;
+              v[j] = ld_nc(Bl + o);
+              a0[j] = ld_nc(Xl + o + n0);
+              a1[j] = ld_nc(Xl + o + n1);
+              a2[j] = ld_nc(Xl + o + n2);
+              a3[j] = ld_nc(Xl + o + n3);
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              q[j] = __float_as_uint(keep * (v[j] + w0 * a0[j] + w1 * a1[j] + w2 * a2[j] + w3 * a3[j]));
+            tmem_st8(t_buf + 64 * buf + r0, q);
           }
-          acc_used = true;
-        } else if (type == PK_UPART) {
-          const int kp = cnt;  // padded to 16; padding columns of U are zero
-          if (nu > 0) {  // the previous U product of this leaf has read the staging tile
-            if (issuer) umma_commit(accbar);
-            if (!wait_mma(accbar, accph)) {
-              failed = true;
-              break;
+        } else if (MODE == MODE_SMOOTH) {
+          const float* Bl = J.B + at + p;
+#pragma unroll
+          for (int r0 = 0; r0 < L; r0 += 32) {
+            float v[32];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = ld_nc(Bl + (long long)(r0 + j) * ld);
+#pragma unroll
+            for (int j = 0; j < 32; j += 8) {
+              uint32_t q[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) q[e] = __float_as_uint(v[j + e] * keep);
+              tmem_st8(t_buf + 64 * buf + r0 + j, q);
             }
           }
-          const int* uz = reinterpret_cast<const int*>(buf + (size_t)L * kp * 2);
-          for (int k0 = 0; k0 < kp; k0 += 8) {
-            float zv[8];
+        } else {
+          const float* Xl = J.X + at + p;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) zv[e] = zpool[uz[k0 + e] * NT + c];
-            put8(zstage, c, k0, kp, zv);
+          for (int r0 = 0; r0 < L; r0 += 32) {
+            float v[32];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = Xl[(long long)(r0 + j) * ld];
+#pragma unroll
+            for (int j = 0; j < 32; j += 16) {
+              uint32_t q[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) q[e] = pack_bf16(v[j + 2 * e] * keep, v[j + 2 * e + 1] * keep);
+              tmem_st8(t_buf + 64 * buf + (r0 + j) / 2, q);
+            }
           }
-          if (!consumer_sync()) {
+        }
+        const Dest d{&J, at + p, i, valid};
+        if (buf)
+          d1 = d;
+        else
+          d0 = d;
+        tmem_st_wait();
+        tc_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(filled + buf);
+      }
+    }
+    if (!failed) failed = (n >= 2 && !write_leaf(n - 2)) || (n >= 1 && !write_leaf(n - 1));
+  } else {
+    // ---- walk warps ----
+    const int c = t;
+    const bool leader = umma_elect() && w == 0;  // issues the MMAs
+    uint32_t cbphase = 0, accph = 0, resph = 0, vph = 0;
+    int cslot = 0;
+    uint32_t cphase = 0;
+    bool failed = false;
+    long long n = 0;  // leaves walked so far
+    // all walk warps meet (bounded); tensor-memory reads and shared writes before it are ordered
+    // before the MMAs issued after it
+    auto walk_sync = [&]() -> bool {
+      async_proxy_fence();
+      tc_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(cbar);
+      const bool ok = mbar_wait_or_abort(cbar, cbphase, abort_flag, B.spin);
+      cbphase ^= 1;
+      tc_after_sync();
+      return !give_up(ok);
+    };
+    auto wait_on = [&](uint64_t* bar, uint32_t& ph) -> bool {
+      const bool ok = mbar_wait_or_abort(bar, ph, abort_flag, B.spin);
+      ph ^= 1;
+      tc_after_sync();
+      return !give_up(ok);
+    };
+    for (long long g = blockIdx.x; g < B.ntiles && !failed; g += gridDim.x) {
+      const WalkJob<float, uint16_t>& J = B.job[job_of(B, g)];
+      const float* ddg = J.ddiag;
+      const int nb = J.P.nb;
+      for (int i = 0; i < nb && !failed; ++i, ++n) {
+        unsigned char* xr_i = ring + (size_t)(i % W) * tile_bytes;
+        const int buf = (int)(n & 1);
+        const uint32_t bphase = (uint32_t)((n >> 1) & 1);
+        const uint32_t t_b = t_buf + 64 * buf;
+        if (MODE == MODE_MATVEC) {
+          // x_i into the ring (its slot's previous tile, x_{i-W}, was last read by leaf i-1's MMAs,
+          // complete since every walk thread waited on their barriers)
+          if (give_up(mbar_wait_or_abort(filled + buf, bphase, abort_flag, B.spin))) {
             failed = true;
             break;
           }
-          if (issuer) {
-            umma_product(t_acc, smem_u32(zstage), b_addr, kp, L, acc_used);
-            umma_commit(empty + cslot);
+          tc_after_sync();
+#pragma unroll
+          for (int r0 = 0; r0 < L / 2; r0 += 16) {
+            float v[16];
+            tmem_ld16(t_b + r0, v);
+            uint32_t q[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) q[j] = __float_as_uint(v[j]);
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) put8_packed(xr_i, c, 2 * (r0 + j), L, &q[j]);
           }
-          acc_used = true;
-          ++nu;
-        } else if (type == PK_DIAG) {
-          if (MODE == MODE_SMOOTH) {
-            if (acc_used) {
-              if (issuer) umma_commit(accbar);
-              if (!wait_mma(accbar, accph)) {
+        }
+        bool acc_used = false;
+        int nu = 0;  // UPART chunks of this leaf so far
+        for (bool leaf_done = false; !leaf_done && !failed;) {
+          if (give_up(mbar_wait_or_abort(full + cslot, cphase, abort_flag, B.spin))) {
+            failed = true;
+            break;
+          }
+          const int4 cd = sdesc[cslot];
+          leaf_done = ((cd.x >> 12) & 1) != 0;
+          const int type = cd.x & 15, cnt = (cd.x >> 4) & 0xff;
+          unsigned char* buf_c = slots + (size_t)cslot * B.slot_bytes;
+          const uint32_t b_addr = smem_u32(buf_c);
+          if (type == PK_DENSE) {
+            if (leader) {
+              tc_after_sync();
+              umma_product(t_acc, smem_u32(ring + (size_t)(cd.y % W) * tile_bytes), b_addr, L, L, acc_used);
+              umma_commit(empty + cslot);
+            }
+            acc_used = true;
+          } else if (type == PK_UPART) {
+            const int kp = cnt;  // padded to 16; padding columns of U are zero
+            if (nu > 0) {  // the previous U product of this leaf has read the staging tile
+              if (leader) umma_commit(accbar);
+              if (!wait_on(accbar, accph)) {
+                failed = true;
+                break;
+              }
+            }
+            const int* uz = reinterpret_cast<const int*>(buf_c + (size_t)L * kp * 2);
+            for (int k0 = 0; k0 < kp; k0 += 8) {
+              float zv[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) zv[e] = zpool[uz[k0 + e] * NT + c];
+              put8(zstage, c, k0, kp, zv);
+            }
+            if (!walk_sync()) {
+              failed = true;
+              break;
+            }
+            if (leader) {
+              umma_product(t_acc, smem_u32(zstage), b_addr, kp, L, acc_used);
+              umma_commit(empty + cslot);
+            }
+            acc_used = true;
+            ++nu;
+          } else if (type == PK_DIAG) {
+            if (MODE == MODE_SMOOTH) {
+              if (acc_used) {
+                if (leader) umma_commit(accbar);
+                if (!wait_on(accbar, accph)) {
+                  failed = true;
+                  break;
+                }
+              }
+              if (give_up(mbar_wait_or_abort(filled + buf, bphase, abort_flag, B.spin))) {
+                failed = true;
+                break;
+              }
+              tc_after_sync();
+              // y = b - acc, kept in the leaf buffer and staged as the A operand of the inverse's product
+#pragma unroll
+              for (int r0 = 0; r0 < L; r0 += 16) {
+                float y[16];
+                tmem_ld16(t_b + r0, y);
+                if (acc_used) {
+                  float a[16];
+                  tmem_ld16(t_acc + lane_base + r0, a);
+#pragma unroll
+                  for (int j = 0; j < 16; ++j) y[j] -= a[j];
+                  tmem_st16(t_b + r0, y);
+                }
+                put8(ystage, c, r0, L, &y[0]);
+                put8(ystage, c, r0 + 8, L, &y[8]);
+              }
+              tmem_st_wait();
+              if (!walk_sync()) {
+                failed = true;
+                break;
+              }
+              if (leader) {
+                umma_product(t_acc, smem_u32(ystage), b_addr, L, L, false);
+                umma_commit(empty + cslot);
+                umma_commit(resbar);
+              }
+              if (!wait_on(resbar, resph)) {
+                failed = true;
+                break;
+              }
+              // x = res + dinv_rr y into the ring and, for the memory warps, the leaf buffer
+              const float* dd = ddg + (long long)i * L;
+#pragma unroll
+              for (int r0 = 0; r0 < L; r0 += 16) {
+                float a[16], y[16];
+                tmem_ld16(t_acc + lane_base + r0, a);
+                tmem_ld16(t_b + r0, y);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) y[j] = a[j] + __ldg(dd + r0 + j) * y[j];
+                put8(xr_i, c, r0, L, &y[0]);
+                put8(xr_i, c, r0 + 8, L, &y[8]);
+                tmem_st16(t_b + r0, y);
+              }
+              tmem_st_wait();
+              if (!walk_sync()) {  // x_i complete in the ring before the V products read it
+                failed = true;
+                break;
+              }
+              if (lane == 0) mbar_arrive(walked + buf);
+            } else {
+              if (!walk_sync()) {  // x_i staged by every thread
+                failed = true;
+                break;
+              }
+              if (leader) {
+                umma_product(t_acc, smem_u32(xr_i), b_addr, L, L, acc_used);
+                umma_commit(empty + cslot);
+                umma_commit(accbar);
+              }
+              if (!wait_on(accbar, accph)) {
                 failed = true;
                 break;
               }
@@ -422,132 +658,58 @@ __global__ void __maxnreg__(168) humma_kernel(const __grid_constant__ WalkBatch<
               for (int r0 = 0; r0 < L; r0 += 16) {
                 float a[16];
                 tmem_ld16(t_acc + lane_base + r0, a);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) b[r0 + j] -= a[j];
+                tmem_st16(t_b + r0, a);
               }
+              tmem_st_wait();
+              if (!walk_sync()) {  // every thread has read acc before the next leaf's MMAs
+                failed = true;
+                break;
+              }
+              if (lane == 0) mbar_arrive(walked + buf);
             }
-            // b now holds y; stage it as the A operand of the inverse's product
-#pragma unroll
-            for (int r = 0; r < L; r += 8) put8(ystage, c, r, L, &b[r]);
-            if (!consumer_sync()) {
-              failed = true;
-              break;
-            }
-            if (issuer) {
-              umma_product(t_res, smem_u32(ystage), b_addr, L, L, false);
+          } else {  // PK_VPART: z entries from x_i
+            const int np = (cnt + 15) / 16 * 16;
+            if (leader) {
+              umma_product(t_v, smem_u32(xr_i), b_addr, L, np, false);
               umma_commit(empty + cslot);
-              umma_commit(resbar);
+              umma_commit(vbar);
             }
-            if (!wait_mma(resbar, resph)) {
+            if (!wait_on(vbar, vph)) {
               failed = true;
               break;
             }
-            const float* dd = ddg + (long long)i * L;
-#pragma unroll
-            for (int r0 = 0; r0 < L; r0 += 16) {
+            const int* codes = reinterpret_cast<const int*>(buf_c + (size_t)np * L * 2);
+            for (int q0 = 0; q0 < cnt; q0 += 16) {
               float a[16];
-              tmem_ld16(t_res + lane_base + r0, a);
-#pragma unroll
-              for (int j = 0; j < 16; ++j) b[r0 + j] = a[j] + __ldg(dd + r0 + j) * b[r0 + j];  // b := x_i
-              put8(xr_i, c, r0, L, &b[r0]);
-              put8(xr_i, c, r0 + 8, L, &b[r0 + 8]);
-            }
-            async_proxy_fence();  // x_i in the ring, ordered before the V products ...
-            tc_before_sync();     // ... and the reads of res before later MMAs
-            // global stores and loads only after the fence, which would otherwise wait for them
-            if (valid) {
-#pragma unroll
-              for (int r = 0; r < L; ++r) X[(long long)(i * L + r) * ld + p] = b[r];
-            }
-            load_leaf(i + 1);
-            if (!arrive_wait()) {  // x_i complete in the ring before the V products read it
-              failed = true;
-              break;
-            }
-          } else {
-            if (!consumer_sync()) {  // x_i staged by every thread
-              failed = true;
-              break;
-            }
-            if (issuer) {
-              umma_product(t_acc, smem_u32(xr_i), b_addr, L, L, acc_used);
-              umma_commit(empty + cslot);
-              umma_commit(accbar);
-            }
-            if (!wait_mma(accbar, accph)) {
-              failed = true;
-              break;
-            }
-#pragma unroll
-            for (int r0 = 0; r0 < L; r0 += 16) {
-              float a[16];
-              tmem_ld16(t_acc + lane_base + r0, a);
+              tmem_ld16(t_v + lane_base + q0, a);
 #pragma unroll
               for (int j = 0; j < 16; ++j) {
-                const float o = b[r0 + j] - a[j];
-                if (valid) {
-                  if (J.OUT) J.OUT[(long long)(i * L + r0 + j) * ld + p] = o;
-                  const double av = fabs((double)o);
-                  local_max = (av > local_max || av != av) ? av : local_max;
+                if (q0 + j < cnt) {
+                  const int code = codes[q0 + j];
+                  float* z = zpool + (code >> 1) * NT + c;
+                  *z = (code & 1) ? a[j] : *z + a[j];
                 }
               }
             }
-            tc_before_sync();  // the reads of acc ordered before the next leaf's MMAs
-            load_leaf(i + 1);
-            if (!arrive_wait()) {  // every thread has read acc before the next leaf's MMAs
+            if (!leaf_done && !walk_sync()) {  // v is read before the next V product overwrites it
               failed = true;
               break;
             }
           }
-        } else {  // PK_VPART: z entries from x_i
-          const int np = (cnt + 15) / 16 * 16;
-          if (issuer) {
-            umma_product(t_v, smem_u32(xr_i), b_addr, L, np, false);
-            umma_commit(empty + cslot);
-            umma_commit(vbar);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(empty + cslot);  // this warp is done with the slot
+          if (++cslot == ns) {
+            cslot = 0;
+            cphase ^= 1;
           }
-          if (!wait_mma(vbar, vph)) {
-            failed = true;
-            break;
-          }
-          const int* codes = reinterpret_cast<const int*>(buf + (size_t)np * L * 2);
-          for (int q0 = 0; q0 < cnt; q0 += 16) {
-            float a[16];
-            tmem_ld16(t_v + lane_base + q0, a);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              if (q0 + j < cnt) {
-                const int code = codes[q0 + j];
-                float* z = zpool + (code >> 1) * NT + c;
-                *z = (code & 1) ? a[j] : *z + a[j];
-              }
-            }
-          }
-          if (!leaf_done && !consumer_sync()) {  // v is read before the next V product overwrites it
-            failed = true;
-            break;
-          }
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(empty + cslot);  // this warp is done with the slot
-        if (++cslot == ns) {
-          cslot = 0;
-          cphase ^= 1;
         }
       }
     }
-    if (MODE == MODE_MATVEC && J.norm != nullptr && !failed) {
-      for (int o = 16; o > 0; o >>= 1) {
-        const double other = __shfl_xor_sync(0xffffffffu, local_max, o);
-        local_max = (other > local_max || other != other) ? other : local_max;
-      }
-      if (lane == 0) atomicMax(J.norm, (unsigned long long)__double_as_longlong(local_max));
-    }
+    if (leader) umma_commit(donebar);
   }
-  // exit (normal or after a wait gave up): the MMAs issued so far complete, every consumer warp is
-  // done with tensor memory (a barrier used once, so its phase is 0 whatever happened before), then
-  // the allocating warp frees it.  Every consumer wait is bounded, so every warp arrives.
-  if (issuer) umma_commit(donebar);
+  // exit (normal or after a wait gave up): the MMAs issued so far complete, every walk and memory warp
+  // is done with tensor memory (a barrier used once, so its phase is 0 whatever happened before), then
+  // the allocating warp frees it.  Every wait is bounded, so every warp arrives.
   tc_before_sync();
   __syncwarp();
   if (lane == 0) mbar_arrive(exitbar);

@@ -92,7 +92,7 @@ int walk_launch_umma(cudaStream_t st, const WalkArgsT<float>* jobs, int njobs, s
     J.dinv_cstride = 0;
     J.ddiag = a.ddiag;
     J.norm = a.norm;
-    tiles += (a.ncols + kUmmaCols - 1) / kUmmaCols;
+    tiles += mode == MODE_SMOOTH ? umma_tiles(a.geo, a.ncols) : (a.ncols + kUmmaCols - 1) / kUmmaCols;
   }
   B.ntiles = tiles;
   B.ns = 2;
