@@ -18,6 +18,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstring>
@@ -26,6 +27,7 @@
 #include <vector>
 
 #include "devinfo.h"
+#include "umma.cuh"
 #include "fhmg.h"
 
 // Kernel launches issued by this file (network training / inference, warm-start projection and
@@ -46,6 +48,14 @@ constexpr int kFeat = 6;
 
 __device__ __forceinline__ float sigm(float x) { return 1.f / (1.f + __expf(-x)); }
 
+// the FP64 value of a float by integer operations (the conversion runs on the 1/64-rate FP64 pipe);
+// subnormals and non-finite values by the conversion
+__device__ __forceinline__ double f2d_exact(float f) {
+  const uint32_t b = __float_as_uint(f), m = b & 0x7FFFFFFFu;
+  if (m - 0x00800000u >= 0x7F000000u) return m == 0 ? __hiloint2double((int)b, 0) : (double)f;
+  return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + (896u << 20))), (int)(b << 29));
+}
+
 // FP32 GEMM arguments: op(A) (M x K) op(B) (K x N); A stored K x M when transposed, B stored N x K when
 // transposed.  Batches and splits run along blockIdx.z.
 struct GemmArgs {
@@ -60,9 +70,11 @@ struct GemmArgs {
   const float* bias;     // EPI_ACT: bias per column; EPI_ACTB: Z (ldc) of the layer below
   float* out2;           // EPI_ACT: the activations (ldc); EPI_SPLIT: column sums of op(A)^T per split
   int act;               // EPI_ACT: SiLU or none
+  double* out64;         // EPI_F64
 };
 // what is written: alpha C | z = C + bias and its activation | C * SiLU'(Z) | partial sums of a split
-enum { EPI_PLAIN = 0, EPI_ACT = 1, EPI_ACTB = 2, EPI_SPLIT = 3 };
+// | C widened to FP64 (out64, batch stride sC; thread columns 16 apart, so that a row's stores are contiguous)
+enum { EPI_PLAIN = 0, EPI_ACT = 1, EPI_ACTB = 2, EPI_SPLIT = 3, EPI_F64 = 4 };
 
 constexpr int kGB = 64, kGK = 16, kGThreads = 128, kGLd = kGB + 4;
 
@@ -150,7 +162,11 @@ __global__ void __launch_bounds__(kGThreads) gemm_f32(const GemmArgs g) {
     for (int kk = 0; kk < kGK; ++kk) {
       const float4 a0 = *reinterpret_cast<const float4*>(&As[b][kk][ty * 8]);
       const float4 a1 = *reinterpret_cast<const float4*>(&As[b][kk][ty * 8 + 4]);
-      const float4 bb = *reinterpret_cast<const float4*>(&Bs[b][kk][tx * 4]);
+      float4 bb;
+      if (EPI == EPI_F64)
+        bb = make_float4(Bs[b][kk][tx], Bs[b][kk][tx + 16], Bs[b][kk][tx + 32], Bs[b][kk][tx + 48]);
+      else
+        bb = *reinterpret_cast<const float4*>(&Bs[b][kk][tx * 4]);
       const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w}, bv[4] = {bb.x, bb.y, bb.z, bb.w};
 #pragma unroll
       for (int i = 0; i < 8; ++i)
@@ -163,6 +179,18 @@ __global__ void __launch_bounds__(kGThreads) gemm_f32(const GemmArgs g) {
     }
     if (next) stage(b ^ 1);
     __syncthreads();
+  }
+  if (EPI == EPI_F64) {
+    double* D = g.out64 + blockIdx.z * g.sC;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int gm = m0 + ty * 8 + i;
+      if (gm >= g.M) break;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (n0 + tx + 16 * j < g.N) D[(long long)gm * g.ldc + n0 + tx + 16 * j] = f2d_exact(acc[i][j]);
+    }
+    return;
   }
   const bool v4 = (g.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0 &&
                   (EPI != EPI_ACT || (reinterpret_cast<uintptr_t>(g.out2) & 15) == 0);
@@ -400,6 +428,301 @@ __global__ void __launch_bounds__(256) gemm_bf16_silu(int M, int N, int K, const
     }
 }
 
+// 1 / d, correctly rounded, for 1 <= d < 2^126 (or NaN): one Newton step (with FMA, after Markstein) from the
+// approximate reciprocal; compared with the division for every mantissa and exponent of the range.
+// The division's range checks put a branch behind every activation: the epilogues of mlp_bf16 took
+// 27 000 cycles per layer and 128 rows with it.
+__device__ __forceinline__ float rcp_1_up(float d) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(d));
+  return __fmaf_rn(y, __fmaf_rn(-d, y, 1.f), y);
+}
+
+// The whole BF16 network on 128 rows at a time, on the tcgen05 tensor cores: input layer, hidden layers
+// of width H and output layer, activations (BF16, SiLU) kept in shared memory between them.  Every
+// layer is a batch of MMAs (M = 128 rows, N = the layer's width, FP32 accumulators in tensor memory) by
+// one warp, then an epilogue by eight warps (bias, SiLU, rounding, the next layer's A operand in the
+// 128-byte swizzle).  The hidden weights pass through a two-stage ring of K tiles of 64 (bulk copies of
+// the operand layout, prepared by pack_weights); the input layer's (K = 6, padded to 16), the output
+// layer's (one row, padded to 16) and the biases stay in shared memory.  The sums run over k16 steps in
+// order and round as mma.sync m16n8k16 does, so the results are those of the one-launch-per-layer path
+// bit for bit.  Bound by the epilogues (two special-function operations per activation).  294912 rows of
+// width 320: 1.25 ms over six launches; fused with mma.sync 0.74 ms; 0.34 ms now.
+struct MlpArgs {
+  int n, layers;                    // rows, hidden layers
+  const float* X;                   // n x kFeat
+  const unsigned char* W;           // pack_weights
+  const float* P;                   // parameters in FP32 (biases)
+  long long boff[9];
+  float* Y;
+  int* err;                         // set if a bounded wait gives up
+};
+
+constexpr int kMlpRows = 128, kMlpMaxH = 320, kMlpEpi = 256, kMlpBlock = kMlpEpi + 64;
+// bytes of the packed weights: input layer (H x 16), output layer (16 x H), then per hidden layer H / 64
+// tiles of H x 64
+__host__ __device__ inline size_t mlp_packed(int H, int layers) {
+  return (size_t)H * 16 * 2 * 2 + (size_t)(layers - 1) * H * H * 2;
+}
+struct MlpSmem {
+  size_t act, ring, win, wout, xin, bias, bar, total;
+};
+__host__ __device__ inline MlpSmem mlp_smem(int H, int layers) {
+  MlpSmem s;
+  s.act = 0;
+  s.ring = (size_t)kMlpRows * H * 2;
+  s.win = s.ring + 2 * (size_t)H * 128;
+  s.wout = s.win + (size_t)H * 32;
+  s.xin = s.wout + (size_t)H * 32;
+  s.bias = s.xin + (size_t)kMlpRows * 32;
+  s.bar = s.bias + (size_t)(layers * H + 4) * 4;
+  s.total = s.bar + 8 * 7 + 16;
+  return s;
+}
+
+// BF16 copies of the weights as MMA operands (W_0: no swizzle, K = 16; W_out and the hidden layers: 64-column
+// tiles, 128-byte swizzle), padding zero
+__global__ void pack_weights(int H, int layers, const float* __restrict__ P, unsigned char* __restrict__ out) {
+  const long long hid = (long long)(layers - 1) * H * H, total = 32LL * H + hid;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+    float v = 0.f;
+    size_t o;
+    if (i < 16LL * H) {
+      const int r = (int)(i / 16), k = (int)(i % 16);
+      if (k < kFeat) v = P[r * kFeat + k];
+      o = fhmg::umma_off(r, k, 16);
+    } else if (i < 32LL * H) {
+      const int r = (int)((i - 16LL * H) / H), k = (int)((i - 16LL * H) % H);
+      if (r == 0) v = P[(long long)(kFeat + 1) * H + (long long)(layers - 1) * (H + 1) * H + k];
+      o = (size_t)H * 32 + (size_t)(k / 64) * 16 * 128 + fhmg::sw128_off(r, k % 64);
+    } else {
+      const long long j = i - 32LL * H;
+      const int l = (int)(j / ((long long)H * H)), r = (int)(j % ((long long)H * H) / H), k = (int)(j % H);
+      v = P[(long long)(kFeat + 1) * H + (long long)l * (H + 1) * H + (long long)r * H + k];
+      o = (size_t)H * 64 + (size_t)l * H * H * 2 + (size_t)(k / 64) * H * 128 + fhmg::sw128_off(r, k % 64);
+    }
+    *reinterpret_cast<__nv_bfloat16*>(out + o) = __float2bfloat16(v);
+  }
+}
+
+__global__ void __launch_bounds__(kMlpBlock, 1) mlp_bf16(int H, const __grid_constant__ MlpArgs g) {
+  using namespace fhmg;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  unsigned char* sm = smraw + ((1024u - (smem_u32(smraw) & 1023u)) & 1023u);  // swizzled tiles: 1024-byte aligned
+  const MlpSmem lay = mlp_smem(H, g.layers);
+  unsigned char* act = sm + lay.act;
+  float* bias = reinterpret_cast<float*>(sm + lay.bias);
+  uint64_t* wfull = reinterpret_cast<uint64_t*>(sm + lay.bar);  // [2]
+  uint64_t* wfree = wfull + 2;                                   // [2]
+  uint64_t* aready = wfull + 4;                                  // the A operand of the next batch is complete
+  uint64_t* accdone = wfull + 5;                                 // a batch's MMAs are complete
+  uint64_t* donebar = wfull + 6;                                 // every MMA issued is complete
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(wfull + 7);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(wfull + 7) + 1;
+  const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+  const int KT = H / 64, nhid = g.layers - 1;
+  const uint32_t tcols = H + 16 <= 128 ? 128 : H + 16 <= 256 ? 256 : 512;
+  if (t == 0) {
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(wfull + s, 1);
+      mbar_init(wfree + s, 1);
+    }
+    mbar_init(aready, kMlpEpi / 32);
+    mbar_init(accdone, 1);
+    mbar_init(donebar, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  // the resident operands: packed input and output layers, biases, the zero half of the input rows
+  for (int i = t; i < H * 64 / 16; i += kMlpBlock)
+    reinterpret_cast<uint4*>(sm + lay.win)[i] = __ldg(reinterpret_cast<const uint4*>(g.W) + i);
+  for (int i = t; i <= g.layers * H; i += kMlpBlock) bias[i] = __ldg(g.P + g.boff[i / H] + i % H);
+  if (t < kMlpRows) *reinterpret_cast<uint4*>(sm + lay.xin + umma_off(t, 8, 16)) = make_uint4(0, 0, 0, 0);
+  if (w == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)), "r"(tcols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  async_proxy_fence();
+  tc_before_sync();
+  __syncthreads();
+  tc_after_sync();
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
+  const int blocks = (g.n + kMlpRows - 1) / kMlpRows;
+  auto raise = [&]() {
+    *abort_flag = 1;
+    atomicExch(g.err, 1);
+  };
+  if (w == kMlpEpi / 32) {
+    // ---- producer: the hidden layers' K tiles, for every row block ----
+    if (lane == 0) {
+      const uint32_t bytes = (uint32_t)H * 128;
+      int slot = 0;
+      uint32_t phase = 1;
+      long long k = 0;
+      bool ok = true;
+      for (int blk = blockIdx.x; blk < blocks && ok; blk += gridDim.x)
+        for (int j = 0; j < nhid * KT; ++j, ++k) {
+          if (!mbar_wait_or_abort(wfree + slot, phase, abort_flag)) {
+            ok = false;
+            break;
+          }
+          bulk_load(sm + lay.ring + (size_t)slot * bytes, g.W + (size_t)H * 64 + (size_t)j * bytes, bytes, wfull + slot);
+          slot ^= 1;
+          phase ^= slot ^ 1;
+        }
+      if (!ok) raise();
+      for (int s = 0; s < 2 && s < k; ++s) mbar_wait(wfull + s, (uint32_t)(((k - 1 - s) / 2) & 1));
+    }
+    __syncwarp();
+  } else if (w == kMlpEpi / 32 + 1) {
+    // ---- MMA warp (uniform; one elected lane issues) ----
+    const bool leader = umma_elect();
+    const int N0 = H < 256 ? H : 256, N1 = H - N0;
+    int slot = 0;
+    uint32_t fphase = 0, aphase = 0;
+    bool ok = true;
+    auto wait = [&](uint64_t* bar, uint32_t ph) -> bool {
+      ok = __all_sync(0xffffffffu, mbar_wait_or_abort(bar, ph, abort_flag));
+      tc_after_sync();
+      return ok;
+    };
+    auto mma = [&](uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, bool accumulate) {
+      asm volatile(
+          "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+          " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+          "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate ? 1u : 0u)
+          : "memory");
+    };
+    for (int blk = blockIdx.x; blk < blocks && ok; blk += gridDim.x) {
+      for (int l = 0; l <= g.layers; ++l) {
+        if (!wait(aready, aphase)) break;
+        aphase ^= 1;
+        if (l == 0) {
+          if (leader) {
+            umma_product(tmem, smem_u32(sm + lay.xin), smem_u32(sm + lay.win), 16, N0, false);
+            if (N1) umma_product(tmem + 256, smem_u32(sm + lay.xin), smem_u32(sm + lay.win) + 256 * 32, 16, N1, false);
+          }
+        } else if (l <= nhid) {
+          for (int kt = 0; kt < KT; ++kt) {
+            if (!wait(wfull + slot, fphase)) break;
+            const uint64_t ad = sw128_desc(smem_u32(act) + (uint32_t)kt * kMlpRows * 128);
+            const uint64_t bd = sw128_desc(smem_u32(sm + lay.ring) + (uint32_t)slot * H * 128);
+            if (leader) {
+#pragma unroll
+              for (int st = 0; st < 4; ++st) mma(tmem, ad + 2 * st, bd + 2 * st, umma_idesc(N0), kt + st > 0);
+              if (N1) {
+#pragma unroll
+                for (int st = 0; st < 4; ++st)
+                  mma(tmem + 256, ad + 2 * st, bd + (256 * 128 >> 4) + 2 * st, umma_idesc(N1), kt + st > 0);
+              }
+              umma_commit(wfree + slot);
+            }
+            slot ^= 1;
+            fphase ^= slot ^ 1;
+          }
+          if (!ok) break;
+        } else {
+          if (leader)
+            for (int kt = 0; kt < KT; ++kt) {
+              const uint64_t ad = sw128_desc(smem_u32(act) + (uint32_t)kt * kMlpRows * 128);
+              const uint64_t bd = sw128_desc(smem_u32(sm + lay.wout) + (uint32_t)kt * 16 * 128);
+#pragma unroll
+              for (int st = 0; st < 4; ++st) mma(tmem + H, ad + 2 * st, bd + 2 * st, umma_idesc(16), kt + st > 0);
+            }
+        }
+        if (leader) umma_commit(accdone);
+      }
+    }
+    if (!ok && leader) raise();
+    if (leader) umma_commit(donebar);
+    mbar_wait(donebar, 0);
+  } else {
+    // ---- epilogue warps: lane quarter w % 4 (rows), column half w / 4 ----
+    const uint32_t lane_base = (uint32_t)(32 * (w & 3)) << 16;
+    const int row = 32 * (w & 3) + lane, c0 = (w >> 2) * (H / 2);
+    uint32_t dphase = 0;
+    bool failed = false;
+    auto ready = [&]() {
+      async_proxy_fence();
+      tc_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(aready);
+    };
+    auto put_x = [&](int blk) {  // the block's input rows (BF16) by the first column half
+      if (w < 4) {
+        const long long r = (long long)blk * kMlpRows + row;
+        float2 a = make_float2(0.f, 0.f), b = a, c = a;
+        if (r < g.n) {
+          const float2* x = reinterpret_cast<const float2*>(g.X + r * kFeat);
+          a = __ldg(x), b = __ldg(x + 1), c = __ldg(x + 2);
+        }
+        *reinterpret_cast<uint4*>(sm + lay.xin + umma_off(row, 0, 16)) =
+            make_uint4(pack_bf16(a.x, a.y), pack_bf16(b.x, b.y), pack_bf16(c.x, c.y), 0u);
+      }
+      ready();
+    };
+    if ((int)blockIdx.x < blocks) put_x(blockIdx.x);
+    for (int blk = blockIdx.x; blk < blocks && !failed; blk += gridDim.x) {
+      for (int l = 0; l <= g.layers; ++l) {
+        if (!__all_sync(0xffffffffu, mbar_wait_or_abort(accdone, dphase, abort_flag))) {
+          if (lane == 0) raise();
+          failed = true;
+          break;
+        }
+        dphase ^= 1;
+        tc_after_sync();
+        if (l == g.layers) {  // the output
+          float v[16];
+          tmem_ld16(tmem + lane_base + H, v);
+          const long long r = (long long)blk * kMlpRows + row;
+          if (w < 4 && r < g.n) g.Y[r] = v[0] + bias[g.layers * H];
+          if (blk + (int)gridDim.x < blocks) put_x(blk + gridDim.x);
+          continue;
+        }
+        for (int c = c0; c < c0 + H / 2; c += 16) {
+          float v[16];
+          tmem_ld16(tmem + lane_base + c, v);
+          const float4* bp = reinterpret_cast<const float4*>(bias + l * H + c);
+#pragma unroll
+          for (int j = 0; j < 16; j += 4) {
+            const float4 b = bp[j / 4];
+            v[j] += b.x, v[j + 1] += b.y, v[j + 2] += b.z, v[j + 3] += b.w;
+          }
+          // SiLU with the correctly rounded reciprocal of sigm(), without a division's branches
+          float d[16], dmax = 0.f;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            d[j] = 1.f + __expf(-v[j]);
+            dmax = fmaxf(dmax, d[j]);
+          }
+          if (__any_sync(0xffffffffu, dmax > 0x1p125f)) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) d[j] = 1.f / d[j];
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) d[j] = rcp_1_up(d[j]);
+          }
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] = v[j] * d[j];
+          unsigned char* dst = act + (size_t)(c / 64) * kMlpRows * 128;
+#pragma unroll
+          for (int j = 0; j < 16; j += 8)
+            *reinterpret_cast<uint4*>(dst + sw128_off(row, c % 64 + j)) =
+                make_uint4(pack_bf16(v[j], v[j + 1]), pack_bf16(v[j + 2], v[j + 3]), pack_bf16(v[j + 4], v[j + 5]),
+                           pack_bf16(v[j + 6], v[j + 7]));
+        }
+        ready();
+      }
+    }
+  }
+  // every wait above is bounded, so every warp gets here, with the MMAs complete
+  tc_before_sync();
+  __syncthreads();
+  tc_after_sync();
+  if (w == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols));
+}
+
 // Z += b (row broadcast); A = SiLU(Z) (act = 1) or Z (act = 0).  Z kept for the backward pass.
 __global__ void bias_act_fwd(int n, int w, float* Z, const float* b, float* A, int act, __nv_bfloat16* Abf) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)n * w;
@@ -446,22 +769,26 @@ int nblk(long long n) { return fhmg::grid_for(n, 16); }
 }  // namespace
 
 // Features of (lam, alpha, t), all O(1): log10(lam)/5, alpha, log10(t)/5 (t > 0), s/(1+s),
-// log1p(s)/10 with s = lam t^alpha, t^alpha.
-__device__ __forceinline__ void ws_features(double lam, double alpha, double t, float* f) {
-  const double ta = pow(t, alpha), s = lam * ta;
-  f[0] = (float)(log10(lam) / 5.0);
+// log1p(s)/10 with s = lam t^alpha, t^alpha.  What depends on the mode or the time level alone comes
+// from a table (the FP64 pipe runs at 1/64 of the FP32 rate): `loglam` per mode, `ta` = t^alpha and
+// `logt` per level.
+__device__ __forceinline__ void ws_features(double lam, float loglam, double alpha, double ta, float logt, float* f) {
+  const double s = lam * ta;
+  f[0] = loglam;
   f[1] = (float)alpha;
-  f[2] = (float)(log10(t) / 5.0);
+  f[2] = logt;
   f[3] = (float)(s / (1.0 + s));
   f[4] = (float)(log1p(s) / 10.0);
   f[5] = (float)ta;
 }
 
-__global__ void build_features(int nmodes, const double* lam, int M, const double* t, double alpha, float* X) {
-  const long long total = (long long)nmodes * M;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int k = (int)(i / M), m = (int)(i % M);
-    ws_features(lam[k], alpha, t[m + 1], X + i * kFeat);
+__global__ void feature_tables(int nm, const double* lam, int M, const double* t, double alpha, float* loglam, double* ta,
+                               float* logt) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < nm) loglam[i] = (float)(log10(lam[i]) / 5.0);
+  if (i < M) {
+    ta[i] = pow(t[i + 1], alpha);
+    logt[i] = (float)(log10(t[i + 1]) / 5.0);
   }
 }
 
@@ -475,6 +802,8 @@ struct fhmg_wsnet_s {
   float* Mo = nullptr;            // Adam moments
   float* Vo = nullptr;
   __nv_bfloat16* Pbf = nullptr;   // BF16 copy of the weights (inference)
+  unsigned char* Wpk = nullptr;   // the weights as MMA operands: widths 64, 128, .., kMlpMaxH (mlp_bf16)
+  int* err = nullptr;             // set by mlp_bf16 if a bounded wait gave up
   long long step = 0;
   // activations for a batch of up to cap rows
   int cap = 0;
@@ -536,6 +865,16 @@ int gemm(cudaStream_t st, int M, int N, int K, float alpha, const float* A, int 
   g.sA = sA, g.sB = sB, g.sC = sC;
   if (ta) return gemm_launch<true, false, EPI_PLAIN>(st, g, batch);
   return tb ? gemm_launch<false, true, EPI_PLAIN>(st, g, batch) : gemm_launch<false, false, EPI_PLAIN>(st, g, batch);
+}
+
+// out (M x N, ldc; FP64) = op(A) op(B), batched
+int gemm_to_f64(cudaStream_t st, int M, int N, int K, const float* A, int lda, const float* B, int ldb, int tb,
+                double* out, int ldc, int batch, long long sA, long long sB, long long sC) {
+  GemmArgs g{};
+  g.M = M, g.N = N, g.K = K;
+  g.A = A, g.B = B, g.lda = lda, g.ldb = ldb, g.ldc = ldc, g.out64 = out;
+  g.sA = sA, g.sB = sB, g.sC = sC;
+  return tb ? gemm_launch<false, true, EPI_F64>(st, g, batch) : gemm_launch<false, false, EPI_F64>(st, g, batch);
 }
 
 int ensure_part(fhmg_wsnet net, size_t n) {
@@ -652,9 +991,11 @@ int fhmg_wsnet_create(int hidden, int layers, unsigned long long seed, fhmg_wsne
   };
   if ((s = nalloc(net, &net->P, host.size())) || (s = nalloc(net, &net->G, host.size())) ||
       (s = nalloc(net, &net->Mo, host.size())) || (s = nalloc(net, &net->Vo, host.size())) ||
-      (s = nalloc(net, &net->Pbf, host.size())) || (s = nalloc(net, &net->loss, 1)))
+      (s = nalloc(net, &net->Pbf, host.size())) || (s = nalloc(net, &net->loss, 1)) || (s = nalloc(net, &net->err, 1)) ||
+      (hidden % 64 == 0 && hidden <= kMlpMaxH && (s = nalloc(net, &net->Wpk, mlp_packed(hidden, layers)))))
     return bail(s);
   if (cudaMemcpy(net->P, host.data(), host.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemset(net->err, 0, sizeof(int)) != cudaSuccess ||
       cudaMemset(net->Mo, 0, host.size() * 4) != cudaSuccess || cudaMemset(net->Vo, 0, host.size() * 4) != cudaSuccess)
     return bail(fhmg_internal_fail(FHMG_ECUDA, "wsnet upload failed"));
   *out = net;
@@ -690,8 +1031,25 @@ int fhmg_wsnet_forward(fhmg_wsnet net, const float* X, int n, int bf16, float* Y
   if (!net || !X || !Y || n < 1) return fhmg_internal_fail(FHMG_EINVAL, "bad arguments");
   cudaStream_t st = (cudaStream_t)stream;
   const int L = (int)net->width.size() - 1;
-  int s = ensure_cap(net, n);
-  if (s) return s;
+  int s;
+  if (bf16 && net->Wpk && reinterpret_cast<uintptr_t>(X) % 8 == 0) {
+    pack_weights<<<nblk(32LL * net->hidden + (long long)(net->layers - 1) * net->hidden * net->hidden), 256, 0, st>>>(
+        net->hidden, net->layers, net->P, net->Wpk);
+    ++g_nn_launches;
+    NCK(cudaGetLastError());
+    MlpArgs a{};
+    a.n = n, a.layers = net->layers, a.X = X, a.W = net->Wpk, a.P = net->P, a.Y = Y, a.err = net->err;
+    for (int l = 0; l < L; ++l) a.boff[l] = net->boff[l];
+    static fhmg::KernelCache cache;
+    const size_t smem = mlp_smem(net->hidden, net->layers).total + 1024;
+    int occ = 1;
+    NCK(fhmg::prepare_launch(mlp_bf16, kMlpBlock, smem, cache, &occ));
+    mlp_bf16<<<std::min((n + kMlpRows - 1) / kMlpRows, fhmg::device_sms()), kMlpBlock, smem, st>>>(net->hidden, a);
+    ++g_nn_launches;
+    NCK(cudaGetLastError());
+    return FHMG_OK;
+  }
+  if ((s = ensure_cap(net, n))) return s;
   if (!bf16) {
     if ((s = forward32(net, st, X, n))) return s;
     NCK(cudaMemcpyAsync(Y, net->A[L], sizeof(float) * n, cudaMemcpyDeviceToDevice, st));
@@ -767,11 +1125,6 @@ __global__ void d2f(long long n, const double* x, float* y) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     y[i] = (float)x[i];
 }
-__global__ void f2d(long long n, const float* x, double* y) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    y[i] = (double)x[i];
-}
-
 // eigenvalue of mode k (2D: k = p K + q) of the 3-/5-point negative Laplacian
 __device__ __forceinline__ double mode_lambda(int dim, int N, double Lx, int K, int k) {
   const double h = Lx / (N + 1);
@@ -808,14 +1161,14 @@ __global__ void mode_targets(int nm, int M, const float* c, const float* uhat, c
   }
 }
 
-__global__ void build_features_kept(int nm, const double* lam, int M, const double* t, double alpha, const int* keep,
-                                    const int* kpos, float* X) {
+__global__ void build_features_kept(int nm, const double* lam, const float* loglam, int M, const double* ta,
+                                    const float* logt, double alpha, const int* keep, const int* kpos, float* X) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)nm * M;
        i += (long long)gridDim.x * blockDim.x) {
     const int k = (int)(i / M), m = (int)(i % M);
     if (!keep || keep[k]) {
       const long long row = (long long)(keep ? kpos[k] : k) * M + m;
-      ws_features(lam[k], alpha, t[m + 1], X + row * kFeat);
+      ws_features(lam[k], loglam[k], alpha, ta[m], logt[m], X + row * kFeat);
     }
   }
 }
@@ -896,6 +1249,19 @@ struct Spectral {
     NCK(cudaMemcpyAsync(tdev, thost, sizeof(double) * (M + 1), cudaMemcpyHostToDevice, st));
     return FHMG_OK;
   }
+  // features of the kept modes (all: keep NULL) at every time level, row order k-major
+  int features(double alpha, const int* keep, const int* kpos, float* X) {
+    float *loglam, *logt;
+    double* ta;
+    int s;
+    if ((s = alloc(&loglam, nm)) || (s = alloc(&logt, M)) || (s = alloc(&ta, M))) return s;
+    feature_tables<<<(std::max(nm, M) + 127) / 128, 128, 0, st>>>(nm, lam, M, tdev, alpha, loglam, ta, logt);
+    ++g_nn_launches;
+    build_features_kept<<<nblk((long long)nm * M), 256, 0, st>>>(nm, lam, loglam, M, ta, logt, alpha, keep, kpos, X);
+    ++g_nn_launches;
+    NCK(cudaGetLastError());
+    return FHMG_OK;
+  }
   // FP64 coefficients (training targets): x is FP64, nl x N^dim; out FP32 nl x K^dim
   int project64(const double* x, int nl, float* out) {
     double *S64, *T;
@@ -945,7 +1311,7 @@ int fhmg_ws_predict(fhmg_wsnet net, fhmg_problem prob, const double* f, double a
   const int N = sp.N, M = sp.M, nm = sp.nm, dim = sp.dim;
   const long long npts = dim == 1 ? N : (long long)N * N;
   // coefficients of the source (constant in time: its last time level)
-  float *f32, *c, *X, *Y, *G, *T1, *U;
+  float *f32, *c, *X, *Y, *G, *T1;
   if ((s = sp.alloc(&f32, npts)) || (s = sp.alloc(&c, nm)) || (s = sp.alloc(&X, (size_t)nm * M * kFeat)) ||
       (s = sp.alloc(&Y, (size_t)nm * M)) || (s = sp.alloc(&G, (size_t)nm * M)))
     return s;
@@ -953,30 +1319,31 @@ int fhmg_ws_predict(fhmg_wsnet net, fhmg_problem prob, const double* f, double a
   ++g_nn_launches;
   NCK(cudaGetLastError());
   if ((s = sp.project(f32, 1, c))) return s;
-  build_features_kept<<<nblk((long long)nm * M), 256, 0, sp.st>>>(nm, sp.lam, M, sp.tdev, alpha, nullptr, nullptr, X);
-  ++g_nn_launches;
-  NCK(cudaGetLastError());
+  if ((s = sp.features(alpha, nullptr, nullptr, X))) return s;
   if ((s = fhmg_wsnet_forward(net, X, nm * M, bf16, Y, sp.st))) return s;
   mode_amplitudes<<<nblk((long long)nm * M), 256, 0, sp.st>>>(nm, M, c, Y, sp.lam, G);
   ++g_nn_launches;
   NCK(cudaGetLastError());
-  // synthesis u0[m] = sum_k G[m][k] s_k, in FP32, then widened to FP64
-  if ((s = sp.alloc(&U, (size_t)M * npts))) return s;
+  // synthesis u0[m] = sum_k G[m][k] s_k, in FP32, written as FP64
   if (dim == 1) {
-    // U (M x N) = G (M x K) S^T (K x N)
-    if ((s = gemm(sp.st, M, N, K, 1.f, G, K, 0, sp.S, K, 1, U, N))) return s;
+    // u0 (M x N) = G (M x K) S^T (K x N)
+    if ((s = gemm_to_f64(sp.st, M, N, sp.K, G, sp.K, sp.S, sp.K, 1, u0, N, 1, 0, 0, 0))) return s;
   } else {
-    if ((s = sp.alloc(&T1, (size_t)M * K * N))) return s;
-    // T1[m] = G[m] (K x K) S^T (K x N);  U[m] = S (N x K) T1[m] (K x N)
-    if ((s = gemm(sp.st, K, N, K, 1.f, G, K, 0, sp.S, K, 1, T1, N, M, (long long)K * K, 0, (long long)K * N)))
+    const int K2 = sp.K;
+    if ((s = sp.alloc(&T1, (size_t)M * K2 * N))) return s;
+    // T1[m] = G[m] (K x K) S^T (K x N);  u0[m] = S (N x K) T1[m] (K x N)
+    if ((s = gemm(sp.st, K2, N, K2, 1.f, G, K2, 0, sp.S, K2, 1, T1, N, M, (long long)K2 * K2, 0, (long long)K2 * N)))
       return s;
-    if ((s = gemm(sp.st, N, N, K, 1.f, sp.S, K, 0, T1, N, 0, U, N, M, 0, (long long)K * N, (long long)N * N)))
+    if ((s = gemm_to_f64(sp.st, N, N, K2, sp.S, K2, T1, N, 0, u0, N, M, 0, (long long)K2 * N, (long long)N * N)))
       return s;
   }
-  f2d<<<nblk((long long)M * npts), 256, 0, sp.st>>>((long long)M * npts, U, u0);
-  ++g_nn_launches;
-  NCK(cudaGetLastError());
+  int err = 0;
+  NCK(cudaMemcpyAsync(&err, net->err, sizeof err, cudaMemcpyDeviceToHost, sp.st));
   NCK(cudaStreamSynchronize(sp.st));
+  if (err) {
+    NCK(cudaMemsetAsync(net->err, 0, sizeof err, sp.st));
+    return fhmg_internal_fail(FHMG_ETIMEOUT, "the network kernel gave up waiting on a shared-memory stage");
+  }
   return FHMG_OK;
 }
 
@@ -1008,8 +1375,7 @@ int fhmg_ws_dataset(fhmg_problem prob, const double* u, const double* f, double 
   if ((s = sp.alloc(&dkeep, nm)) || (s = sp.alloc(&dkpos, nm))) return s;
   NCK(cudaMemcpyAsync(dkeep, keep.data(), sizeof(int) * nm, cudaMemcpyHostToDevice, sp.st));
   NCK(cudaMemcpyAsync(dkpos, kpos.data(), sizeof(int) * nm, cudaMemcpyHostToDevice, sp.st));
-  build_features_kept<<<nblk((long long)nm * M), 256, 0, sp.st>>>(nm, sp.lam, M, sp.tdev, alpha, dkeep, dkpos, X_out);
-  ++g_nn_launches;
+  if ((s = sp.features(alpha, dkeep, dkpos, X_out))) return s;
   mode_targets<<<nblk((long long)nm * M), 256, 0, sp.st>>>(nm, M, c, uh, sp.lam, rel_thr, dkeep, dkpos, Y_out);
   ++g_nn_launches;
   NCK(cudaGetLastError());

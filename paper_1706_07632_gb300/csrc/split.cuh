@@ -70,21 +70,6 @@ __host__ __device__ inline SplitSmem split_smem(int ns) {
   return s;
 }
 
-// ---- operand layout: K-major, 128-byte swizzle ----
-// A tile row holds its 64 K entries (BF16) in 128 bytes; 8-row groups form 1024-byte atoms in which
-// the 16-byte chunk c of row r sits at chunk position c ^ (r % 8) (the tensor core reads the atoms
-// without bank conflicts).  Tiles start on 1024-byte boundaries.
-__host__ __device__ inline uint32_t sp_sw128_off(int r, int k) {
-  return (uint32_t)((r >> 3) * 1024 + (r & 7) * 128 + ((((k >> 3) ^ r) & 7) << 4) + (k & 7) * 2);
-}
-// shared-memory descriptor of such a tile: start address, leading byte offset unused (1), 8-row
-// groups 1024 bytes apart, fixed bits 46-48 = 0b001, swizzle mode 128B (2 in bits 61-63); a K step
-// of 16 entries (32 bytes) advances the start address field by 2
-__device__ __forceinline__ uint64_t sp_desc_sw128(uint32_t addr) {
-  return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
-         ((uint64_t)2 << 61);
-}
-
 // ---- integer views of FP64 values (no FP64 arithmetic) ----
 
 // FP64 value of float f times 2^k, exactly, by integer operations (a conversion runs on the 1/64-rate
@@ -261,13 +246,6 @@ __global__ void __launch_bounds__(kPrepThreads) split_prep_kernel(const double* 
     if (r < ny) atomicMax(fe + (long long)(y0 + r) * N + x, (int)(mx[r] >> 20));
 }
 
-// one lane of a converged warp
-__device__ __forceinline__ bool sp_elect() {
-  uint32_t p;
-  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
-  return p != 0;
-}
-
 // Order of R~'s digits within a block: digit a takes part in 7 - a products, so long and short ones
 // alternate (0, 6, 1, 5, ...) and any two successive ring slots are held for about the same time.
 __host__ __device__ constexpr int sp_digit_at(int i) { return i & 1 ? kSpG - 1 - i / 2 : i / 2; }
@@ -383,10 +361,10 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
     // ---- MMA warp: every lane runs the loop, so that the descriptors stay in uniform registers; one
     // elected lane issues ----
     {
-      const bool leader = sp_elect();
+      const bool leader = umma_elect();
       const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
       // descriptors: K-major, 128-byte swizzle; a K step of 16 adds 2 to the address field
-      const uint64_t dbase = sp_desc_sw128(0);
+      const uint64_t dbase = sw128_desc(0);
       const uint32_t ring16 = smem_u32(ring) >> 4, xbuf16 = smem_u32(xbuf) >> 4;
       int slot = 0;
       uint32_t fphase = 0, accphase = 1, xphase = 0;  // accfree: the first block finds tensor memory free
@@ -548,7 +526,7 @@ __global__ void __launch_bounds__(kSpBlock, 1) split_defect_kernel(const __grid_
               sp_digit_pairs(sp_biased(v[8 * h + 2 * j], fe), sp_biased(v[8 * h + 2 * j + 1], fe), pk[j]);
 #pragma unroll
             for (int a = 0; a < kSpG; ++a)
-              *reinterpret_cast<uint4*>(xb + (size_t)a * kSpBtile + sp_sw128_off(sn, sk + 8 * h)) =
+              *reinterpret_cast<uint4*>(xb + (size_t)a * kSpBtile + sw128_off(sn, sk + 8 * h)) =
                   make_uint4(pk[0][a], pk[1][a], pk[2][a], pk[3][a]);
           }
           async_proxy_fence();

@@ -76,6 +76,21 @@ __device__ __forceinline__ uint32_t umma_idesc(int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kUmmaCols >> 4) << 24);
 }
 
+// ---- operand layout of 64-column tiles: K-major, 128-byte swizzle ----
+// A tile row holds its 64 K entries (BF16) in 128 bytes; 8-row groups form 1024-byte atoms in which
+// the 16-byte chunk c of row r sits at chunk position c ^ (r % 8) (the tensor core reads the atoms
+// without bank conflicts).  Tiles start on 1024-byte boundaries.
+__host__ __device__ inline uint32_t sw128_off(int r, int k) {
+  return (uint32_t)((r >> 3) * 1024 + (r & 7) * 128 + ((((k >> 3) ^ r) & 7) << 4) + (k & 7) * 2);
+}
+// shared-memory descriptor of such a tile: start address, leading byte offset unused (1), 8-row
+// groups 1024 bytes apart, fixed bits 46-48 = 0b001, swizzle mode 128B (2 in bits 61-63); a K step
+// of 16 entries (32 bytes) advances the start address field by 2
+__device__ __forceinline__ uint64_t sw128_desc(uint32_t addr) {
+  return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
+         ((uint64_t)2 << 61);
+}
+
 // D[tmem] (+)= A B^T over K = 16 * steps, A (128 x K) and B (N x K) K-major tiles at a_addr / b_addr
 __device__ __forceinline__ void umma_product(uint32_t tmem, uint32_t a_addr, uint32_t b_addr, int K, int N,
                                              bool accumulate) {

@@ -1,4 +1,4 @@
-"""Gradients of the warm-start network on ragged batch and layer widths (edges of the GEMM tiles, of the
+"""Gradients of the warm-start network and its one-launch BF16 inference on ragged batch and layer widths (edges of the GEMM tiles, of the
 16-byte loads and of the row splits), against the float64 oracle.
 
 Tolerance: every entry is a chain of at most 2 layers + 1 = 9 dot products; a float32 dot product of
@@ -32,3 +32,27 @@ def test_loss_and_gradient_on_ragged_shapes(hidden, layers, batch):
         n = w[l] * w[l + 1] + w[l + 1]
         assert np.linalg.norm(g[off:off + n] - ref[off:off + n]) <= 5e-5 * np.linalg.norm(ref[off:off + n])
         off += n
+
+
+def _bf16(x):
+    return torch.as_tensor(np.asarray(x, dtype=np.float32)).to(torch.bfloat16).to(torch.float64).numpy()
+
+
+@pytest.mark.parametrize("hidden,layers,rows", [(64, 1, 1), (64, 8, 129), (128, 2, 127), (192, 3, 128), (256, 4, 640),
+                                                (320, 1, 257), (320, 3, 50001)])
+def test_bf16_network_in_one_launch(hidden, layers, rows):
+    """Every width the one-launch network serves (row blocks of 128, several per CTA at 50001 rows; no
+    hidden product at one layer) against a layer-by-layer emulation.  An activation whose FP32 sum lies
+    near a rounding boundary may round to the neighbouring BF16 value (2^-8 relative), in a small share
+    of the terms of the next sum: 5e-3 of max|y|."""
+    net = fh.WSNet(hidden, layers, seed=5)
+    rng = np.random.default_rng(rows)
+    X = rng.uniform(-1, 1, (rows, 6)).astype(np.float32)
+    y = torch.empty(rows, dtype=torch.float32, device="cuda")
+    net.forward(torch.as_tensor(X, device="cuda"), y, bf16=True)
+    w = nn.widths(hidden, layers)
+    a = _bf16(X)
+    for l, (W, b) in enumerate(nn.unpack(net.get_params(), w)):
+        z = a @ _bf16(W).T + b.astype(np.float64)
+        a = _bf16(z / (1 + np.exp(-z))) if l < layers else z
+    assert np.max(np.abs(y.cpu().numpy() - a[:, 0])) <= 5e-3 * np.max(np.abs(a))
