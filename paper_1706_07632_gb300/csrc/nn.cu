@@ -24,6 +24,7 @@
 #include <cstring>
 #include <random>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "devinfo.h"
@@ -812,6 +813,10 @@ struct fhmg_wsnet_s {
   size_t part_n = 0;
   float* loss = nullptr;
   __nv_bfloat16* Abf[2] = {nullptr, nullptr};
+  // scratch of predictions, kept from call to call (the i-th buffer a prediction asks for, grown when it
+  // asks for more): every prediction ends synchronised, so no two use it at a time unless the net itself
+  // is shared by threads, which its other buffers exclude
+  std::vector<std::pair<void*, size_t>> ws;
   std::vector<void*> allocs;
 };
 
@@ -1005,6 +1010,7 @@ int fhmg_wsnet_create(int hidden, int layers, unsigned long long seed, fhmg_wsne
 int fhmg_wsnet_destroy(fhmg_wsnet net) {
   if (!net) return FHMG_OK;
   for (void* a : net->allocs) cudaFree(a);
+  for (auto& w : net->ws) cudaFree(w.first);
   delete net;
   return FHMG_OK;
 }
@@ -1219,7 +1225,9 @@ struct Spectral {
   double Lx;
   cudaStream_t st;
   const double* thost;
-  std::vector<void*> mem;
+  std::vector<void*> mem;  // buffers of its own (no net)
+  fhmg_wsnet net = nullptr;  // or the net whose scratch it uses, and the buffers taken so far
+  size_t taken = 0;
   float* S = nullptr;   // N x K
   double* lam = nullptr;
   double* tdev = nullptr;
@@ -1228,9 +1236,20 @@ struct Spectral {
   }
   template <typename T>
   int alloc(T** p, size_t n) {
-    cudaError_t e = cudaMalloc((void**)p, (n ? n : 1) * sizeof(T));
+    const size_t bytes = (n ? n : 1) * sizeof(T);
+    if (net && taken < net->ws.size() && net->ws[taken].second >= bytes) {
+      *p = (T*)net->ws[taken++].first;
+      return FHMG_OK;
+    }
+    cudaError_t e = cudaMalloc((void**)p, bytes);
     if (e != cudaSuccess) return fhmg_internal_fail(FHMG_ENOMEM, cudaGetErrorString(e));
-    mem.push_back(*p);
+    if (!net) {
+      mem.push_back(*p);
+      return FHMG_OK;
+    }
+    if (taken == net->ws.size()) net->ws.push_back({nullptr, 0});
+    cudaFree(net->ws[taken].first);
+    net->ws[taken++] = {*p, bytes};
     return FHMG_OK;
   }
   int init(fhmg_problem p, int K_) {
@@ -1306,6 +1325,7 @@ int fhmg_wsnet_launches(long long* n) {
 int fhmg_ws_predict(fhmg_wsnet net, fhmg_problem prob, const double* f, double alpha, int K, int bf16, double* u0) {
   if (!net || !prob || !f || !u0 || K < 1) return fhmg_internal_fail(FHMG_EINVAL, "bad arguments");
   Spectral sp;
+  sp.net = net;
   int s = sp.init(prob, K);
   if (s) return s;
   const int N = sp.N, M = sp.M, nm = sp.nm, dim = sp.dim;
