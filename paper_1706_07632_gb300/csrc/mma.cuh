@@ -257,32 +257,58 @@ __global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkB
       }
     const long long nstep[4] = {-1, 1, -(long long)J.geo.N, (long long)J.geo.N};
     double local_max = 0.0;
-    T bn[NTL][4], xn[NTL][4], dn[2];
+    // RAW (tile 16): the neighbours are kept as loaded and summed when the leaf begins; summed here they
+    // would make the warp wait for them at once (172 -> 160 us per half-sweep of 4095 x 512; a tile of
+    // 32 has no registers to spare for them).  Missing neighbours and columns past the panel's end read
+    // an element of their column 0 or their own and are replaced by zeros, so that no load sits behind a
+    // branch: the loads of an n-tile are in flight together (with branches a leaf's loads took 7300 of
+    // its 20100 cycles at tile 32).
+    constexpr bool RAW = MODE == MODE_SMOOTH && NTL == 1;
+    T bn[NTL][4], xn[NTL][4], dn[2], un[RAW ? NTL : 1][4][4];
     auto load_rhs = [&](int leaf) {
+      if (leaf >= nb) return;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) dn[h] = (leaf < nb) ? ddg[(long long)leaf * L + rt * 16 + g + 8 * h] : (T)0;
+      for (int h = 0; h < 2; ++h) dn[h] = ddg[(long long)leaf * L + rt * 16 + g + 8 * h];
 #pragma unroll
-      for (int nt = 0; nt < NTL; ++nt)
+      for (int nt = 0; nt < NTL; ++nt) {
+        T v[4], u[4][4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const int h = j >> 1, e = j & 1;
-          T b = 0, x = 0;
-          if (leaf < nb && vcol[nt][e]) {
-            const long long base = (long long)(leaf * L + rt * 16 + g + 8 * h) * ld + pcol[nt][e];
-            b = Bsrc[base];
-            if (MODE == MODE_SMOOTH) {
-              T s = 0;
+          const long long base = (long long)(leaf * L + rt * 16 + g + 8 * h) * ld + (vcol[nt][e] ? pcol[nt][e] : 0);
+          v[j] = Bsrc[base];
+          if (MODE == MODE_SMOOTH) {
+            if (J.geo.dim > 0) {
 #pragma unroll
-              for (int d = 0; d < 4; ++d)
-                if (nmask[nt][e] & (1 << d)) s += X[base + nstep[d]];
-              b += s * inv_h2;
+              for (int d = 0; d < 4; ++d) u[j][d] = X[base + ((nmask[nt][e] >> d) & 1 ? nstep[d] : 0)];
             } else {
-              x = X[base];
+#pragma unroll
+              for (int d = 0; d < 4; ++d) u[j][d] = 0;
             }
+          } else {
+            xn[nt][j] = X[base];
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int e = j & 1;
+          T b = vcol[nt][e] ? v[j] : (T)0;
+          if (MODE == MODE_SMOOTH) {
+#pragma unroll
+            for (int d = 0; d < 4; ++d) {
+              if (!((nmask[nt][e] >> d) & 1)) u[j][d] = 0;
+              if (RAW) un[RAW ? nt : 0][j][d] = u[j][d];
+            }
+            if (!RAW) {
+              const T s = ((u[j][0] + u[j][1]) + u[j][2]) + u[j][3];
+              b += s * inv_h2;
+            }
+          } else if (!vcol[nt][e]) {
+            xn[nt][j] = 0;
           }
           bn[nt][j] = b;
-          xn[nt][j] = x;
         }
+      }
     };
     load_rhs(0);
 
@@ -295,6 +321,11 @@ __global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkB
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           rhs[nt][j] = bn[nt][j];
+          if (RAW) {
+            const int r = RAW ? nt : 0;
+            const T s = ((un[r][j][0] + un[r][j][1]) + un[r][j][2]) + un[r][j][3];
+            rhs[nt][j] += s * inv_h2;
+          }
           xcur[nt][j] = xn[nt][j];
         }
       }

@@ -264,6 +264,7 @@ __global__ void __launch_bounds__(NT_ + 32) hpanel_kernel(const __grid_constant_
   constexpr int STEP = TC * RL;            // lane offset between splits
   constexpr int LP = L + VE;               // padded x-tile column
   constexpr bool SPLITD = sizeof(TM) < 8;  // FP32 products: diagonal from ddiag, in T
+  constexpr bool RAW = MODE == MODE_SMOOTH && (Q == 1 || (Q == 2 && sizeof(T) == 8));
   extern __shared__ __align__(16) unsigned char sm[];
   const PanelSmem lay = panel_smem(L, TC, B.pool, B.W, B.slot_bytes, B.ns, sizeof(TM));
   unsigned char* slots = sm;
@@ -393,22 +394,44 @@ __global__ void __launch_bounds__(NT_ + 32) hpanel_kernel(const __grid_constant_
     // right-hand side, x tile (product) and diagonal term (FP32 products) of the next leaf,
     // prefetched a leaf ahead by the threads that use them (issued at the diagonal step: issuing
     // them a whole leaf ahead raised the register count past the two-CTA occupancy)
-    T bn[Q], xn[Q], dn[Q];
+    // RAW (few values per thread): the neighbours are kept as loaded and summed at the next diagonal
+    // step; summed here they would make the warp wait for them (about 1000 cycles per leaf)
+    T bn[Q], xn[Q], dn[Q], un[RAW ? Q : 1][4];
     auto load_rhs = [&](int leaf) {
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
         const int r = rb + RG * q;
         T b = 0, x = 0, d = 0;
+        if (RAW) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) un[RAW ? q : 0][e] = 0;
+        }
         if (act && sp == 0 && leaf < nb) {
           if (SPLITD) d = ddg[(long long)leaf * L + r];
           if (valid) {
             const long long base = (long long)(leaf * L + r) * ld;
             b = Bsrc[base + p];
-            if (MODE == MODE_SMOOTH) {
-              T s = 0;
+            if (MODE == MODE_SMOOTH && RAW) {
 #pragma unroll
               for (int e = 0; e < 4; ++e)
-                if (nbr[e] >= 0) s += X[base + nbr[e]];
+                if (nbr[e] >= 0) un[RAW ? q : 0][e] = X[base + nbr[e]];
+            } else if (MODE == MODE_SMOOTH) {
+              T s = 0;
+              if (SPLITD && J.geo.dim > 0) {
+                // FP32 products: no load behind a branch (missing neighbours read the column itself), so
+                // that the loads of several values are in flight together (111 -> 102 us per half-sweep
+                // of 63^2 x 1024); the FP64 products' tiles lose more by the registers (682 -> 700 us at
+                // 127^2 x 256)
+                T u[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) u[e] = X[base + (nbr[e] >= 0 ? nbr[e] : p)];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) s += nbr[e] >= 0 ? u[e] : (T)0;
+              } else if (!SPLITD) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                  if (nbr[e] >= 0) s += X[base + nbr[e]];
+              }
               b += s * inv_h2;
             } else {
               x = X[base + p];
@@ -476,7 +499,13 @@ __global__ void __launch_bounds__(NT_ + 32) hpanel_kernel(const __grid_constant_
           }
         } else if (type == PK_DIAG) {
 #pragma unroll
-          for (int q = 0; q < Q; ++q) acc[q] = reduce_splits<T, STEP>(acc[q] - (T)sum4(part[q]));
+          for (int q = 0; q < Q; ++q) {
+            if (RAW && MODE == MODE_SMOOTH) {
+              const T s = ((un[q][0] + un[q][1]) + un[q][2]) + un[q][3];
+              acc[q] += s * inv_h2;
+            }
+            acc[q] = reduce_splits<T, STEP>(acc[q] - (T)sum4(part[q]));
+          }
           // the operand of the diagonal product: y (smoother) or x_i (product), in TM
           TM* opnd = MODE == MODE_SMOOTH ? ysm + cl * LP : xr_i;
           if (sp == 0 && act) {
