@@ -94,7 +94,7 @@ int panel_dispatch(cudaStream_t st, const WalkArgsT<T>* jobs, int njobs, std::st
       mma_ok = mma_ok && jobs[j].PM.pkg != nullptr && !jobs[j].PM.far && jobs[j].dinv_cstride == 0;
     if (mma_ok) {
       int tcm = jobs[0].tile;
-      if (tcm == 0) tcm = total_cols >= 32LL * sms ? 32 : (total_cols + 15) / 16 >= 128 ? 16 : 0;
+      if (tcm == 0) tcm = total_cols >= 32LL * sms ? 32 : total_cols >= 2048 ? 16 : 0;
       if (tcm == 16 || tcm == 32) {
         if (tile_used) *tile_used = tcm;
         WalkBatch<T, float> Bm;
