@@ -14,6 +14,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "kernels.cuh"
+
 namespace fhmg {
 
 // (D_ii + lam_k I)^{-1} for every diagonal leaf i of R~ and every mode k, in the layout of the
@@ -89,11 +91,22 @@ __global__ void sine_fft_kernel(const Tin* __restrict__ in, Tout* __restrict__ o
     base = m * (long long)ny * nx + x;
     stride = nx;
   }
+  // FP32 grid functions of 2D problems are stored by colour (lines along x: axis 0)
+  const int iy = (int)(line % ny);
+  const long long mbase = line / ny * ((long long)ny * nx);
+  auto src = [&](int k) -> long long {
+    if (sizeof(Tin) == 4 && ny > 1) return mbase + split_pos(nx, iy, k);
+    return base + (long long)k * stride;
+  };
+  auto dst = [&](int k) -> long long {
+    if (sizeof(Tout) == 4 && ny > 1) return mbase + split_pos(nx, iy, k);
+    return base + (long long)k * stride;
+  };
   // odd extension, stored at bit-reversed positions
   for (int j = threadIdx.x; j < P; j += blockDim.x) {
     double v = 0.0;
-    if (j >= 1 && j <= n) v = (double)in[base + (long long)(j - 1) * stride];
-    else if (j >= n + 2) v = -(double)in[base + (long long)(P - j - 1) * stride];
+    if (j >= 1 && j <= n) v = (double)in[src(j - 1)];
+    else if (j >= n + 2) v = -(double)in[src(P - j - 1)];
     const int r = (int)(__brev((unsigned)j) >> (32 - log2P));
     re[r] = v;
     im[r] = 0.0;
@@ -115,7 +128,7 @@ __global__ void sine_fft_kernel(const Tin* __restrict__ in, Tout* __restrict__ o
     __syncthreads();
   }
   const double sc = -0.5 * sqrt(2.0 / (n + 1));
-  for (int k = threadIdx.x; k < n; k += blockDim.x) out[base + (long long)k * stride] = (Tout)(sc * im[k + 1]);
+  for (int k = threadIdx.x; k < n; k += blockDim.x) out[dst(k)] = (Tout)(sc * im[k + 1]);
 }
 
 }  // namespace fhmg

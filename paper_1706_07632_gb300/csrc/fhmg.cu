@@ -219,6 +219,8 @@ dim3 coarse_grid(int dim, int Nf, int M) {
   return fhmg::plane_grid(Nc, dim == 1 ? 1 : Nc, M, fhmg::device_sms());
 }
 dim3 fine_grid(int dim, int N, int M) { return fhmg::plane_grid(N, dim == 1 ? 1 : N, M, fhmg::device_sms()); }
+// ... a thread per pair of points of a row (2D)
+dim3 pair_grid(int N, int M) { return fhmg::plane_grid((N + 1) / 2, N, M, fhmg::device_sms()); }
 dim3 colour_grid(int dim, int N, int M) {
   return fhmg::plane_grid((N + 1) / 2, dim == 1 ? 1 : N, M, fhmg::device_sms());
 }
@@ -297,6 +299,12 @@ template <> float* lev_RC<float>(LevelData& lv) { return lv.RC32; }
 template <typename T> T* scratch_X(fhmg_problem p);
 template <> double* scratch_X<double>(fhmg_problem p) { return p->Xs; }
 template <> float* scratch_X<float>(fhmg_problem p) { return p->Xs32; }
+
+// FP32 grid functions of 2D problems are stored by colour (split_pos), all others by rows.
+template <typename T>
+int by_colour(fhmg_problem p) {
+  return sizeof(T) == 4 && p->dim == 2 ? 1 : 0;
+}
 
 // A smoother half-sweep / line-solve job on level l (shift of that level).
 template <typename T>
@@ -419,7 +427,7 @@ int sweep(fhmg_problem p, int l, T* u, const T* F, int kind) {
   for (int colour = 0; colour < 2; ++colour) {
     const long long nc = fhmg::colour_count(p->dim, lv.N, colour);
     if (nc == 0) continue;
-    Geo g{p->dim, lv.N, colour, lv.npts, lv.inv_h2};
+    Geo g{p->dim, lv.N, colour, lv.npts, lv.inv_h2, by_colour<T>(p)};
     const bool rec = p->profile && l == p->nlev - 1;
     if (rec) TRY(record_event(p, p->ev, p->ev_used));
     TRY(walk_smooth<T>(p, l, kind, g, nc, u, F));
@@ -434,8 +442,12 @@ int restrict_defect(fhmg_problem p, int l, const T* u, const T* F, T* rc, int ki
   LevelData& lv = p->lev[l];
   LevelData& lc = p->lev[l - 1];
   T* xs = scratch_X<T>(p);
-  fhmg::restrict_pre_kernel<T><<<coarse_grid(p->dim, lv.N, p->M), 256, 0, p->st>>>(p->dim, lv.N, lv.inv_h2, p->M, u, F,
-                                                                                  xs, rc);
+  if (by_colour<T>(p))
+    fhmg::restrict_pre_split_kernel<T><<<fhmg::split_grid(lc.N, lc.N, p->M, fhmg::device_sms()), fhmg::split_block(), 0,
+                                         p->st>>>(lv.N, lv.inv_h2, p->M, u, F, xs, rc);
+  else
+    fhmg::restrict_pre_kernel<T><<<coarse_grid(p->dim, lv.N, p->M), 256, 0, p->st>>>(p->dim, lv.N, lv.inv_h2, p->M, u, F,
+                                                                                    xs, rc);
   ++p->launches;
   CK(cudaGetLastError());
   return walk_matvec<T>(p, kind, lc.npts, xs, rc, rc, nullptr);
@@ -443,7 +455,11 @@ int restrict_defect(fhmg_problem p, int l, const T* u, const T* F, T* rc, int ki
 
 template <typename T>
 int prolong_add(fhmg_problem p, int l, const T* e, T* u) {
-  fhmg::prolong_add_kernel<T><<<fine_grid(p->dim, p->lev[l].N, p->M), 256, 0, p->st>>>(p->dim, p->lev[l].N, p->M, e, u);
+  if (by_colour<T>(p))
+    fhmg::prolong_add_split_kernel<T><<<fhmg::split_grid((p->lev[l].N + 1) / 2, p->lev[l].N, p->M, fhmg::device_sms()),
+                                        fhmg::split_block(), 0, p->st>>>(p->lev[l].N, p->M, e, u);
+  else
+    fhmg::prolong_add_kernel<T><<<fine_grid(p->dim, p->lev[l].N, p->M), 256, 0, p->st>>>(p->dim, p->lev[l].N, p->M, e, u);
   ++p->launches;
   CK(cudaGetLastError());
   return FHMG_OK;
@@ -531,6 +547,41 @@ __global__ void add_float_kernel(double* y, const float* x, long long n) {
     y[i] += (double)x[i];
 }
 
+struct ToFloat {
+  __device__ float operator()(double v) const { return d2f_int(v); }
+};
+// y = x (FP32 from FP64), x = y and x += y on the grid functions of a level of N points per dimension
+int copy_to_float(fhmg_problem p, int N, const double* x, float* y) {
+  if (p->dim == 2)
+    fhmg::split_copy_kernel<fhmg::SPLIT_FROM><<<pair_grid(N, p->M), 256, 0, p->st>>>(N, p->M, const_cast<double*>(x), y,
+                                                                                     ToFloat());
+  else
+    to_float_kernel<<<blocks_for((long long)N * p->M), 256, 0, p->st>>>(x, y, (long long)N * p->M);
+  ++p->launches;
+  CK(cudaGetLastError());
+  return FHMG_OK;
+}
+int copy_to_double(fhmg_problem p, int N, const float* y, double* x) {
+  if (p->dim == 2)
+    fhmg::split_copy_kernel<fhmg::SPLIT_TO><<<pair_grid(N, p->M), 256, 0, p->st>>>(N, p->M, x, const_cast<float*>(y),
+                                                                                   ToFloat());
+  else
+    to_double_kernel<<<blocks_for((long long)N * p->M), 256, 0, p->st>>>(y, x, (long long)N * p->M);
+  ++p->launches;
+  CK(cudaGetLastError());
+  return FHMG_OK;
+}
+int add_from_float(fhmg_problem p, int N, double* x, const float* y) {
+  if (p->dim == 2)
+    fhmg::split_copy_kernel<fhmg::SPLIT_ADD><<<pair_grid(N, p->M), 256, 0, p->st>>>(N, p->M, x, const_cast<float*>(y),
+                                                                                    ToFloat());
+  else
+    add_float_kernel<<<blocks_for((long long)N * p->M), 256, 0, p->st>>>(x, y, (long long)N * p->M);
+  ++p->launches;
+  CK(cudaGetLastError());
+  return FHMG_OK;
+}
+
 // Storage of a coarse-grid correction on level l inside FP64-storage inner cycles (automatic
 // mixed storage only): FP32 where the stencil's conditioning allows it,
 // eps32 * cond(A_h) ~ 6e-8 * 4 (N+1)^2 / pi^2 <= 0.05 (N <= 1023 per dimension).
@@ -555,15 +606,10 @@ int coarse_correction(fhmg_problem p, int l, int nu1, int nu2, int kind) {
   const int reps = l - 1 > 0 ? p->cycle_index : 1;
   if constexpr (std::is_same<T, double>::value) {
     if (kind == KSPLIT && level_fp32(p, l - 1)) {
-      to_float_kernel<<<blocks_for(n), 256, 0, p->st>>>(lc.RC, lc.RC32, n);
-      ++p->launches;
-      CK(cudaGetLastError());
+      TRY(copy_to_float(p, lc.N, lc.RC, lc.RC32));
       CK(cudaMemsetAsync(lc.E32, 0, sizeof(float) * n, p->st));
       for (int r = 0; r < reps; ++r) TRY(vcycle_rec<float>(p, l - 1, lc.E32, lc.RC32, nu1, nu2, K32));
-      to_double_kernel<<<blocks_for(n), 256, 0, p->st>>>(lc.E32, lc.E, n);
-      ++p->launches;
-      CK(cudaGetLastError());
-      return FHMG_OK;
+      return copy_to_double(p, lc.N, lc.E32, lc.E);
     }
   }
   CK(cudaMemsetAsync(lev_E<T>(lc), 0, sizeof(T) * n, p->st));
@@ -806,15 +852,11 @@ int solve_mixed(fhmg_problem p, double* u, const double* F, int nu1, int nu2, do
     }
     const int k_round = k;
     if (f32) {
-      to_float_kernel<<<blocks_for(n), 256, 0, p->st>>>(p->Rs, p->Rs32, n);
-      ++p->launches;
-      CK(cudaGetLastError());
+      TRY(copy_to_float(p, p->N, p->Rs, p->Rs32));
       CK(cudaMemsetAsync(p->Ef32, 0, sizeof(float) * n, p->st));
       for (int j = 0; j < cyc && k < max_cycles; ++j, ++k)
         TRY(vcycle_rec<float>(p, p->nlev - 1, p->Ef32, p->Rs32, nu1, nu2, K32));
-      add_float_kernel<<<blocks_for(n), 256, 0, p->st>>>(u, p->Ef32, n);
-      ++p->launches;
-      CK(cudaGetLastError());
+      TRY(add_from_float(p, p->N, u, p->Ef32));
     } else {
       CK(cudaMemsetAsync(p->Ef, 0, sizeof(double) * n, p->st));
       for (int j = 0; j < cyc && k < max_cycles; ++j, ++k)

@@ -238,7 +238,12 @@ __global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkB
     const int nb = J.P.nb;
     // the lane's accumulator columns: n-tile nt, e = 0, 1 -> column cb + nt*8 + 2 tq + e
     long long pcol[NTL][2];
-    int nmask[NTL][2];  // bit d: neighbour d exists (1D: -1, +1; 2D: also -N, +N)
+    int nmask[NTL][2];  // bit d: neighbour d exists (1D: left, right; 2D: also up, down)
+    // places of the left, upper and lower neighbours relative to the point (FP32 grid functions, which may
+    // be stored by colour; the others' are -1, -N, N)
+    constexpr bool SPL = sizeof(T) == 4;
+    int noff[NTL][2][3];
+    const NbrOffsets off = nbr_offsets(J.geo);
     bool vcol[NTL][2];
 #pragma unroll
     for (int nt = 0; nt < NTL; ++nt)
@@ -248,14 +253,21 @@ __global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkB
         vcol[nt][e] = cg < J.ncols;
         pcol[nt][e] = cg;
         nmask[nt][e] = 0;
+        noff[nt][e][0] = noff[nt][e][1] = noff[nt][e][2] = 0;
         if (vcol[nt][e] && MODE == MODE_SMOOTH && J.geo.dim > 0) {
           int iy, ix;
           pcol[nt][e] = colour_pos(J.geo.dim, J.geo.N, J.geo.colour, cg, &iy, &ix);
+          if (SPL && J.geo.split) pcol[nt][e] = cg + (J.geo.colour ? colour_count(2, J.geo.N, 0) : 0);
           nmask[nt][e] = (ix > 0 ? 1 : 0) | (ix < J.geo.N - 1 ? 2 : 0);
           if (J.geo.dim == 2) nmask[nt][e] |= (iy > 0 ? 4 : 0) | (iy < J.geo.N - 1 ? 8 : 0);
+          if (SPL) {
+            const bool odd = iy & 1;
+            noff[nt][e][0] = odd ? off.left[1] : off.left[0];
+            noff[nt][e][1] = odd ? off.up[1] : off.up[0];
+            noff[nt][e][2] = odd ? off.down[1] : off.down[0];
+          }
         }
       }
-    const long long nstep[4] = {-1, 1, -(long long)J.geo.N, (long long)J.geo.N};
     double local_max = 0.0;
     // RAW (tile 16): the neighbours are kept as loaded and summed when the leaf begins; summed here they
     // would make the warp wait for them at once (172 -> 160 us per half-sweep of 4095 x 512; a tile of
@@ -280,7 +292,12 @@ __global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkB
           if (MODE == MODE_SMOOTH) {
             if (J.geo.dim > 0) {
 #pragma unroll
-              for (int d = 0; d < 4; ++d) u[j][d] = X[base + ((nmask[nt][e] >> d) & 1 ? nstep[d] : 0)];
+              for (int d = 0; d < 4; ++d) {
+                const int o = !SPL ? (d == 0 ? -1 : d == 1 ? 1 : d == 2 ? -J.geo.N : J.geo.N)
+                              : d < 2 ? noff[nt][e][0] + (d ? off.step : 0)
+                                      : noff[nt][e][d - 1];
+                u[j][d] = X[base + ((nmask[nt][e] >> d) & 1 ? o : 0)];
+              }
             } else {
 #pragma unroll
               for (int d = 0; d < 4; ++d) u[j][d] = 0;

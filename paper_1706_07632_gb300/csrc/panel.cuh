@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(NT_ + 32) hpanel_kernel(const __grid_constant_
   constexpr int STEP = TC * RL;            // lane offset between splits
   constexpr int LP = L + VE;               // padded x-tile column
   constexpr bool SPLITD = sizeof(TM) < 8;  // FP32 products: diagonal from ddiag, in T
-  constexpr bool RAW = MODE == MODE_SMOOTH && (Q == 1 || (Q == 2 && sizeof(T) == 8));
+  constexpr bool RAW = MODE == MODE_SMOOTH && SPLITD && (Q == 1 || (Q == 2 && sizeof(T) == 8));
   extern __shared__ __align__(16) unsigned char sm[];
   const PanelSmem lay = panel_smem(L, TC, B.pool, B.W, B.slot_bytes, B.ns, sizeof(TM));
   unsigned char* slots = sm;
@@ -380,11 +380,21 @@ __global__ void __launch_bounds__(NT_ + 32) hpanel_kernel(const __grid_constant_
       if (MODE == MODE_SMOOTH && J.geo.dim > 0) {
         int iy, ix;
         p = colour_pos(J.geo.dim, J.geo.N, J.geo.colour, cg, &iy, &ix);
-        nbr[0] = ix > 0 ? p - 1 : -1;
-        nbr[1] = ix < J.geo.N - 1 ? p + 1 : -1;
+        long long left = -1, right = 1, up = -(long long)J.geo.N, down = J.geo.N;
+        if (sizeof(T) == 4 && J.geo.split) {  // only FP32 grid functions are stored by colour
+          p = cg + (J.geo.colour ? colour_count(2, J.geo.N, 0) : 0);
+          const NbrOffsets off = nbr_offsets(J.geo);
+          const bool odd = iy & 1;
+          left = odd ? off.left[1] : off.left[0];
+          right = left + 1;
+          up = odd ? off.up[1] : off.up[0];
+          down = odd ? off.down[1] : off.down[0];
+        }
+        nbr[0] = ix > 0 ? p + left : -1;
+        nbr[1] = ix < J.geo.N - 1 ? p + right : -1;
         if (J.geo.dim == 2) {
-          nbr[2] = iy > 0 ? p - J.geo.N : -1;
-          nbr[3] = iy < J.geo.N - 1 ? p + J.geo.N : -1;
+          nbr[2] = iy > 0 ? p + up : -1;
+          nbr[3] = iy < J.geo.N - 1 ? p + down : -1;
         }
       } else {
         p = cg;
@@ -394,7 +404,7 @@ __global__ void __launch_bounds__(NT_ + 32) hpanel_kernel(const __grid_constant_
     // right-hand side, x tile (product) and diagonal term (FP32 products) of the next leaf,
     // prefetched a leaf ahead by the threads that use them (issued at the diagonal step: issuing
     // them a whole leaf ahead raised the register count past the two-CTA occupancy)
-    // RAW (few values per thread): the neighbours are kept as loaded and summed at the next diagonal
+    // RAW (FP32 products, few values per thread): the neighbours are kept as loaded and summed at the next diagonal
     // step; summed here they would make the warp wait for them (about 1000 cycles per leaf)
     T bn[Q], xn[Q], dn[Q], un[RAW ? Q : 1][4];
     auto load_rhs = [&](int leaf) {

@@ -412,10 +412,14 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
           if (J.geo.dim == 2 && iy > 0) w2 = inv_h2;
           if (J.geo.dim == 2 && iy < N - 1) w3 = inv_h2;
         }
-        n0 = w0 != 0.f ? p - 1 : p;
-        n1 = w1 != 0.f ? p + 1 : p;
-        n2 = w2 != 0.f ? p - N : p;
-        n3 = w3 != 0.f ? p + N : p;
+        if (J.geo.split && valid) p = split_pos(N, iy, ix);
+        const NbrOffsets off = nbr_offsets(J.geo);
+        const bool odd = iy & 1;
+        const int left = odd ? off.left[1] : off.left[0];
+        n0 = w0 != 0.f ? p + left : p;
+        n1 = w1 != 0.f ? p + left + off.step : p;
+        n2 = w2 != 0.f ? p + (odd ? off.up[1] : off.up[0]) : p;
+        n3 = w3 != 0.f ? p + (odd ? off.down[1] : off.down[0]) : p;
       } else {
         const long long cg = (g - J.tile0) * NT + c;
         valid = cg < J.ncols;
