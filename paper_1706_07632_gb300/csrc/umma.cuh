@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
       tc_after_sync();
       const Dest d = buf ? d1 : d0;
       const long long ld = d.J->geo.ld;
-#pragma unroll
+#pragma unroll 1
       for (int r0 = 0; r0 < L; r0 += 16) {
         float a[16];
         tmem_ld16(t_buf + 64 * buf + r0, a);
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
         if (grid) {
           const float* Bl = J.B + at + p;
           const float* Xl = J.X + at;
-#pragma unroll
+#pragma unroll 1
           for (int r0 = 0; r0 < L; r0 += 8) {
             float v[8], a0[8], a1[8], a2[8], a3[8];
             uint32_t q[8];
@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
           }
         } else if (MODE == MODE_SMOOTH) {
           const float* Bl = J.B + at + p;
-#pragma unroll
+#pragma unroll 1
           for (int r0 = 0; r0 < L; r0 += 32) {
             float v[32];
 #pragma unroll
@@ -471,7 +471,7 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
           }
         } else {
           const float* Xl = J.X + at + p;
-#pragma unroll
+#pragma unroll 1
           for (int r0 = 0; r0 < L; r0 += 32) {
             float v[32];
 #pragma unroll
@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
             break;
           }
           tc_after_sync();
-#pragma unroll
+#pragma unroll 1
           for (int r0 = 0; r0 < L / 2; r0 += 16) {
             float v[16];
             tmem_ld16(t_b + r0, v);
@@ -612,7 +612,7 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
               }
               tc_after_sync();
               // y = b - acc, kept in the leaf buffer and staged as the A operand of the inverse's product
-#pragma unroll
+#pragma unroll 1
               for (int r0 = 0; r0 < L; r0 += 16) {
                 float y[16];
                 tmem_ld16(t_b + r0, y);
@@ -642,7 +642,7 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
               }
               // x = res + dinv_rr y into the ring and, for the memory warps, the leaf buffer
               const float* dd = ddg + (long long)i * L;
-#pragma unroll
+#pragma unroll 1
               for (int r0 = 0; r0 < L; r0 += 16) {
                 float a[16], y[16];
                 tmem_ld16(t_acc + lane_base + r0, a);
@@ -673,7 +673,7 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
                 failed = true;
                 break;
               }
-#pragma unroll
+#pragma unroll 1
               for (int r0 = 0; r0 < L; r0 += 16) {
                 float a[16];
                 tmem_ld16(t_acc + lane_base + r0, a);
