@@ -76,6 +76,27 @@ inline cudaError_t prepare_launch(K kern, int block, size_t smem, KernelCache& c
   return cudaSuccess;
 }
 
+// Launches kern with the smallest shared-memory configuration that holds `per_sm` CTAs of smem bytes (each
+// with 1 KB of the system's), so that the rest of the SM's 256 KB serves as L1 cache: left to itself the
+// driver takes the largest.  The preference belongs to this launch alone.
+template <typename A>
+inline cudaError_t launch_sized(void (*kern)(A), long long grid, int block, size_t smem, int per_sm, cudaStream_t st,
+                                const A& arg) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  const size_t most = 228 * 1024;
+  const size_t pct = ((smem + 1024) * (size_t)per_sm * 100 + most - 1) / most;
+  at[0].val.sharedMemCarveout = (unsigned)(pct > 100 ? 100 : pct);
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, arg);
+}
+
 // Grid of a grid-stride elementwise kernel over n items with 256-thread blocks: enough blocks for
 // every item, at most per_sm blocks per SM of the current device.
 inline int grid_for(long long n, int per_sm) {

@@ -34,20 +34,21 @@ constexpr int kUmmaBlock = 2 * kUmmaCols + 32;  // walk threads, memory threads,
 constexpr uint32_t kUmmaTmemCols = 256;        // acc / res [0,64), v [64,128), two leaf buffers [128,256)
 
 struct UmmaSmem {
-  size_t ring, ystage, zstage, zpool, bar, ebar, cbar, xbar, desc, flag, tslot, total;
+  size_t ring, zstage, zpool, bar, ebar, cbar, xbar, desc, flag, tslot, total;
 };
-// x ring (W tiles), one staging tile (128 x 64 BF16 each) that holds the columns' z values for the
-// U products and, later in the same leaf, y for the inverse's product (the U products have then
-// completed), z pool (pool x 128 FP32), mbarriers, slot descriptors, abort flag, TMEM address.
+// x ring (W tiles of 128 x 64 BF16), for the product one staging tile that holds the columns' z values for
+// the U products, z pool (pool x 128 FP32), mbarriers, slot descriptors, abort flag, TMEM address.  The
+// smoother stages z, then y (for the inverse's product), in the tile that x_i takes at the end of the
+// leaf (each is read by MMAs that completed before the next is written), and so leaves the L1 cache
+// room: its lines are what the memory warps' loads in flight wait for (see umma_launch_t).
 // Operand tiles are 128-byte aligned.
-__host__ __device__ inline UmmaSmem umma_smem(int pool, int W, int slot_bytes, int ns) {
+__host__ __device__ inline UmmaSmem umma_smem(int pool, int W, int slot_bytes, int ns, bool smoother) {
   auto a128 = [](size_t x) { return (x + 127) & ~(size_t)127; };
   const size_t tile = (size_t)kUmmaCols * kUmmaL * 2;
   UmmaSmem s;
   s.ring = a128((size_t)ns * slot_bytes);
-  s.ystage = s.ring + (size_t)W * tile;
-  s.zstage = s.ystage;
-  s.zpool = s.ystage + tile;
+  s.zstage = s.ring + (size_t)W * tile;
+  s.zpool = s.zstage + (smoother ? 0 : tile);
   s.bar = a128(s.zpool + (size_t)pool * kUmmaCols * 4);
   s.ebar = s.bar + 8 * (size_t)ns;
   s.cbar = s.ebar + 8 * (size_t)ns;  // consumer warps' barrier
@@ -212,11 +213,9 @@ template <int MODE>
 __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_constant__ WalkBatch<float, uint16_t> B) {
   constexpr int L = kUmmaL, NT = kUmmaCols;
   extern __shared__ __align__(16) unsigned char sm[];
-  const UmmaSmem lay = umma_smem(B.pool, B.W, B.slot_bytes, B.ns);
+  const UmmaSmem lay = umma_smem(B.pool, B.W, B.slot_bytes, B.ns, MODE == MODE_SMOOTH);
   unsigned char* slots = sm;
   unsigned char* ring = sm + lay.ring;
-  unsigned char* ystage = sm + lay.ystage;
-  unsigned char* zstage = sm + lay.zstage;
   float* zpool = reinterpret_cast<float*>(sm + lay.zpool);
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + lay.bar);
   uint64_t* empty = reinterpret_cast<uint64_t*>(sm + lay.ebar);
@@ -530,6 +529,8 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
       const int nb = J.P.nb;
       for (int i = 0; i < nb && !failed; ++i, ++n) {
         unsigned char* xr_i = ring + (size_t)(i % W) * tile_bytes;
+        unsigned char* const ystage = xr_i;  // smoother: until x_i takes its place
+        unsigned char* const zstage = MODE == MODE_SMOOTH ? xr_i : sm + lay.zstage;
         const int buf = (int)(n & 1);
         const uint32_t bphase = (uint32_t)((n >> 1) & 1);
         const uint32_t t_b = t_buf + 64 * buf;

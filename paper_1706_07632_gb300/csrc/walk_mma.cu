@@ -14,10 +14,14 @@ constexpr size_t kMmaSmemMax = 227 * 1024;
 template <typename T, int TC, int MODE>
 int mma_launch_t(cudaStream_t st, WalkBatch<T, float>& B, std::string* err) {
   auto kern = hmma_kernel<T, TC, MODE>;
-  // the deepest chunk ring that fits beside the x tiles and the z pool
+  // A short chunk ring leaves the SM's memory to the L1 cache, whose lines the neighbour loads in flight
+  // hold: with 2 slots for tile 32 a 255^2 x 1024 FP32 solve takes 117.8 ms (3 slots 119.1, 4 120.1, 8 121.5),
+  // with 3 for tile 16, whose chunks are used up twice as fast, a batch of 16 solves of up to 1023 columns x
+  // M = 1024 takes 73.1 ms (2 slots 74.0, 4 73.5, 8 73.8)
+  constexpr int kSlots = TC == 32 ? 2 : 3;
   const size_t other = mma_smem(TC, B.pool, B.W, B.slot_bytes, 0).total + 64;
   int ns = other < kMmaSmemMax ? (int)((kMmaSmemMax - other) / (size_t)B.slot_bytes) : 0;
-  ns = std::min(ns, 8);
+  ns = std::min(ns, kSlots);
   if (ns < 2) {
     *err = "tensor-core walk: no room for two chunk slots in shared memory";
     return 2;
@@ -35,8 +39,7 @@ int mma_launch_t(cudaStream_t st, WalkBatch<T, float>& B, std::string* err) {
   }
   if (B.ntiles <= 0) return 0;
   const long long grid = std::min<long long>(B.ntiles, (long long)device_sms() * occ);
-  kern<<<(unsigned)grid, kMmaBlock, smem, st>>>(B);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_sized(kern, grid, kMmaBlock, smem, occ, st, B);
   if (e != cudaSuccess) {
     *err = std::string("tensor-core walk launch: ") + cudaGetErrorString(e);
     return 1;

@@ -11,23 +11,33 @@ namespace {
 
 constexpr size_t kUmmaSmemMax = 227 * 1024;
 constexpr size_t kUmmaTwoPerSM = 112 * 1024;  // two CTAs share an SM's 228 KB (1 KB reserved each)
+// ... and in the 196 KB configuration, which leaves 60 KB of L1 instead of 28.  Loads in flight hold L1
+// lines, and their number bounded the memory warps: with two chunk slots in the small size instead of three
+// in the large one the finest half-sweep of a 1023^2 x 512 grid takes 1.04 ms instead of 1.44, the product of
+// 100,003 columns x M = 512 151 us instead of 174.
+constexpr size_t kUmmaTwoSmall = 97 * 1024;
 
 template <int MODE>
 int umma_launch_t(cudaStream_t st, WalkBatch<float, uint16_t>& B, std::string* err) {
   auto kern = humma_kernel<MODE>;
-  // two CTAs per SM (their chunk rings and tensor-memory round trips interleave) when at least three
-  // slots fit beside the operand tiles, else one CTA with the deepest ring that fits
-  const size_t other = umma_smem(B.pool, B.W, B.slot_bytes, 0).total + 128;
-  int ns = other < kUmmaTwoPerSM ? (int)((kUmmaTwoPerSM - other) / (size_t)B.slot_bytes) : 0;
-  const bool two = ns >= 3;
-  if (!two) ns = other < kUmmaSmemMax ? (int)((kUmmaSmemMax - other) / (size_t)B.slot_bytes) : 0;
+  // two CTAs per SM (their chunk rings and tensor-memory round trips interleave) with at least two slots
+  // in the smaller configuration or three in the larger, else one CTA with the deepest ring that fits
+  const size_t other = umma_smem(B.pool, B.W, B.slot_bytes, 0, MODE == MODE_SMOOTH).total + 128;
+  auto slots = [&](size_t limit) { return other < limit ? (int)((limit - other) / (size_t)B.slot_bytes) : 0; };
+  int ns = slots(kUmmaTwoSmall);
+  bool two = ns >= 2;
+  if (!two) {
+    ns = slots(kUmmaTwoPerSM);
+    two = ns >= 3;
+  }
+  if (!two) ns = slots(kUmmaSmemMax);
   ns = std::min(ns, 12);
   if (ns < 2) {
     *err = "tcgen05 walk: no room for two chunk slots in shared memory";
     return 2;
   }
   B.ns = ns;
-  const size_t smem = umma_smem(B.pool, B.W, B.slot_bytes, ns).total;
+  const size_t smem = umma_smem(B.pool, B.W, B.slot_bytes, ns, MODE == MODE_SMOOTH).total;
   static KernelCache cache;
   int occ = 1;
   {
@@ -44,8 +54,7 @@ int umma_launch_t(cudaStream_t st, WalkBatch<float, uint16_t>& B, std::string* e
   const long long per_sm = two ? 2 : 1;
   (void)occ;
   const long long grid = std::min<long long>(B.ntiles, (long long)device_sms() * per_sm);
-  kern<<<(unsigned)grid, kUmmaBlock, smem, st>>>(B);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_sized(kern, grid, kUmmaBlock, smem, two ? 2 : 1, st, B);
   if (e != cudaSuccess) {
     *err = std::string("tcgen05 walk launch: ") + cudaGetErrorString(e);
     return 1;
