@@ -19,6 +19,7 @@
 #include "walk.h"
 
 using fhmg::Geo;
+using fhmg::TransferJob;
 
 namespace {
 
@@ -214,10 +215,6 @@ void dense_of(const fhmg::HostH& h, std::vector<double>& R) {
 
 // Launch shapes of the grid-function kernels (kernels.cuh): points along x, rows along y, time
 // levels strided along z.
-dim3 coarse_grid(int dim, int Nf, int M) {
-  const int Nc = (Nf - 1) / 2;
-  return fhmg::plane_grid(Nc, dim == 1 ? 1 : Nc, M, fhmg::device_sms());
-}
 dim3 fine_grid(int dim, int N, int M) { return fhmg::plane_grid(N, dim == 1 ? 1 : N, M, fhmg::device_sms()); }
 // ... a thread per pair of points of a row (2D)
 dim3 pair_grid(int N, int M) { return fhmg::plane_grid((N + 1) / 2, N, M, fhmg::device_sms()); }
@@ -436,6 +433,32 @@ int sweep(fhmg_problem p, int l, T* u, const T* F, int kind) {
   return FHMG_OK;
 }
 
+// Transfers of up to NJ instances in one launch
+template <typename T>
+TransferJob<T> restrict_job(fhmg_problem p, int l, const T* u, const T* F, T* xs, T* rc, T* zero) {
+  return TransferJob<T>{F, const_cast<T*>(u), xs, rc, zero, p->lev[l].inv_h2, 0, p->dim, p->lev[l].N, p->M, 0, 0, 0, 0};
+}
+template <typename T>
+TransferJob<T> prolong_job(fhmg_problem p, int l, const T* e, T* u) {
+  return TransferJob<T>{nullptr, u, nullptr, nullptr, const_cast<T*>(e), 0.0, 0, p->dim, p->lev[l].N, p->M, 0, 0, 0, 0};
+}
+template <typename T, int NJ>
+int launch_transfer(cudaStream_t st, const std::vector<TransferJob<T>>& jobs, bool restriction, long long* nl = nullptr) {
+  for (size_t at = 0; at < jobs.size(); at += NJ) {
+    fhmg::TransferBatch<T, NJ> B;
+    B.n = (int)std::min<size_t>(NJ, jobs.size() - at);
+    std::copy(jobs.begin() + at, jobs.begin() + at + B.n, B.job);
+    const long long blocks = fhmg::transfer_shape(B.job, B.n, restriction, fhmg::device_sms());
+    if (restriction)
+      fhmg::restrict_pre_kernel<T, NJ><<<(unsigned)blocks, 256, 0, st>>>(B);
+    else
+      fhmg::prolong_add_kernel<T, NJ><<<(unsigned)blocks, 256, 0, st>>>(B);
+    CK(cudaGetLastError());
+    if (nl) ++*nl;
+  }
+  return FHMG_OK;
+}
+
 // rc = FW(F - A_h u) - R~ FW(u) on level l-1
 template <typename T>
 int restrict_defect(fhmg_problem p, int l, const T* u, const T* F, T* rc, int kind) {
@@ -446,8 +469,7 @@ int restrict_defect(fhmg_problem p, int l, const T* u, const T* F, T* rc, int ki
     fhmg::restrict_pre_split_kernel<T><<<fhmg::split_grid(lc.N, lc.N, p->M, fhmg::device_sms()), fhmg::split_block(), 0,
                                          p->st>>>(lv.N, lv.inv_h2, p->M, u, F, xs, rc);
   else
-    fhmg::restrict_pre_kernel<T><<<coarse_grid(p->dim, lv.N, p->M), 256, 0, p->st>>>(p->dim, lv.N, lv.inv_h2, p->M, u, F,
-                                                                                    xs, rc);
+    TRY((launch_transfer<T, 1>(p->st, {restrict_job<T>(p, l, u, F, xs, rc, nullptr)}, true)));
   ++p->launches;
   CK(cudaGetLastError());
   return walk_matvec<T>(p, kind, lc.npts, xs, rc, rc, nullptr);
@@ -459,7 +481,7 @@ int prolong_add(fhmg_problem p, int l, const T* e, T* u) {
     fhmg::prolong_add_split_kernel<T><<<fhmg::split_grid((p->lev[l].N + 1) / 2, p->lev[l].N, p->M, fhmg::device_sms()),
                                         fhmg::split_block(), 0, p->st>>>(p->lev[l].N, p->M, e, u);
   else
-    fhmg::prolong_add_kernel<T><<<fine_grid(p->dim, p->lev[l].N, p->M), 256, 0, p->st>>>(p->dim, p->lev[l].N, p->M, e, u);
+    TRY((launch_transfer<T, 1>(p->st, {prolong_job<T>(p, l, e, u)}, false)));
   ++p->launches;
   CK(cudaGetLastError());
   return FHMG_OK;
@@ -909,27 +931,19 @@ int batched_vcycle(cudaStream_t st, std::vector<BLev> cur, int nu1, int nu2, int
   TRY(batched_sweeps(st, rest, nu1, kind, nl));
   std::vector<fhmg::WalkArgsT<double>> jobs;
   std::vector<BLev> next;
+  std::vector<TransferJob<double>> transfers;
   for (auto& b : rest) {
-    LevelData& lv = b.p->lev[b.l];
     LevelData& lc = b.p->lev[b.l - 1];
-    const long long n = lc.npts * b.p->M;
-    fhmg::restrict_pre_kernel<double><<<coarse_grid(b.p->dim, lv.N, b.p->M), 256, 0, st>>>(b.p->dim, lv.N, lv.inv_h2,
-                                                                                         b.p->M, b.u, b.F, b.p->Xs, lc.RC);
-    CK(cudaGetLastError());
-    ++*nl;
+    transfers.push_back(restrict_job<double>(b.p, b.l, b.u, b.F, b.p->Xs, lc.RC, lc.E));  // and lc.E = 0
     jobs.push_back(matvec_job<double>(b.p, kind, lc.npts, b.p->Xs, lc.RC, lc.RC, nullptr));
-    CK(cudaMemsetAsync(lc.E, 0, sizeof(double) * n, st));
     next.push_back(BLev{b.p, b.l - 1, lc.E, lc.RC});
   }
+  TRY((launch_transfer<double, fhmg::kMaxJobs>(st, transfers, true, nl)));
   TRY(launch_jobs(st, kind, jobs, nl));
   TRY(batched_vcycle(st, next, nu1, nu2, kind, nl));
-  for (auto& b : rest) {
-    LevelData& lc = b.p->lev[b.l - 1];
-    fhmg::prolong_add_kernel<double><<<fine_grid(b.p->dim, b.p->lev[b.l].N, b.p->M), 256, 0, st>>>(
-        b.p->dim, b.p->lev[b.l].N, b.p->M, lc.E, b.u);
-    CK(cudaGetLastError());
-    ++*nl;
-  }
+  transfers.clear();
+  for (auto& b : rest) transfers.push_back(prolong_job<double>(b.p, b.l, b.p->lev[b.l - 1].E, b.u));
+  TRY((launch_transfer<double, fhmg::kMaxJobs>(st, transfers, false, nl)));
   return batched_sweeps(st, rest, nu2, kind, nl);
 }
 

@@ -7,6 +7,7 @@
 // geometry helpers and the stencil / transfer kernels around it.
 #pragma once
 #include <cstdint>
+#include <algorithm>
 #include <cuda_runtime.h>
 
 namespace fhmg {
@@ -100,37 +101,132 @@ __host__ __device__ inline NbrOffsets nbr_offsets(const Geo& g) {
 // blockIdx.y is the row (y; 0 in 1D), blockIdx.z strides over the time levels, so no index is
 // recovered by a division.
 
+// Transfers between a level (fine) and the one below it, for up to NJ instances in one launch (a
+// batched cycle has an instance's grids at every depth: one launch for each took a third of the launches of
+// a batch of 16 and, with the gaps between them, 14 of its 74 ms: 73.7 -> 66.2 ms).  Block b works on the instance whose
+// range of blocks holds it.  Within an instance 2^lx threads run along a grid row (x) and 256 / 2^lx
+// along the time levels, so that short rows fill their blocks too.
+template <typename T>
+struct TransferJob {
+  const T* F;   // restriction: right-hand side
+  T* U;         // fine grid function (restriction: read; prolongation: corrected)
+  T* Xc;        // restriction: FW(u)
+  T* Bc;        // restriction: FW(F - A_h u)
+  T* E;         // prolongation: the correction; restriction: its start, set to zero (null: left alone)
+  double inv_h2;
+  long long first;  // first block
+  int dim, Nf, M, lx, bx, by, bz;
+};
+template <typename T, int NJ>
+struct TransferBatch {
+  TransferJob<T> job[NJ];
+  int n;
+};
+
+// Launch shape for n instances (restriction: a thread per coarse point, else per fine point): returns the
+// number of blocks, about 16 per SM over all of them, each with an equal share of the time levels' work.
+// A block takes as many time levels side by side as short rows leave threads for, unless that leaves
+// SMs without a block (the FP64 pipe, 2 lanes per clock and SM, is what the work must be spread over).
+template <typename T>
+inline long long transfer_shape(TransferJob<T>* jobs, int n, bool restriction, int sms) {
+  long long units = 0;  // blocks of one step each
+  auto rows = [&](const TransferJob<T>& j) { return restriction ? (j.Nf - 1) / 2 : j.Nf; };
+  auto steps = [](const TransferJob<T>& j) { return (j.M + (256 >> j.lx) - 1) / (256 >> j.lx); };
+  for (int k = 0; k < n; ++k) {
+    TransferJob<T>& j = jobs[k];
+    const int nx = rows(j);
+    j.by = j.dim == 1 ? 1 : nx;
+    for (j.lx = 0;; ++j.lx) {
+      j.bx = (nx + (1 << j.lx) - 1) >> j.lx;
+      if (j.lx == 8 || (j.bx == 1 && (long long)j.by * steps(j) * n >= 4LL * sms)) break;
+    }
+    units += (long long)j.bx * j.by * steps(j);
+  }
+  const long long per = std::max<long long>(1, (units + 16LL * sms - 1) / (16LL * sms));
+  long long blocks = 0;
+  for (int k = 0; k < n; ++k) {
+    TransferJob<T>& j = jobs[k];
+    j.first = blocks;
+    j.bz = (int)((steps(j) + per - 1) / per);
+    blocks += (long long)j.bx * j.by * j.bz;
+  }
+  return blocks;
+}
+
+struct TransferPlace {
+  int x, y, m0, dm;  // point, first time level of this thread and the step to its next one
+};
+template <typename T, int NJ>
+__device__ __forceinline__ const TransferJob<T>& transfer_place(const TransferBatch<T, NJ>& B, TransferPlace& q) {
+  int k = 0;
+  if (NJ > 1)
+    while (k + 1 < B.n && B.job[k + 1].first <= (long long)blockIdx.x) ++k;
+  const TransferJob<T>& J = B.job[k];
+  const unsigned b = (unsigned)((long long)blockIdx.x - J.first);
+  const unsigned row = b / (unsigned)J.bx;
+  q.x = (int)((b - row * (unsigned)J.bx) << J.lx) + (int)(threadIdx.x & ((1u << J.lx) - 1));
+  const unsigned z = row / (unsigned)J.by;
+  q.y = (int)(row - z * (unsigned)J.by);
+  const int tm = 256 >> J.lx;
+  q.m0 = (int)z * tm + (int)(threadIdx.x >> J.lx);
+  q.dm = J.bz * tm;
+  return J;
+}
+
 // Restriction of the defect with the time operator commuted out:
 //   Xc = FW(u)  and  Bc = FW(F - A_h u), so that the coarse right-hand side is Bc - R~ Xc
 // (FW acts per time level and R~ per spatial point, so FW(R~ u) = R~ FW(u)).  One thread per
-// coarse point (cx, cy) per time level.
-template <typename T>
-__global__ void restrict_pre_kernel(int dim, int Nf, double inv_h2, int M, const T* __restrict__ U,
-                                    const T* __restrict__ F, T* __restrict__ Xc, T* __restrict__ Bc) {
+// coarse point (cx, cy) per time level.  In FP64 the FP64 pipe bounds it (15 operations
+// per point in 1D: 4095 points x M = 4096 take 0.29 ms, of which the pipe needs 0.22), else memory.  A
+// missing neighbour reads the next point instead and counts as zero, so that no load sits behind a branch.
+template <typename T, int NJ>
+__global__ void __launch_bounds__(256) restrict_pre_kernel(const __grid_constant__ TransferBatch<T, NJ> B) {
+  TransferPlace q;
+  const TransferJob<T>& J = transfer_place(B, q);
+  const int Nf = J.Nf, M = J.M;
   const int Nc = (Nf - 1) / 2;
-  const int cx = blockIdx.x * blockDim.x + threadIdx.x, cy = blockIdx.y;
+  const int cx = q.x, cy = q.y;
   if (cx >= Nc) return;
-  const long long nc = dim == 1 ? Nc : (long long)Nc * Nc;
-  const long long nf = dim == 1 ? Nf : (long long)Nf * Nf;
-  const T ih2 = (T)inv_h2;
-  for (int m = blockIdx.z; m < M; m += gridDim.z) {
-    const T* u = U + (long long)m * nf;
-    const T* f = F + (long long)m * nf;
-    T xs = 0, bs = 0;
-    if (dim == 1) {
-      const int pc = 2 * cx + 1;
+  const T* __restrict__ U = J.U;
+  const T* __restrict__ F = J.F;
+  T* __restrict__ Xc = J.Xc;
+  T* __restrict__ Bc = J.Bc;
+  T* __restrict__ E = J.E;
+  const T ih2 = (T)J.inv_h2;
+  if (J.dim == 1) {
+    const bool l = cx > 0, r = 2 * cx + 2 < Nf - 1;  // the outer neighbours exist
+    for (int m = q.m0; m < M; m += q.dm) {
+      const long long pc = (long long)m * Nf + 2 * cx + 1;
+      T u[5], f[3];
 #pragma unroll
-      for (int o = -1; o <= 1; ++o) {
-        const int pp = pc + o;
-        const T w = o == 0 ? (T)0.5 : (T)0.25;
-        const T uc = u[pp];
-        const T ul = pp > 0 ? u[pp - 1] : (T)0;
-        const T ur = pp < Nf - 1 ? u[pp + 1] : (T)0;
-        xs += w * uc;
-        bs += w * (f[pp] - (2 * uc - ul - ur) * ih2);
+      for (int o = 0; o < 3; ++o) {
+        u[o + 1] = U[pc + o - 1];
+        f[o] = F[pc + o - 1];
       }
-    } else {
-      const int py = 2 * cy + 1, px = 2 * cx + 1;
+      u[0] = U[pc - (l ? 2 : 1)];
+      u[4] = U[pc + (r ? 2 : 1)];
+      if (!l) u[0] = 0;
+      if (!r) u[4] = 0;
+      T xs = 0, bs = 0;
+#pragma unroll
+      for (int o = 0; o < 3; ++o) {
+        const T w = o == 1 ? (T)0.5 : (T)0.25;
+        const T uc = u[o + 1], ul = u[o], ur = u[o + 2];
+        xs += w * uc;
+        bs += w * (f[o] - (2 * uc - ul - ur) * ih2);
+      }
+      const long long c = (long long)m * Nc + cx;
+      Xc[c] = xs;
+      Bc[c] = bs;
+      if (E) E[c] = 0;
+    }
+  } else {
+    const long long nc = (long long)Nc * Nc, nf = (long long)Nf * Nf;
+    const int py = 2 * cy + 1, px = 2 * cx + 1;
+    for (int m = q.m0; m < M; m += q.dm) {
+      const T* u = U + (long long)m * nf;
+      const T* f = F + (long long)m * nf;
+      T xs = 0, bs = 0;
 #pragma unroll
       for (int oy = -1; oy <= 1; ++oy)
 #pragma unroll
@@ -140,17 +236,20 @@ __global__ void restrict_pre_kernel(int dim, int Nf, double inv_h2, int M, const
           const long long pp = (long long)yy * Nf + xx;
           const T uc = u[pp];
           T s = 0;
-          if (xx > 0) s += u[pp - 1];
-          if (xx < Nf - 1) s += u[pp + 1];
-          if (yy > 0) s += u[pp - Nf];
-          if (yy < Nf - 1) s += u[pp + Nf];
+          const T a0 = u[pp - (xx > 0 ? 1 : 0)], a1 = u[pp + (xx < Nf - 1 ? 1 : 0)];
+          const T a2 = u[pp - (yy > 0 ? Nf : 0)], a3 = u[pp + (yy < Nf - 1 ? Nf : 0)];
+          s += xx > 0 ? a0 : (T)0;
+          s += xx < Nf - 1 ? a1 : (T)0;
+          s += yy > 0 ? a2 : (T)0;
+          s += yy < Nf - 1 ? a3 : (T)0;
           xs += w * uc;
           bs += w * (f[pp] - (4 * uc - s) * ih2);
         }
+      const long long c = (long long)m * nc + (long long)cy * Nc + cx;
+      Xc[c] = xs;
+      Bc[c] = bs;
+      if (E) E[c] = 0;
     }
-    const long long c = (long long)cy * Nc + cx;
-    Xc[(long long)m * nc + c] = xs;
-    Bc[(long long)m * nc + c] = bs;
   }
 }
 
@@ -168,29 +267,37 @@ __device__ __forceinline__ void lin_weights(int x, int Nc, int& c0, T& w0, int& 
 }
 
 // u_f += P e_c, linear (1D) / bilinear (2D) interpolation in space, per time level; one thread per
-// fine point.
-template <typename T>
-__global__ void prolong_add_kernel(int dim, int Nf, int M, const T* __restrict__ E, T* __restrict__ U) {
+// fine point (1D, 4095 points x M = 4096, FP64: 0.10 ms, of which the FP64 pipe needs 0.09).
+template <typename T, int NJ>
+__global__ void __launch_bounds__(256) prolong_add_kernel(const __grid_constant__ TransferBatch<T, NJ> B) {
+  TransferPlace q;
+  const TransferJob<T>& J = transfer_place(B, q);
+  const int Nf = J.Nf, M = J.M;
   const int Nc = (Nf - 1) / 2;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+  const int x = q.x, y = q.y;
   if (x >= Nf) return;
-  const long long nf = dim == 1 ? Nf : (long long)Nf * Nf;
-  const long long nc = dim == 1 ? Nc : (long long)Nc * Nc;
-  int ax0, ax1, ay0 = 0, ay1 = 0;
-  T wx0, wx1, wy0 = 1, wy1 = 0;
+  const T* __restrict__ E = J.E;
+  T* __restrict__ U = J.U;
+  int ax0, ax1;
+  T wx0, wx1;
   lin_weights<T>(x, Nc, ax0, wx0, ax1, wx1);
-  if (dim == 2) lin_weights<T>(y, Nc, ay0, wy0, ay1, wy1);
-  const long long pp = (long long)y * Nf + x;
-  for (int m = blockIdx.z; m < M; m += gridDim.z) {
-    const T* e = E + (long long)m * nc;
-    T v;
-    if (dim == 1) {
-      v = wx0 * e[ax0] + wx1 * e[ax1];
-    } else {
-      v = wy0 * (wx0 * e[(long long)ay0 * Nc + ax0] + wx1 * e[(long long)ay0 * Nc + ax1]) +
-          wy1 * (wx0 * e[(long long)ay1 * Nc + ax0] + wx1 * e[(long long)ay1 * Nc + ax1]);
+  if (J.dim == 1) {
+    for (int m = q.m0; m < M; m += q.dm) {
+      const T* e = E + (long long)m * Nc;
+      U[(long long)m * Nf + x] += wx0 * e[ax0] + wx1 * e[ax1];
     }
-    U[(long long)m * nf + pp] += v;
+  } else {
+    const long long nc = (long long)Nc * Nc, nf = (long long)Nf * Nf;
+    int ay0, ay1;
+    T wy0, wy1;
+    lin_weights<T>(y, Nc, ay0, wy0, ay1, wy1);
+    const long long pp = (long long)y * Nf + x;
+    for (int m = q.m0; m < M; m += q.dm) {
+      const T* e = E + (long long)m * nc;
+      const T v = wy0 * (wx0 * e[(long long)ay0 * Nc + ax0] + wx1 * e[(long long)ay0 * Nc + ax1]) +
+                  wy1 * (wx0 * e[(long long)ay1 * Nc + ax0] + wx1 * e[(long long)ay1 * Nc + ax1]);
+      U[(long long)m * nf + pp] += v;
+    }
   }
 }
 
