@@ -8,7 +8,7 @@
 // run as mma.sync m16n8k8 TF32 with FP32 accumulation, each product split in three,
 // hi*hi + hi*lo + lo*hi (hi = tf32(a), lo = tf32(a - hi)), which keeps FP32 accuracy; each term
 // has its own accumulator.  The matrices arrive pre-split in the fragment layout of
-// build_panel_mma; x tiles are split once when written (tiles of <= 16 columns) or on load.
+// build_panel_mma; x tiles are split once when written, or on every load where the pairs do not fit.
 //
 // Warps: 8 consumer warps, warp w owns row tile rt = w % 4 (16 rows of the leaf) and column half
 // w / 4 (TC / 2 columns = TC / 16 n-tiles of 8).  Lane (g, t) = (lane / 4, lane % 4) holds the
@@ -28,13 +28,13 @@ constexpr int kMmaLP = 80;  // padded x-tile column (floats): 8 columns x 4 lane
 struct MmaSmem {
   size_t ysm, ring, zp, bar, ebar, cbar, desc, flag, total;
 };
-// x tiles (y of the current leaf, the ring of recent x) of tiles up to 16 columns are kept as TF32
-// hi/lo pairs ([hi: TC x LP][lo: TC x LP] per tile), split once when written; wider tiles keep
-// one float per entry and split on every load (their shared memory would not hold the pairs).
-__host__ __device__ inline int mma_xsplit(int TC) { return TC <= 16 ? 2 : 1; }
-__host__ __device__ inline MmaSmem mma_smem(int TC, int pool, int W, int slot_bytes, int ns) {
+// x tiles (y of the current leaf, the ring of recent x) are kept as TF32 hi/lo pairs (XS = 2: [hi: TC x LP]
+// [lo: TC x LP] per tile), split once when written, where shared memory holds them beside two chunk slots;
+// else (tile 32 with a wide near field) as one float per entry, split on every load (XS = 1): 905 vs
+// 830 us per half-sweep of 255^2 points x M = 1024.
+__host__ __device__ inline MmaSmem mma_smem(int TC, int xs, int pool, int W, int slot_bytes, int ns) {
   auto a16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
-  const size_t tile = (size_t)mma_xsplit(TC) * TC * kMmaLP * 4;
+  const size_t tile = (size_t)xs * TC * kMmaLP * 4;
   MmaSmem s;
   s.ysm = a16((size_t)ns * slot_bytes);
   s.ring = a16(s.ysm + tile);
@@ -106,13 +106,13 @@ __device__ __forceinline__ void load_a(const float4* A, int rt, int kb, int nkb,
   l1 = p[96];
 }
 
-template <typename T, int TC, int MODE>
+template <typename T, int TC, int MODE, int XS>
 __global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkBatch<T, float> B) {
   constexpr int L = 64, NT = 256, NTL = TC / 16;  // n-tiles of 8 columns per warp
   constexpr int LP = kMmaLP;
   static_assert(TC == 16 || TC == 32, "tensor-core tile");
   extern __shared__ __align__(16) unsigned char sm[];
-  const MmaSmem lay = mma_smem(TC, B.pool, B.W, B.slot_bytes, B.ns);
+  const MmaSmem lay = mma_smem(TC, XS, B.pool, B.W, B.slot_bytes, B.ns);
   unsigned char* slots = sm;
   float* ysm = reinterpret_cast<float*>(sm + lay.ysm);
   float* ring = reinterpret_cast<float*>(sm + lay.ring);
@@ -186,7 +186,6 @@ __global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkB
   const int rt = w & 3;                 // row tile
   const int cb = (w >> 2) * (TC / 2);   // first column of this warp
   const int g = lane >> 2, tq = lane & 3;
-  constexpr int XS = TC <= 16 ? 2 : 1;        // mma_xsplit(TC)
   constexpr int TS = XS * TC * LP;            // floats per x tile
   // B operand of column col, k-block kb from an x tile (pre-split, or split here)
   auto load_b = [&](const float* tile, int col, int kb, uint32_t(&bh)[4], uint32_t(&bl)[4]) {
