@@ -23,26 +23,40 @@
 
 namespace fhmg {
 
+constexpr int kMmaL = 64;
 constexpr int kMmaLP = 80;  // padded x-tile column (floats): 8 columns x 4 lanes of 16-byte reads hit distinct banks
 
+// Memory warps of the smoother (MEM): they load the right-hand sides and neighbours a leaf ahead, column by
+// column of the tile (in the products' lane layout a load covers 8 rows x 2 columns), so that the products
+// never wait for them and their threads hold no load state.  Tile 32 takes three warps, which with the
+// eight consumer warps and the producer leave each thread 168 registers (with four: 128, and the products
+// spill).  Half-sweep of 255^2 points x M = 1024 at tile 32: 830 -> 694 us (four warps 795); of 4095
+// points x M = 4096 in FP64 at tile 16: 511 -> 403 us.
+__host__ __device__ constexpr int mma_mem(int TC) { return TC == 32 ? 96 : 128; }
+constexpr int kMmaRhsPad = 8;  // columns of padding of a right-hand-side row: the rows a warp reads hit distinct banks
+__host__ __device__ constexpr int mma_threads(int TC, bool mem) { return 256 + (mem ? mma_mem(TC) : 0) + 32; }
+
 struct MmaSmem {
-  size_t ysm, ring, zp, bar, ebar, cbar, desc, flag, total;
+  size_t ysm, ring, zp, rhs, bar, ebar, cbar, rbar, desc, flag, total;
 };
+// The memory warps' right-hand sides have a double buffer (rhs_bytes: size of T, 0 without them).
 // x tiles (y of the current leaf, the ring of recent x) are kept as TF32 hi/lo pairs (XS = 2: [hi: TC x LP]
 // [lo: TC x LP] per tile), split once when written, where shared memory holds them beside two chunk slots;
 // else (tile 32 with a wide near field) as one float per entry, split on every load (XS = 1): 905 vs
 // 830 us per half-sweep of 255^2 points x M = 1024.
-__host__ __device__ inline MmaSmem mma_smem(int TC, int xs, int pool, int W, int slot_bytes, int ns) {
+__host__ __device__ inline MmaSmem mma_smem(int TC, int xs, int pool, int W, int slot_bytes, int ns, int rhs_bytes) {
   auto a16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
   const size_t tile = (size_t)xs * TC * kMmaLP * 4;
   MmaSmem s;
   s.ysm = a16((size_t)ns * slot_bytes);
   s.ring = a16(s.ysm + tile);
   s.zp = a16(s.ring + (size_t)W * tile);
-  s.bar = a16(s.zp + (size_t)pool * TC * 4);
+  s.rhs = a16(s.zp + (size_t)pool * TC * 4);
+  s.bar = s.rhs + 2 * (size_t)kMmaL * (TC + kMmaRhsPad) * rhs_bytes;
   s.ebar = s.bar + 8 * (size_t)ns;
   s.cbar = s.ebar + 8 * (size_t)ns;
-  s.desc = a16(s.cbar + 8);
+  s.rbar = s.cbar + 8;
+  s.desc = a16(s.rbar + 4 * 8);
   s.flag = s.desc + 16 * (size_t)ns;
   s.total = a16(s.flag + 16);
   return s;
@@ -106,13 +120,13 @@ __device__ __forceinline__ void load_a(const float4* A, int rt, int kb, int nkb,
   l1 = p[96];
 }
 
-template <typename T, int TC, int MODE, int XS>
-__global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkBatch<T, float> B) {
+template <typename T, int TC, int MODE, int XS, bool MEM>
+__global__ void __launch_bounds__(mma_threads(TC, MEM)) hmma_kernel(const __grid_constant__ WalkBatch<T, float> B) {
   constexpr int L = 64, NT = 256, NTL = TC / 16;  // n-tiles of 8 columns per warp
   constexpr int LP = kMmaLP;
   static_assert(TC == 16 || TC == 32, "tensor-core tile");
   extern __shared__ __align__(16) unsigned char sm[];
-  const MmaSmem lay = mma_smem(TC, XS, B.pool, B.W, B.slot_bytes, B.ns);
+  const MmaSmem lay = mma_smem(TC, XS, B.pool, B.W, B.slot_bytes, B.ns, MEM ? sizeof(T) : 0);
   unsigned char* slots = sm;
   float* ysm = reinterpret_cast<float*>(sm + lay.ysm);
   float* ring = reinterpret_cast<float*>(sm + lay.ring);
@@ -120,6 +134,10 @@ __global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkB
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + lay.bar);
   uint64_t* empty = reinterpret_cast<uint64_t*>(sm + lay.ebar);
   uint64_t* cbar = reinterpret_cast<uint64_t*>(sm + lay.cbar);
+  constexpr int MT = mma_mem(TC), RL = TC + kMmaRhsPad;
+  T* rbuf = reinterpret_cast<T*>(sm + lay.rhs);                   // [2][L][RL]
+  uint64_t* filled = reinterpret_cast<uint64_t*>(sm + lay.rbar);  // [2] a buffer holds a leaf's right-hand sides
+  uint64_t* taken = filled + 2;                                   // [2] ... has been read
   int4* sdesc = reinterpret_cast<int4*>(sm + lay.desc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + lay.flag);
 
@@ -134,14 +152,105 @@ __global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkB
       mbar_init(empty + s, NT / 32);
     }
     mbar_init(cbar, NT / 32);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(filled + b, MT / 32);
+      mbar_init(taken + b, NT / 32);
+    }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
 
+  if (MEM && t >= NT && t < NT + MT) {
+    // ---- memory warps: right-hand sides b + (sum of the neighbours) / h^2, a leaf ahead of the products ----
+    const int mt = t - NT;
+    const int col = mt % TC, r0 = mt / TC;
+    constexpr int RS = MT / TC, BATCH = TC == 32 ? 11 : 8;  // row step, rows in flight
+    long long n = 0;
+    for (long long gt = blockIdx.x; gt < B.ntiles; gt += gridDim.x) {
+      const WalkJob<T, float>& J = B.job[job_of(B, gt)];
+      const long long ld = J.geo.ld;
+      const T inv_h2 = (T)J.geo.inv_h2;
+      const long long cg = (gt - J.tile0) * TC + col;
+      const bool valid = cg < J.ncols;
+      // missing neighbours and columns past the panel's end read an element that exists and count as zeros,
+      // so that no load sits behind a branch
+      long long p = valid ? cg : 0;
+      int o[4] = {0, 0, 0, 0};
+      bool have[4] = {false, false, false, false};
+      if (valid && J.geo.dim > 0) {
+        int iy, ix;
+        p = colour_pos(J.geo.dim, J.geo.N, J.geo.colour, cg, &iy, &ix);
+        have[0] = ix > 0;
+        have[1] = ix < J.geo.N - 1;
+        have[2] = J.geo.dim == 2 && iy > 0;
+        have[3] = J.geo.dim == 2 && iy < J.geo.N - 1;
+        if (sizeof(T) == 4) {  // FP32 grid functions may be stored by colour
+          const NbrOffsets off = nbr_offsets(J.geo);
+          if (J.geo.split) p = cg + (J.geo.colour ? colour_count(2, J.geo.N, 0) : 0);
+          const bool odd = iy & 1;
+          o[0] = odd ? off.left[1] : off.left[0];
+          o[1] = o[0] + off.step;
+          o[2] = odd ? off.up[1] : off.up[0];
+          o[3] = odd ? off.down[1] : off.down[0];
+        } else {
+          o[0] = -1, o[1] = 1, o[2] = -J.geo.N, o[3] = J.geo.N;
+        }
+#pragma unroll
+        for (int d = 0; d < 4; ++d)
+          if (!have[d]) o[d] = 0;
+      }
+      const int dim = J.geo.dim;
+      const T* const Bp = J.B + p;
+      const T* const Xp = J.X + p;
+      const int nb = J.P.nb;
+      for (int i = 0; i < nb; ++i, ++n) {
+        const int buf = (int)(n & 1);
+        if (n >= 2 && !__all_sync(0xffffffffu, mbar_wait_or_abort(taken + buf, (uint32_t)(((n >> 1) - 1) & 1),
+                                                                  abort_flag, B.spin))) {
+          if (lane == 0 && !*abort_flag) {
+            *abort_flag = 1;
+            atomicExch(B.err, 1);
+          }
+          return;
+        }
+        T* const rb = rbuf + (size_t)buf * L * RL;
+#pragma unroll 1
+        for (int r = r0; r < L; r += RS * BATCH) {
+          T v[BATCH], u[BATCH][4];
+#pragma unroll
+          for (int k = 0; k < BATCH; ++k) {
+            const long long at = (long long)(i * L + min(r + k * RS, L - 1)) * ld;
+            v[k] = Bp[at];
+            if (dim > 0) {
+              u[k][0] = Xp[at + o[0]];
+              u[k][1] = Xp[at + o[1]];
+              if (dim == 2) {
+                u[k][2] = Xp[at + o[2]];
+                u[k][3] = Xp[at + o[3]];
+              }
+            }
+          }
+#pragma unroll
+          for (int k = 0; k < BATCH; ++k) {
+            T b = valid ? v[k] : (T)0;
+#pragma unroll
+            for (int d = 0; d < 4; ++d)
+              if (!have[d]) u[k][d] = 0;
+            const T s = ((u[k][0] + u[k][1]) + u[k][2]) + u[k][3];
+            b += s * inv_h2;
+            if (r + k * RS < L) rb[(r + k * RS) * RL + col] = b;
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(filled + buf);
+      }
+    }
+    return;
+  }
   if (t >= NT) {
     // ---- producer (as in hpanel_kernel; the level inverses hold hi/lo pairs: 2 L^2 floats) ----
-    if (t != NT) return;
+    if (t != NT + (MEM ? MT : 0)) return;
     long long k = 0;
     int slot = 0;
     bool ok = true, stop = false;
@@ -225,6 +334,7 @@ __global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkB
     return !give_up(ok);
   };
 
+  long long leaves = 0;  // walked so far
   int cslot = 0;
   uint32_t cphase = 0;
   for (long long gt = blockIdx.x; gt < B.ntiles; gt += gridDim.x) {
@@ -274,61 +384,63 @@ __global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkB
     // an element of their column 0 or their own and are replaced by zeros, so that no load sits behind a
     // branch: the loads of an n-tile are in flight together (with branches a leaf's loads took 7300 of
     // its 20100 cycles at tile 32).
-    constexpr bool RAW = MODE == MODE_SMOOTH && NTL == 1;
+    constexpr bool RAW = MODE == MODE_SMOOTH && !MEM && NTL == 1;
     T bn[NTL][4], xn[NTL][4], dn[2], un[RAW ? NTL : 1][4][4];
     auto load_rhs = [&](int leaf) {
       if (leaf >= nb) return;
 #pragma unroll
       for (int h = 0; h < 2; ++h) dn[h] = ddg[(long long)leaf * L + rt * 16 + g + 8 * h];
+      if constexpr (!MEM) {
 #pragma unroll
-      for (int nt = 0; nt < NTL; ++nt) {
-        T v[4], u[4][4];
+        for (int nt = 0; nt < NTL; ++nt) {
+          T v[4], u[4][4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int h = j >> 1, e = j & 1;
-          const long long base = (long long)(leaf * L + rt * 16 + g + 8 * h) * ld + (vcol[nt][e] ? pcol[nt][e] : 0);
-          v[j] = Bsrc[base];
-          if (MODE == MODE_SMOOTH) {
-            if (J.geo.dim > 0) {
+          for (int j = 0; j < 4; ++j) {
+            const int h = j >> 1, e = j & 1;
+            const long long base = (long long)(leaf * L + rt * 16 + g + 8 * h) * ld + (vcol[nt][e] ? pcol[nt][e] : 0);
+            v[j] = Bsrc[base];
+            if (MODE == MODE_SMOOTH) {
+              if (J.geo.dim > 0) {
 #pragma unroll
-              for (int d = 0; d < 4; ++d) {
-                const int o = !SPL ? (d == 0 ? -1 : d == 1 ? 1 : d == 2 ? -J.geo.N : J.geo.N)
-                              : d < 2 ? noff[nt][e][0] + (d ? off.step : 0)
-                                      : noff[nt][e][d - 1];
-                u[j][d] = X[base + ((nmask[nt][e] >> d) & 1 ? o : 0)];
+                for (int d = 0; d < 4; ++d) {
+                  const int o = !SPL ? (d == 0 ? -1 : d == 1 ? 1 : d == 2 ? -J.geo.N : J.geo.N)
+                                : d < 2 ? noff[nt][e][0] + (d ? off.step : 0)
+                                        : noff[nt][e][d - 1];
+                  u[j][d] = X[base + ((nmask[nt][e] >> d) & 1 ? o : 0)];
+                }
+              } else {
+#pragma unroll
+                for (int d = 0; d < 4; ++d) u[j][d] = 0;
               }
             } else {
-#pragma unroll
-              for (int d = 0; d < 4; ++d) u[j][d] = 0;
+              xn[nt][j] = X[base];
             }
-          } else {
-            xn[nt][j] = X[base];
           }
-        }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int e = j & 1;
-          T b = vcol[nt][e] ? v[j] : (T)0;
-          if (MODE == MODE_SMOOTH) {
+          for (int j = 0; j < 4; ++j) {
+            const int e = j & 1;
+            T b = vcol[nt][e] ? v[j] : (T)0;
+            if (MODE == MODE_SMOOTH) {
 #pragma unroll
-            for (int d = 0; d < 4; ++d) {
-              if (!((nmask[nt][e] >> d) & 1)) u[j][d] = 0;
-              if (RAW) un[RAW ? nt : 0][j][d] = u[j][d];
+              for (int d = 0; d < 4; ++d) {
+                if (!((nmask[nt][e] >> d) & 1)) u[j][d] = 0;
+                if (RAW) un[RAW ? nt : 0][j][d] = u[j][d];
+              }
+              if (!RAW) {
+                const T s = ((u[j][0] + u[j][1]) + u[j][2]) + u[j][3];
+                b += s * inv_h2;
+              }
+            } else if (!vcol[nt][e]) {
+              xn[nt][j] = 0;
             }
-            if (!RAW) {
-              const T s = ((u[j][0] + u[j][1]) + u[j][2]) + u[j][3];
-              b += s * inv_h2;
-            }
-          } else if (!vcol[nt][e]) {
-            xn[nt][j] = 0;
+            bn[nt][j] = b;
           }
-          bn[nt][j] = b;
         }
       }
     };
     load_rhs(0);
 
-    for (int i = 0; i < nb; ++i) {
+    for (int i = 0; i < nb; ++i, ++leaves) {
       T rhs[NTL][4], xcur[NTL][4], ddv[2];
       Acc3 acc[NTL];
 #pragma unroll
@@ -336,13 +448,15 @@ __global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkB
         acc_zero(acc[nt]);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          rhs[nt][j] = bn[nt][j];
-          if (RAW) {
-            const int r = RAW ? nt : 0;
-            const T s = ((un[r][j][0] + un[r][j][1]) + un[r][j][2]) + un[r][j][3];
-            rhs[nt][j] += s * inv_h2;
+          if constexpr (!MEM) {
+            rhs[nt][j] = bn[nt][j];
+            if (RAW) {
+              const int r = RAW ? nt : 0;
+              const T s = ((un[r][j][0] + un[r][j][1]) + un[r][j][2]) + un[r][j][3];
+              rhs[nt][j] += s * inv_h2;
+            }
+            xcur[nt][j] = xn[nt][j];
           }
-          xcur[nt][j] = xn[nt][j];
         }
       }
       ddv[0] = dn[0];
@@ -390,6 +504,17 @@ __global__ void __launch_bounds__(288) hmma_kernel(const __grid_constant__ WalkB
         } else if (type == PK_DIAG) {
           // y = right-hand side - sum of the products (in T); the diagonal product's operand
           float* opnd = MODE == MODE_SMOOTH ? ysm : xr_i;
+          if constexpr (MEM) {
+            const int buf_i = (int)(leaves & 1);
+            if (give_up(mbar_wait_or_abort(filled + buf_i, (uint32_t)((leaves >> 1) & 1), abort_flag, B.spin))) return;
+            const T* rb = rbuf + (size_t)buf_i * L * RL + (rt * 16 + g) * RL + cb + 2 * tq;
+#pragma unroll
+            for (int nt = 0; nt < NTL; ++nt)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) rhs[nt][j] = rb[8 * (j >> 1) * RL + nt * 8 + (j & 1)];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(taken + buf_i);
+          }
 #pragma unroll
           for (int nt = 0; nt < NTL; ++nt)
 #pragma unroll

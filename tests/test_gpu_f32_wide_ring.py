@@ -31,3 +31,18 @@ def test_wide_ring(M, tile, ncols):
     assert rel(direct.solve_o2_mode(R, 2.0 * 16.0**2, B)) < 2e-5
     P.hmatvec_f32(X, Bd, tile)
     assert rel(R @ B) < 2e-6
+
+
+@pytest.mark.parametrize("M,rank,tile", [(1024, 12, 32), (1024, 20, 32), (1024, 30, 32), (4096, 12, 16), (4096, 36, 16)])
+def test_many_live_z_values(M, rank, tile):
+    # the Taylor form keeps hundreds of z values alive: shared memory holds the TF32 pairs and the buffers of
+    # right-hand sides, only the buffers, or neither; against the SIMT walk at tile 1 (bar as for the
+    # other comparisons of the two kernels)
+    P = fh.Problem(fh.HMatrix(0.5, 2.0, 1.0, M, 64, rank, 0.0), 1, 63, prec=fh.MIXED_FP32)
+    B = torch.as_tensor(inputs.random_field(43, (M, 333)), dtype=torch.float64, device="cuda")
+    X, Y = torch.empty_like(B), torch.empty_like(B)
+    for product in (False, True):
+        for tc, out, t in ((True, X, tile), (False, Y, 1)):
+            P.set_tensor_cores(tc)
+            P.hmatvec_f32(out, B, t) if product else P.line_solve_f32(4, out, B, t)
+        assert float((X - Y).abs().max() / Y.abs().max()) < 1e-5
