@@ -313,23 +313,29 @@ __global__ void __launch_bounds__(288) hdf_kernel(const __grid_constant__ WalkBa
           }
           const bool far = type == PK_DENSE && i - cd.y >= W;
           const double* xj = X + (long long)cd.y * L * ld + p;
+          // blocks beyond the ring have a loop of their own: a branch per vector kept the next vector's loads
+          // behind it (as did the U slabs' bound; 4095 columns x M = 2048: 1.42 -> 1.35 ms)
+          if (!far) {
 #pragma unroll 2  // full unrolling overflows the instruction cache
-          for (int gg = 0; gg < NVT; ++gg) {
-            const int g = sp + gg * S;
-            float4 vh, vl;
-            if (!far) {
-              vh = *reinterpret_cast<const float4*>(xh + g * VE);
-              vl = *reinterpret_cast<const float4*>(xl + g * VE);
-            } else {
+            for (int gg = 0; gg < NVT; ++gg) {
+              const int g = sp + gg * S;
+              const float4 vh = *reinterpret_cast<const float4*>(xh + g * VE);
+              const float4 vl = *reinterpret_cast<const float4*>(xl + g * VE);
+#pragma unroll
+              for (int q = 0; q < Q; ++q) df_vec(ph[q], pl[q], Ah[g * L + rb + RG * q], Al[g * L + rb + RG * q], vh, vl);
+            }
+          } else {
+#pragma unroll 1
+            for (int gg = 0; gg < NVT; ++gg) {
+              const int g = sp + gg * S;
               float e[8] = {0, 0, 0, 0, 0, 0, 0, 0};
               if (valid)
 #pragma unroll
                 for (int u = 0; u < 4; ++u) df_split(xj[(long long)(g * VE + u) * ld], e[u], e[4 + u]);
-              vh = make_float4(e[0], e[1], e[2], e[3]);
-              vl = make_float4(e[4], e[5], e[6], e[7]);
-            }
+              const float4 vh = make_float4(e[0], e[1], e[2], e[3]), vl = make_float4(e[4], e[5], e[6], e[7]);
 #pragma unroll
-            for (int q = 0; q < Q; ++q) df_vec(ph[q], pl[q], Ah[g * L + rb + RG * q], Al[g * L + rb + RG * q], vh, vl);
+              for (int q = 0; q < Q; ++q) df_vec(ph[q], pl[q], Ah[g * L + rb + RG * q], Al[g * L + rb + RG * q], vh, vl);
+            }
           }
           if (type == PK_DIAG) {
 #pragma unroll
@@ -357,17 +363,14 @@ __global__ void __launch_bounds__(288) hdf_kernel(const __grid_constant__ WalkBa
           const int* uz = reinterpret_cast<const int*>(buf + (size_t)cnt * L * 8);
           const int nvq = cnt / VE;
 #pragma unroll 2  // full unrolling overflows the instruction cache
-          for (int gg = 0; gg < NVT; ++gg) {
-            const int g = sp + gg * S;
-            if (g < nvq) {
-              const int4 zi = *reinterpret_cast<const int4*>(uz + g * VE);
-              const float4 vh =
-                  make_float4(zph[zi.x * TC + cl], zph[zi.y * TC + cl], zph[zi.z * TC + cl], zph[zi.w * TC + cl]);
-              const float4 vl =
-                  make_float4(zpl[zi.x * TC + cl], zpl[zi.y * TC + cl], zpl[zi.z * TC + cl], zpl[zi.w * TC + cl]);
+          for (int g = sp; g < nvq; g += S) {
+            const int4 zi = *reinterpret_cast<const int4*>(uz + g * VE);
+            const float4 vh =
+                make_float4(zph[zi.x * TC + cl], zph[zi.y * TC + cl], zph[zi.z * TC + cl], zph[zi.w * TC + cl]);
+            const float4 vl =
+                make_float4(zpl[zi.x * TC + cl], zpl[zi.y * TC + cl], zpl[zi.z * TC + cl], zpl[zi.w * TC + cl]);
 #pragma unroll
-              for (int q = 0; q < Q; ++q) df_vec(ph[q], pl[q], Ah[g * L + rb + RG * q], Al[g * L + rb + RG * q], vh, vl);
-            }
+            for (int q = 0; q < Q; ++q) df_vec(ph[q], pl[q], Ah[g * L + rb + RG * q], Al[g * L + rb + RG * q], vh, vl);
           }
         } else {  // PK_VPART: rows are z entries, the reduction runs over x_i
           const float4* Al = Ah + cnt * L / 4;
@@ -378,6 +381,7 @@ __global__ void __launch_bounds__(288) hdf_kernel(const __grid_constant__ WalkBa
           for (int q = 0; q < Q; ++q) {
             const int r = rb + RG * q;
             const bool live = act && r < cnt;
+            if (!__any_sync(0xffffffffu, live)) continue;  // none of the warp's rows
             float zh[4] = {0, 0, 0, 0}, zl[4] = {0, 0, 0, 0};
             if (live) {
 #pragma unroll 2
