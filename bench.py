@@ -61,8 +61,8 @@ METRIC = "space-time DOF*cycles/s (time-to-1e-8 solve): mixed+warm-start vs plai
 # (same kernels and tiles on the 2D 255^2 x 512 case, scaled by columns); traffic is reported as
 # null for another M, and the entries are dropped whenever the kernel they describe changes
 TRAFFIC_PER_COLUMN = {
-    "smooth": (512, 349.2e6 / 32513),                     # profiles/humma_smooth_2d_255x512.md
-    "defect": (512, (770.95e6 + 770.24e6) / 65025),       # profiles/split_defect_2d_255x512.md (both kernels)
+    "smooth": (512, (150.61e6 + 30.52e6) / 32513),                     # profiles/humma_smooth_2d_255x512.md
+    "defect": (512, (772.95e6 + 803.34e6) / 65025),       # profiles/split_defect_2d_255x512.md (both kernels)
 }
 
 

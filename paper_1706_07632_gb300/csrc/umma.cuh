@@ -2,7 +2,8 @@
 // accumulation in tensor memory, FP32 grid functions.
 //
 // The walk of panel.cuh transposed onto the 5th-generation tensor cores.  A CTA owns a tile of
-// 128 spatial columns; thread c of the four consumer warps owns column c (TMEM lane c).  Every
+// 128 spatial columns; thread c of the four walk warps owns column c (TMEM lane c), and four memory
+// warps load and store the columns a leaf ahead and behind (see the kernel).  Every
 // chunk product of a leaf row i becomes one tcgen05.mma with M = 128 (the columns), N = the chunk's
 // output rows, K = its reduction index, A from shared memory (the columns' operand tile, 128 x K,
 // K-major) and B = the chunk itself (N x K, K-major, streamed by TMA bulk copies in the canonical
@@ -14,10 +15,10 @@
 //   VPART     v[c, q] = sum_k x_i[c, k] V_i[q, k], then z[c, code_q] (+)= v[c, q]
 // (D', Dinv': without their diagonal, which is applied in FP32 by the threads).  One elected thread
 // issues the MMAs; tcgen05.commit signals their completion on mbarriers: the slot's "empty" barrier
-// (which also collects one arrival per consumer warp, so a slot is refilled only when the MMA and
+// (which also collects one arrival per walk warp, so a slot is refilled only when the MMA and
 // every warp are done with it) and the acc / res / v barriers that the threads wait on before they
 // read tensor memory with tcgen05.ld.  Threads write the A tiles (x ring, y, z) with 16-byte stores
-// in the core-matrix layout, then fence.proxy.async and meet on a consumer mbarrier before the MMA
+// in the core-matrix layout, then fence.proxy.async and meet on the walk warps' mbarrier before the MMA
 // that reads them is issued.  Every wait is bounded and watches the shared abort flag; every exit
 // path frees the tensor memory after the MMAs in flight completed.
 #pragma once
@@ -206,9 +207,11 @@ __host__ __device__ inline long long umma_tiles(const Geo& g, long long ncols) {
 // neighbour sum / h^2; product: x, as BF16 pairs) into one while the walk works on the other, and
 // write the leaf's result (x; B - d x - sum) back once the walk has left it there.  The walk then
 // never waits for DRAM, which took most of its time when its own threads loaded the next leaf
-// (2.37 ms per finest half-sweep of a 1023^2 x 512 grid, 2.31 ms now, the traffic between L2 and the SMs
-// bounding it; 214 -> 176 us for a line solve of 100003 x 512 columns).  96 registers and 112 KB of shared
-// memory: two CTAs per SM.
+// (a line solve of 100003 x 512 columns 214 -> 176 us; with room for the L1 cache 151).  What bounds the
+// memory warps is the loads they can keep in flight: a finest half-sweep of a 1023^2 x 512 grid took 2.37
+// ms with loads by the walk, 2.31 with memory warps, 1.60 with grid functions stored by colour (whole
+// sectors), 1.47 with rolled loops (instruction cache), 1.04 with 60 instead of 28 KB of L1; its bytes
+// need 0.48 ms.  96 registers and at most 97 KB of shared memory: two CTAs per SM.
 template <int MODE>
 __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_constant__ WalkBatch<float, uint16_t> B) {
   constexpr int L = kUmmaL, NT = kUmmaCols;
