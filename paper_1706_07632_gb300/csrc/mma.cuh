@@ -30,7 +30,7 @@ constexpr int kMmaLP = 80;  // padded x-tile column (floats): 8 columns x 4 lane
 // column of the tile (in the products' lane layout a load covers 8 rows x 2 columns), so that the products
 // never wait for them and their threads hold no load state.  Tile 32 takes three warps, which with the
 // eight consumer warps and the producer leave each thread 168 registers (with four: 128, and the products
-// spill).  Half-sweep of 255^2 points x M = 1024 at tile 32: 830 -> 694 us (four warps 795); of 4095
+// spill).  Half-sweep of 255^2 points x M = 1024 at tile 32: 830 -> 631 us (four warps 795); of 4095
 // points x M = 4096 in FP64 at tile 16: 511 -> 403 us.
 __host__ __device__ constexpr int mma_mem(int TC) { return TC == 32 ? 96 : 128; }
 constexpr int kMmaRhsPad = 8;  // columns of padding of a right-hand-side row: the rows a warp reads hit distinct banks
