@@ -175,11 +175,12 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// a load of data that no thread writes during the launch, kept in program order with its like (so that
-// a group of loads is in flight before the first use)
-__device__ __forceinline__ float ld_nc(const float* p) {
+// a load kept in program order with its like and with every other access to memory (so that a group of
+// loads is in flight before the first use).  Not by the non-coherent path: a line solve may work in place
+// (X aliases B), so its launch writes what it reads, each element after its only read, by the same thread
+__device__ __forceinline__ float ld_ordered(const float* p) {
   float v;
-  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
   return v;
 }
 
@@ -390,8 +391,9 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
       bool valid;
       long long p = 0;
       // columns past the panel's end read column 0 (any valid address) and are zeroed, so that the loads
-      // carry no predicate; missing neighbours read the column itself with weight 0
-      long long n0 = 0, n1 = 0, n2 = 0, n3 = 0;
+      // carry no predicate; missing neighbours read the right-hand side with weight 0 (never X: the point
+      // itself and column 0 are of the colour that this launch writes)
+      const float *q0 = J.B, *q1 = J.B, *q2 = J.B, *q3 = J.B;
       float w0 = 0.f, w1 = 0.f, w2 = 0.f, w3 = 0.f;
       if (grid) {
         const int N = J.geo.N;
@@ -418,10 +420,10 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
         const NbrOffsets off = nbr_offsets(J.geo);
         const bool odd = iy & 1;
         const int left = odd ? off.left[1] : off.left[0];
-        n0 = w0 != 0.f ? p + left : p;
-        n1 = w1 != 0.f ? p + left + off.step : p;
-        n2 = w2 != 0.f ? p + (odd ? off.up[1] : off.up[0]) : p;
-        n3 = w3 != 0.f ? p + (odd ? off.down[1] : off.down[0]) : p;
+        q0 = w0 != 0.f ? J.X + p + left : J.B + p;
+        q1 = w1 != 0.f ? J.X + p + left + off.step : J.B + p;
+        q2 = w2 != 0.f ? J.X + p + (odd ? off.up[1] : off.up[0]) : J.B + p;
+        q3 = w3 != 0.f ? J.X + p + (odd ? off.down[1] : off.down[0]) : J.B + p;
       } else {
         const long long cg = (g - J.tile0) * NT + c;
         valid = cg < J.ncols;
@@ -436,20 +438,19 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
         }
         const long long at = (long long)i * L * ld;
         if (grid) {
-          const float* Bl = J.B + at + p;
-          const float* Xl = J.X + at;
+          const float* Bl = J.B + p;
 #pragma unroll 1
           for (int r0 = 0; r0 < L; r0 += 8) {
             float v[8], a0[8], a1[8], a2[8], a3[8];
             uint32_t q[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-              const long long o = (long long)(r0 + j) * ld;
-              v[j] = ld_nc(Bl + o);
-              a0[j] = ld_nc(Xl + o + n0);
-              a1[j] = ld_nc(Xl + o + n1);
-              a2[j] = ld_nc(Xl + o + n2);
-              a3[j] = ld_nc(Xl + o + n3);
+              const long long o = at + (long long)(r0 + j) * ld;
+              v[j] = ld_ordered(Bl + o);
+              a0[j] = ld_ordered(q0 + o);
+              a1[j] = ld_ordered(q1 + o);
+              a2[j] = ld_ordered(q2 + o);
+              a3[j] = ld_ordered(q3 + o);
             }
 #pragma unroll
             for (int j = 0; j < 8; ++j)
@@ -462,7 +463,7 @@ __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_const
           for (int r0 = 0; r0 < L; r0 += 32) {
             float v[32];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = ld_nc(Bl + (long long)(r0 + j) * ld);
+            for (int j = 0; j < 32; ++j) v[j] = ld_ordered(Bl + (long long)(r0 + j) * ld);
 #pragma unroll
             for (int j = 0; j < 32; j += 8) {
               uint32_t q[8];
