@@ -25,9 +25,9 @@
  *  - fhmg_last_error() returns a message for the last failure of the calling thread.
  *  - A problem lives on the CUDA device that was current when it was created; every call on it
  *    makes that device current for its duration and restores the caller's device afterwards.
- *  - Every device-side wait of the walk kernels is bounded.  A walk whose wait gives up leaves
- *    early and sets the problem's error word; the next call that returns a host value (a norm, a
- *    solve) reports it as FHMG_ETIMEOUT and clears it, so the problem stays usable.
+ *  - Every device-side wait is bounded.  A walk whose wait gives up leaves early and sets the
+ *    problem's error word; the next call that returns a host value (a norm, a solve) reports it as
+ *    FHMG_ETIMEOUT and clears it, so the problem stays usable.  The network's waits: fhmg_wsnet_forward.
  */
 #ifndef FHMG_H_
 #define FHMG_H_
@@ -311,8 +311,19 @@ int fhmg_wsnet_destroy(fhmg_wsnet net);
 int fhmg_wsnet_num_params(fhmg_wsnet net, long long* n);
 int fhmg_wsnet_get_params(fhmg_wsnet net, float* host);
 int fhmg_wsnet_set_params(fhmg_wsnet net, const float* host);
-/* Y (n device floats) = network(X) for X (n x 6 device floats); bf16 != 0: BF16 tensor cores. */
+/* Y (n device floats) = network(X) for X (n x 6 device floats); bf16 != 0: BF16 tensor cores.  Returns
+ * before the GPU work ends.  The BF16 network of hidden widths 64, 128, .., 320 is one kernel with bounded
+ * device waits: if one gives up, the rows of Y that its CTA works on are NaN and fhmg_wsnet_status
+ * reports it (later calls on the network run as usual). */
 int fhmg_wsnet_forward(fhmg_wsnet net, const float* X, int n, int bf16, float* Y, void* stream);
+/* Synchronises the stream and returns FHMG_ETIMEOUT if a device wait of an fhmg_wsnet_forward on this network
+ * gave up since the last report (which this call clears), else FHMG_OK.  A wait that gives up in
+ * fhmg_ws_predict is that call's own status. */
+int fhmg_wsnet_status(fhmg_wsnet net, void* stream);
+/* Test hook, as fhmg_problem_inject_timeout: the network's next one-kernel BF16 pass never gets one of its
+ * weight tiles and its waits give up after consumer_spin polls (1 .. 2^24).  EINVAL for networks that
+ * stream no tiles (one hidden layer, or a width outside 64, 128, .., 320). */
+int fhmg_wsnet_inject_timeout(fhmg_wsnet net, long long consumer_spin);
 /* Mean-squared loss against targets Y and its gradient (host outputs, either may be NULL). */
 int fhmg_wsnet_loss_grad(fhmg_wsnet net, const float* X, const float* Y, int n, float* loss_host,
                          float* grad_host, void* stream);

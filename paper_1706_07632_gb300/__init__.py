@@ -81,6 +81,8 @@ _SIGS = {
     "fhmg_wsnet_get_params": (_I, [_P, _P]),
     "fhmg_wsnet_set_params": (_I, [_P, _P]),
     "fhmg_wsnet_forward": (_I, [_P, _P, _I, _I, _P, _P]),
+    "fhmg_wsnet_status": (_I, [_P, _P]),
+    "fhmg_wsnet_inject_timeout": (_I, [_P, _LL]),
     "fhmg_wsnet_loss_grad": (_I, [_P, _P, _P, _I, _P, _P, _P]),
     "fhmg_wsnet_train": (_I, [_P, _P, _P, _LL, _I, _I, _c.c_float, _c.c_ulonglong, _c.POINTER(_c.c_float), _P]),
     "fhmg_ws_dataset": (_I, [_P, _P, _P, _D, _I, _c.c_float, _P, _P, _c.POINTER(_LL)]),
@@ -395,6 +397,14 @@ class WSNet:
 
     def forward(self, X, Y, bf16=False, stream=None):
         _check(lib().fhmg_wsnet_forward(self._h, _fptr(X), X.shape[0], 1 if bf16 else 0, _fptr(Y), _stream_ptr(stream)))
+
+    def status(self, stream=None):
+        """Raises FHMG_ETIMEOUT if a device wait of a forward() gave up since the last call (synchronises)."""
+        _check(lib().fhmg_wsnet_status(self._h, _stream_ptr(stream)))
+
+    def inject_timeout(self, consumer_spin=1024):
+        """Test hook: the next one-kernel BF16 pass misses a weight tile and its waits give up."""
+        _check(lib().fhmg_wsnet_inject_timeout(self._h, consumer_spin))
 
     def loss_grad(self, X, Y, stream=None):
         import numpy as np

@@ -457,6 +457,7 @@ struct MlpArgs {
   long long boff[9];
   float* Y;
   int* err;                         // set if a bounded wait gives up
+  long long spin, withhold;         // polls of the MMA and epilogue warps' waits; 1-based tile never loaded (test hook)
 };
 
 constexpr int kMlpRows = 128, kMlpMaxH = 320, kMlpEpi = 256, kMlpBlock = kMlpEpi + 64;
@@ -560,9 +561,13 @@ __global__ void __launch_bounds__(kMlpBlock, 1) mlp_bf16(int H, const __grid_con
       int slot = 0;
       uint32_t phase = 1;
       long long k = 0;
-      bool ok = true;
-      for (int blk = blockIdx.x; blk < blocks && ok; blk += gridDim.x)
+      bool ok = true, stop = false;
+      for (int blk = blockIdx.x; blk < blocks && ok && !stop; blk += gridDim.x)
         for (int j = 0; j < nhid * KT; ++j, ++k) {
+          if (k + 1 == g.withhold) {
+            stop = true;
+            break;
+          }
           if (!mbar_wait_or_abort(wfree + slot, phase, abort_flag)) {
             ok = false;
             break;
@@ -583,7 +588,7 @@ __global__ void __launch_bounds__(kMlpBlock, 1) mlp_bf16(int H, const __grid_con
     uint32_t fphase = 0, aphase = 0;
     bool ok = true;
     auto wait = [&](uint64_t* bar, uint32_t ph) -> bool {
-      ok = __all_sync(0xffffffffu, mbar_wait_or_abort(bar, ph, abort_flag));
+      ok = __all_sync(0xffffffffu, mbar_wait_or_abort(bar, ph, abort_flag, g.spin));
       tc_after_sync();
       return ok;
     };
@@ -665,7 +670,7 @@ __global__ void __launch_bounds__(kMlpBlock, 1) mlp_bf16(int H, const __grid_con
     if ((int)blockIdx.x < blocks) put_x(blockIdx.x);
     for (int blk = blockIdx.x; blk < blocks && !failed; blk += gridDim.x) {
       for (int l = 0; l <= g.layers; ++l) {
-        if (!__all_sync(0xffffffffu, mbar_wait_or_abort(accdone, dphase, abort_flag))) {
+        if (!__all_sync(0xffffffffu, mbar_wait_or_abort(accdone, dphase, abort_flag, g.spin))) {
           if (lane == 0) raise();
           failed = true;
           break;
@@ -722,6 +727,11 @@ __global__ void __launch_bounds__(kMlpBlock, 1) mlp_bf16(int H, const __grid_con
   tc_after_sync();
   if (w == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols));
+  // after a wait gave up: none of this CTA's rows keeps what the array held before (here and not where the
+  // epilogue gives up: in its loop the branch cost 14 of 338 us for 294912 rows)
+  if (*abort_flag && t < kMlpRows)
+    for (long long r = (long long)blockIdx.x * kMlpRows + t; r < g.n; r += (long long)gridDim.x * kMlpRows)
+      g.Y[r] = __int_as_float(0x7FC00000);
 }
 
 // Z += b (row broadcast); A = SiLU(Z) (act = 1) or Z (act = 0).  Z kept for the backward pass.
@@ -804,7 +814,8 @@ struct fhmg_wsnet_s {
   float* Vo = nullptr;
   __nv_bfloat16* Pbf = nullptr;   // BF16 copy of the weights (inference)
   unsigned char* Wpk = nullptr;   // the weights as MMA operands: widths 64, 128, .., kMlpMaxH (mlp_bf16)
-  int* err = nullptr;             // set by mlp_bf16 if a bounded wait gave up
+  int* err = nullptr;             // set by mlp_bf16 if a bounded wait gave up: [0] in a prediction, [1] in a forward call
+  long long inj_spin = 0;         // armed test hook: the next mlp_bf16 withholds a weight tile, waits poll inj_spin times
   long long step = 0;
   // activations for a batch of up to cap rows
   int cap = 0;
@@ -963,6 +974,9 @@ int backward32(fhmg_wsnet net, cudaStream_t st, const float* X, const float* Y, 
   return FHMG_OK;
 }
 
+// Y = network(X); err: the word that the one-launch network sets if a wait gives up
+int forward_rows(fhmg_wsnet net, const float* X, int n, int bf16, float* Y, cudaStream_t st, int* err);
+
 }  // namespace
 
 extern "C" {
@@ -996,11 +1010,11 @@ int fhmg_wsnet_create(int hidden, int layers, unsigned long long seed, fhmg_wsne
   };
   if ((s = nalloc(net, &net->P, host.size())) || (s = nalloc(net, &net->G, host.size())) ||
       (s = nalloc(net, &net->Mo, host.size())) || (s = nalloc(net, &net->Vo, host.size())) ||
-      (s = nalloc(net, &net->Pbf, host.size())) || (s = nalloc(net, &net->loss, 1)) || (s = nalloc(net, &net->err, 1)) ||
+      (s = nalloc(net, &net->Pbf, host.size())) || (s = nalloc(net, &net->loss, 1)) || (s = nalloc(net, &net->err, 2)) ||
       (hidden % 64 == 0 && hidden <= kMlpMaxH && (s = nalloc(net, &net->Wpk, mlp_packed(hidden, layers)))))
     return bail(s);
   if (cudaMemcpy(net->P, host.data(), host.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemset(net->err, 0, sizeof(int)) != cudaSuccess ||
+      cudaMemset(net->err, 0, 2 * sizeof(int)) != cudaSuccess ||
       cudaMemset(net->Mo, 0, host.size() * 4) != cudaSuccess || cudaMemset(net->Vo, 0, host.size() * 4) != cudaSuccess)
     return bail(fhmg_internal_fail(FHMG_ECUDA, "wsnet upload failed"));
   *out = net;
@@ -1035,7 +1049,46 @@ int fhmg_wsnet_set_params(fhmg_wsnet net, const float* host) {
 
 int fhmg_wsnet_forward(fhmg_wsnet net, const float* X, int n, int bf16, float* Y, void* stream) {
   if (!net || !X || !Y || n < 1) return fhmg_internal_fail(FHMG_EINVAL, "bad arguments");
+  return forward_rows(net, X, n, bf16, Y, (cudaStream_t)stream, net->err + 1);
+}
+
+int fhmg_wsnet_status(fhmg_wsnet net, void* stream) {
+  if (!net) return fhmg_internal_fail(FHMG_EINVAL, "null argument");
   cudaStream_t st = (cudaStream_t)stream;
+  int err = 0;
+  NCK(cudaMemcpyAsync(&err, net->err + 1, sizeof err, cudaMemcpyDeviceToHost, st));
+  NCK(cudaStreamSynchronize(st));
+  if (!err) return FHMG_OK;
+  NCK(cudaMemsetAsync(net->err + 1, 0, sizeof err, st));
+  return fhmg_internal_fail(FHMG_ETIMEOUT, "the network kernel gave up waiting on a shared-memory stage");
+}
+
+int fhmg_wsnet_inject_timeout(fhmg_wsnet net, long long consumer_spin) {
+  if (!net) return fhmg_internal_fail(FHMG_EINVAL, "null argument");
+  if (consumer_spin < 1 || consumer_spin > fhmg::kSpinLimit)
+    return fhmg_internal_fail(FHMG_EINVAL, "consumer spin limit must be in 1..2^24");
+  if (!net->Wpk || net->layers < 2) return fhmg_internal_fail(FHMG_EINVAL, "the network streams no weight tiles");
+  net->inj_spin = consumer_spin;
+  return FHMG_OK;
+}
+
+int fhmg_wsnet_loss_grad(fhmg_wsnet net, const float* X, const float* Y, int n, float* loss_host, float* grad_host,
+                         void* stream) {
+  if (!net || !X || !Y || n < 1) return fhmg_internal_fail(FHMG_EINVAL, "bad arguments");
+  cudaStream_t st = (cudaStream_t)stream;
+  int s = forward32(net, st, X, n);
+  if (s || (s = backward32(net, st, X, Y, n))) return s;
+  if (loss_host) NCK(cudaMemcpyAsync(loss_host, net->loss, 4, cudaMemcpyDeviceToHost, st));
+  if (grad_host) NCK(cudaMemcpyAsync(grad_host, net->G, net->nparams * 4, cudaMemcpyDeviceToHost, st));
+  NCK(cudaStreamSynchronize(st));
+  return FHMG_OK;
+}
+
+}  // extern "C"
+
+namespace {
+
+int forward_rows(fhmg_wsnet net, const float* X, int n, int bf16, float* Y, cudaStream_t st, int* err) {
   const int L = (int)net->width.size() - 1;
   int s;
   if (bf16 && net->Wpk && reinterpret_cast<uintptr_t>(X) % 8 == 0) {
@@ -1044,7 +1097,13 @@ int fhmg_wsnet_forward(fhmg_wsnet net, const float* X, int n, int bf16, float* Y
     ++g_nn_launches;
     NCK(cudaGetLastError());
     MlpArgs a{};
-    a.n = n, a.layers = net->layers, a.X = X, a.W = net->Wpk, a.P = net->P, a.Y = Y, a.err = net->err;
+    a.n = n, a.layers = net->layers, a.X = X, a.W = net->Wpk, a.P = net->P, a.Y = Y, a.err = err;
+    a.spin = fhmg::kSpinLimit;
+    if (net->inj_spin > 0) {
+      a.spin = net->inj_spin;
+      a.withhold = (net->layers - 1) * (net->hidden / 64) > 1 ? 2 : 1;  // within the first block of rows
+      net->inj_spin = 0;
+    }
     for (int l = 0; l < L; ++l) a.boff[l] = net->boff[l];
     static fhmg::KernelCache cache;
     const size_t smem = mlp_smem(net->hidden, net->layers).total + 1024;
@@ -1097,19 +1156,7 @@ int fhmg_wsnet_forward(fhmg_wsnet net, const float* X, int n, int bf16, float* Y
   return FHMG_OK;
 }
 
-int fhmg_wsnet_loss_grad(fhmg_wsnet net, const float* X, const float* Y, int n, float* loss_host, float* grad_host,
-                         void* stream) {
-  if (!net || !X || !Y || n < 1) return fhmg_internal_fail(FHMG_EINVAL, "bad arguments");
-  cudaStream_t st = (cudaStream_t)stream;
-  int s = forward32(net, st, X, n);
-  if (s || (s = backward32(net, st, X, Y, n))) return s;
-  if (loss_host) NCK(cudaMemcpyAsync(loss_host, net->loss, 4, cudaMemcpyDeviceToHost, st));
-  if (grad_host) NCK(cudaMemcpyAsync(grad_host, net->G, net->nparams * 4, cudaMemcpyDeviceToHost, st));
-  NCK(cudaStreamSynchronize(st));
-  return FHMG_OK;
-}
-
-}  // extern "C"
+}  // namespace
 
 // ---------------------------------------------------------------- spectral warm start
 
@@ -1340,7 +1387,7 @@ int fhmg_ws_predict(fhmg_wsnet net, fhmg_problem prob, const double* f, double a
   NCK(cudaGetLastError());
   if ((s = sp.project(f32, 1, c))) return s;
   if ((s = sp.features(alpha, nullptr, nullptr, X))) return s;
-  if ((s = fhmg_wsnet_forward(net, X, nm * M, bf16, Y, sp.st))) return s;
+  if ((s = forward_rows(net, X, nm * M, bf16, Y, sp.st, net->err))) return s;
   mode_amplitudes<<<nblk((long long)nm * M), 256, 0, sp.st>>>(nm, M, c, Y, sp.lam, G);
   ++g_nn_launches;
   NCK(cudaGetLastError());
