@@ -730,8 +730,8 @@ __global__ void __launch_bounds__(kMlpBlock, 1) mlp_bf16(int H, const __grid_con
   // after a wait gave up: none of this CTA's rows keeps what the array held before (here and not where the
   // epilogue gives up: in its loop the branch cost 14 of 338 us for 294912 rows)
   if (*abort_flag && t < kMlpRows)
-    for (long long r = (long long)blockIdx.x * kMlpRows + t; r < g.n; r += (long long)gridDim.x * kMlpRows)
-      g.Y[r] = __int_as_float(0x7FC00000);
+    for (int blk = blockIdx.x; blk < blocks; blk += gridDim.x)
+      if (t < g.n - blk * kMlpRows) g.Y[blk * kMlpRows + t] = __int_as_float(0x7FC00000);
 }
 
 // Z += b (row broadcast); A = SiLU(Z) (act = 1) or Z (act = 0).  Z kept for the backward pass.
