@@ -336,7 +336,10 @@ int fhmg_wsnet_train(fhmg_wsnet net, const float* X, const float* Y, long long n
  * for K^dim * M rows; *nrows receives the count). */
 int fhmg_ws_dataset(fhmg_problem prob, const double* u, const double* f, double alpha, int K, float rel_thr,
                     float* X_out, float* Y_out, long long* nrows);
-/* u0 (device, M x N^dim) = warm start for source f (constant in time) and order alpha. */
+/* u0 (device, M x N^dim) = warm start for source f (constant in time) and order alpha; synchronises the
+ * problem's stream.  Its scratch (in 2D chiefly 4 M min(K, N) N bytes, and 32 bytes per network row, of which
+ * there are M min(K, N)^dim) stays with the network, grown to the largest prediction so far and freed by
+ * fhmg_wsnet_destroy: predictions on one network come one after another, on whatever problems. */
 int fhmg_ws_predict(fhmg_wsnet net, fhmg_problem prob, const double* f, double alpha, int K, int bf16, double* u0);
 /* Kernel launches issued so far by the network and warm-start kernels (training, inference,
  * projection, synthesis) of the whole process. */

@@ -825,8 +825,8 @@ struct fhmg_wsnet_s {
   float* loss = nullptr;
   __nv_bfloat16* Abf[2] = {nullptr, nullptr};
   // scratch of predictions, kept from call to call (the i-th buffer a prediction asks for, grown when it
-  // asks for more): every prediction ends synchronised, so no two use it at a time unless the net itself
-  // is shared by threads, which its other buffers exclude
+  // asks for more): every prediction ends synchronised, also one that fails on the way, so no two use it at a
+  // time unless the net itself is shared by threads, which its other buffers exclude
   std::vector<std::pair<void*, size_t>> ws;
   std::vector<void*> allocs;
 };
@@ -836,7 +836,10 @@ namespace {
 template <typename T>
 int nalloc(fhmg_wsnet net, T** p, size_t n) {
   cudaError_t e = cudaMalloc((void**)p, (n ? n : 1) * sizeof(T));
-  if (e != cudaSuccess) return fhmg_internal_fail(FHMG_ENOMEM, cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // not sticky; keep it out of the next launch check
+    return fhmg_internal_fail(FHMG_ENOMEM, cudaGetErrorString(e));
+  }
   net->allocs.push_back(*p);
   return FHMG_OK;
 }
@@ -1275,11 +1278,16 @@ struct Spectral {
   std::vector<void*> mem;  // buffers of its own (no net)
   fhmg_wsnet net = nullptr;  // or the net whose scratch it uses, and the buffers taken so far
   size_t taken = 0;
+  bool running = false;      // kernels issued on st may still use the net's scratch
   float* S = nullptr;   // N x K
   double* lam = nullptr;
   double* tdev = nullptr;
   ~Spectral() {
     for (void* p : mem) cudaFree(p);
+    if (net && running) {  // a prediction that stops early: its kernels end before the next one takes the scratch
+      cudaMemsetAsync(net->err, 0, sizeof(int), st);
+      cudaStreamSynchronize(st);
+    }
   }
   template <typename T>
   int alloc(T** p, size_t n) {
@@ -1288,15 +1296,28 @@ struct Spectral {
       *p = (T*)net->ws[taken++].first;
       return FHMG_OK;
     }
-    cudaError_t e = cudaMalloc((void**)p, bytes);
-    if (e != cudaSuccess) return fhmg_internal_fail(FHMG_ENOMEM, cudaGetErrorString(e));
-    if (!net) {
-      mem.push_back(*p);
-      return FHMG_OK;
+    auto give_back = [&](size_t i) {  // (frees wait for the device)
+      cudaFree(net->ws[i].first);
+      net->ws[i] = {nullptr, 0};
+    };
+    if (net) {  // the smaller buffer goes first, so that the two are never held at once
+      if (taken == net->ws.size()) net->ws.push_back({nullptr, 0});
+      give_back(taken);
     }
-    if (taken == net->ws.size()) net->ws.push_back({nullptr, 0});
-    cudaFree(net->ws[taken].first);
-    net->ws[taken++] = {*p, bytes};
+    cudaError_t e = cudaMalloc((void**)p, bytes);
+    if (e != cudaSuccess && net) {  // nor do buffers of an earlier prediction stand in this one's way
+      cudaGetLastError();
+      for (size_t i = taken + 1; i < net->ws.size(); ++i) give_back(i);
+      e = cudaMalloc((void**)p, bytes);
+    }
+    if (e != cudaSuccess) {
+      cudaGetLastError();  // not sticky; keep it out of the next launch check
+      return fhmg_internal_fail(FHMG_ENOMEM, cudaGetErrorString(e));
+    }
+    if (net)
+      net->ws[taken++] = {*p, bytes};
+    else
+      mem.push_back(*p);
     return FHMG_OK;
   }
   int init(fhmg_problem p, int K_) {
@@ -1307,6 +1328,7 @@ struct Spectral {
     K = K_ < N ? K_ : N;
     nm = dim == 1 ? K : K * K;
     if ((s = alloc(&S, (size_t)N * K)) || (s = alloc(&lam, nm)) || (s = alloc(&tdev, M + 1))) return s;
+    running = true;
     sine_basis<<<nblk((long long)N * K), 256, 0, st>>>(N, K, S);
     ++g_nn_launches;
     mode_lambdas<<<(nm + 127) / 128, 128, 0, st>>>(dim, N, Lx, K, nm, lam);
@@ -1407,10 +1429,8 @@ int fhmg_ws_predict(fhmg_wsnet net, fhmg_problem prob, const double* f, double a
   int err = 0;
   NCK(cudaMemcpyAsync(&err, net->err, sizeof err, cudaMemcpyDeviceToHost, sp.st));
   NCK(cudaStreamSynchronize(sp.st));
-  if (err) {
-    NCK(cudaMemsetAsync(net->err, 0, sizeof err, sp.st));
-    return fhmg_internal_fail(FHMG_ETIMEOUT, "the network kernel gave up waiting on a shared-memory stage");
-  }
+  if (err) return fhmg_internal_fail(FHMG_ETIMEOUT, "the network kernel gave up waiting on a shared-memory stage");
+  sp.running = false;
   return FHMG_OK;
 }
 
