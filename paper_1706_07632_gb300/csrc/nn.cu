@@ -820,8 +820,8 @@ struct fhmg_wsnet_s {
   // activations for a batch of up to cap rows
   int cap = 0;
   std::vector<float*> Z, A, dA;   // per layer
-  float* part = nullptr;          // partial sums of split weight gradients (part_n floats)
-  size_t part_n = 0;
+  float* part = nullptr;          // partial sums of split weight gradients (part_n floats, not in allocs): as many as
+  size_t part_n = 0;              // the largest batch so far needs
   float* loss = nullptr;
   __nv_bfloat16* Abf[2] = {nullptr, nullptr};
   // scratch of predictions, kept from call to call (the i-th buffer a prediction asks for, grown when it
@@ -896,11 +896,36 @@ int gemm_to_f64(cudaStream_t st, int M, int N, int K, const float* A, int lda, c
   return tb ? gemm_launch<false, true, EPI_F64>(st, g, batch) : gemm_launch<false, false, EPI_F64>(st, g, batch);
 }
 
-int ensure_part(fhmg_wsnet net, size_t n) {
-  if (n <= net->part_n) return FHMG_OK;
-  const int s = nalloc(net, &net->part, n);
-  if (s == FHMG_OK) net->part_n = n;
-  return s;
+// Rows per split of the weight gradient of layer l < L - 1 over a batch of n rows (a multiple of the K tile):
+// enough splits that the tiles fill every SM twice.
+int split_rows(fhmg_wsnet net, int n, int l) {
+  const int wi = net->width[l], wo = net->width[l + 1];
+  const long long tiles = (long long)((wi + kGB - 1) / kGB) * ((wo + kGB - 1) / kGB);
+  const long long want = (2LL * fhmg::device_sms() + tiles - 1) / tiles;
+  const int kper = (int)((n + want - 1) / want);
+  return (kper + kGK - 1) / kGK * kGK;
+}
+
+// Room for the partial sums of every layer, before the backward pass begins (a pass that grew it layer by layer
+// held all the smaller ones as well, and stood still at each allocation)
+int ensure_part(fhmg_wsnet net, int n) {
+  const int L = (int)net->width.size() - 1;
+  size_t need = (size_t)((n + kOutRows - 1) / kOutRows) * (net->width[L - 1] + 1);
+  for (int l = 0; l < L - 1; ++l) {
+    const int kper = split_rows(net, n, l);
+    need = std::max(need, (size_t)((n + kper - 1) / kper) * net->width[l + 1] * (net->width[l] + 1));
+  }
+  if (need <= net->part_n) return FHMG_OK;
+  cudaFree(net->part);  // waits for the device
+  net->part = nullptr, net->part_n = 0;
+  const cudaError_t e = cudaMalloc((void**)&net->part, need * sizeof(float));
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    net->part = nullptr;
+    return fhmg_internal_fail(FHMG_ENOMEM, cudaGetErrorString(e));
+  }
+  net->part_n = need;
+  return FHMG_OK;
 }
 
 // FP32 forward of n rows X (n x kFeat) -> output A[L] (n x 1); activations kept.
@@ -926,9 +951,11 @@ int forward32(fhmg_wsnet net, cudaStream_t st, const float* X, int n) {
 
 // Backward of the MSE loss against targets Y; gradients into net->G (overwritten).  The gradient of
 // layer l (its weights, then its bias, consecutive in G) is summed over splits of the rows into
-// partial sums, then over the splits: enough splits that the tiles fill every SM twice.
+// partial sums, then over the splits.
 int backward32(fhmg_wsnet net, cudaStream_t st, const float* X, const float* Y, int n) {
   const int L = (int)net->width.size() - 1;
+  int s = ensure_part(net, n);
+  if (s) return s;
   NCK(cudaMemsetAsync(net->loss, 0, sizeof(float), st));
   mse_fwd_bwd<<<nblk(n), 256, 0, st>>>(n, net->A[L], Y, net->dA[L], net->loss);
   ++g_nn_launches;
@@ -939,10 +966,8 @@ int backward32(fhmg_wsnet net, cudaStream_t st, const float* X, const float* Y, 
     NCK(cudaGetLastError());
     return FHMG_OK;
   };
-  int s;
   {
     const int l = L - 1, w = net->width[l], nr = (n + kOutRows - 1) / kOutRows;
-    if ((s = ensure_part(net, (size_t)nr * (w + 1)))) return s;
     out_layer_bwd<<<dim3(w / 128 + 1, nr), 128, 0, st>>>(n, w, l > 0, net->dA[L], net->P + net->woff[l],
                                                          l > 0 ? net->A[l] : X, l > 0 ? net->Z[l - 1] : nullptr,
                                                          net->dA[l], net->part);
@@ -954,12 +979,8 @@ int backward32(fhmg_wsnet net, cudaStream_t st, const float* X, const float* Y, 
     const int wi = net->width[l], wo = net->width[l + 1];
     const float* dz = net->dA[l + 1];  // gradient of the layer's pre-activation, n x wo
     const long long m = (long long)wo * wi + wo;
-    const long long tiles = (long long)((wi + kGB - 1) / kGB) * ((wo + kGB - 1) / kGB);
-    const long long want = (2LL * fhmg::device_sms() + tiles - 1) / tiles;
-    int kper = (int)((n + want - 1) / want);
-    kper = (kper + kGK - 1) / kGK * kGK;
+    const int kper = split_rows(net, n, l);
     const int splits = (n + kper - 1) / kper;
-    if ((s = ensure_part(net, (size_t)splits * m))) return s;
     GemmArgs g{};  // dW = dz^T in (wo x wi), db = column sums of dz
     g.M = wo, g.N = wi, g.K = n, g.kper = kper;
     g.A = dz, g.lda = wo, g.B = l == 0 ? X : net->A[l], g.ldb = wi;
@@ -1027,6 +1048,7 @@ int fhmg_wsnet_create(int hidden, int layers, unsigned long long seed, fhmg_wsne
 int fhmg_wsnet_destroy(fhmg_wsnet net) {
   if (!net) return FHMG_OK;
   for (void* a : net->allocs) cudaFree(a);
+  cudaFree(net->part);
   for (auto& w : net->ws) cudaFree(w.first);
   delete net;
   return FHMG_OK;
