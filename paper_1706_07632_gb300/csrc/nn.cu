@@ -817,8 +817,9 @@ struct fhmg_wsnet_s {
   int* err = nullptr;             // set by mlp_bf16 if a bounded wait gave up: [0] in a prediction, [1] in a forward call
   long long inj_spin = 0;         // armed test hook: the next mlp_bf16 withholds a weight tile, waits poll inj_spin times
   long long step = 0;
-  // activations for a batch of up to cap rows
+  // activations for a batch of up to cap rows, owned by act
   int cap = 0;
+  std::vector<void*> act;
   std::vector<float*> Z, A, dA;   // per layer
   float* part = nullptr;          // partial sums of split weight gradients (part_n floats, not in allocs): as many as
   size_t part_n = 0;              // the largest batch so far needs
@@ -834,33 +835,41 @@ struct fhmg_wsnet_s {
 namespace {
 
 template <typename T>
-int nalloc(fhmg_wsnet net, T** p, size_t n) {
+int nalloc(std::vector<void*>& owner, T** p, size_t n) {
   cudaError_t e = cudaMalloc((void**)p, (n ? n : 1) * sizeof(T));
   if (e != cudaSuccess) {
     cudaGetLastError();  // not sticky; keep it out of the next launch check
     return fhmg_internal_fail(FHMG_ENOMEM, cudaGetErrorString(e));
   }
-  net->allocs.push_back(*p);
+  owner.push_back(*p);
   return FHMG_OK;
 }
 
+// Activations for batches of n rows.  The smaller ones are freed first (which waits for the device); where the
+// larger do not fit, the network is left without any, so that the next call allocates what it needs.
 int ensure_cap(fhmg_wsnet net, int n) {
   if (n <= net->cap) return FHMG_OK;
   const int L = (int)net->width.size() - 1;
+  for (void* p : net->act) cudaFree(p);
+  net->act.clear();
+  net->cap = 0;
   net->Z.assign(L, nullptr);
   net->A.assign(L + 1, nullptr);
   net->dA.assign(L + 1, nullptr);
   int maxw = 0;
   for (int w : net->width) maxw = w > maxw ? w : maxw;
-  for (int l = 0; l < L; ++l) {
-    int s = nalloc(net, &net->Z[l], (size_t)n * net->width[l + 1]);
-    if (s) return s;
-    if ((s = nalloc(net, &net->A[l + 1], (size_t)n * net->width[l + 1]))) return s;
-    if ((s = nalloc(net, &net->dA[l + 1], (size_t)n * net->width[l + 1]))) return s;
+  int s = FHMG_OK;
+  for (int l = 0; l < L && s == FHMG_OK; ++l) {
+    const size_t m = (size_t)n * net->width[l + 1];
+    if ((s = nalloc(net->act, &net->Z[l], m)) == FHMG_OK && (s = nalloc(net->act, &net->A[l + 1], m)) == FHMG_OK)
+      s = nalloc(net->act, &net->dA[l + 1], m);
   }
-  int s;
-  if ((s = nalloc(net, &net->Abf[0], (size_t)n * maxw))) return s;
-  if ((s = nalloc(net, &net->Abf[1], (size_t)n * maxw))) return s;
+  for (int i = 0; i < 2 && s == FHMG_OK; ++i) s = nalloc(net->act, &net->Abf[i], (size_t)n * maxw);
+  if (s != FHMG_OK) {
+    for (void* p : net->act) cudaFree(p);
+    net->act.clear();
+    return s;
+  }
   net->cap = n;
   return FHMG_OK;
 }
@@ -1032,10 +1041,10 @@ int fhmg_wsnet_create(int hidden, int layers, unsigned long long seed, fhmg_wsne
     fhmg_wsnet_destroy(net);
     return st;
   };
-  if ((s = nalloc(net, &net->P, host.size())) || (s = nalloc(net, &net->G, host.size())) ||
-      (s = nalloc(net, &net->Mo, host.size())) || (s = nalloc(net, &net->Vo, host.size())) ||
-      (s = nalloc(net, &net->Pbf, host.size())) || (s = nalloc(net, &net->loss, 1)) || (s = nalloc(net, &net->err, 2)) ||
-      (hidden % 64 == 0 && hidden <= kMlpMaxH && (s = nalloc(net, &net->Wpk, mlp_packed(hidden, layers)))))
+  if ((s = nalloc(net->allocs, &net->P, host.size())) || (s = nalloc(net->allocs, &net->G, host.size())) ||
+      (s = nalloc(net->allocs, &net->Mo, host.size())) || (s = nalloc(net->allocs, &net->Vo, host.size())) ||
+      (s = nalloc(net->allocs, &net->Pbf, host.size())) || (s = nalloc(net->allocs, &net->loss, 1)) || (s = nalloc(net->allocs, &net->err, 2)) ||
+      (hidden % 64 == 0 && hidden <= kMlpMaxH && (s = nalloc(net->allocs, &net->Wpk, mlp_packed(hidden, layers)))))
     return bail(s);
   if (cudaMemcpy(net->P, host.data(), host.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(net->err, 0, 2 * sizeof(int)) != cudaSuccess ||
@@ -1048,6 +1057,7 @@ int fhmg_wsnet_create(int hidden, int layers, unsigned long long seed, fhmg_wsne
 int fhmg_wsnet_destroy(fhmg_wsnet net) {
   if (!net) return FHMG_OK;
   for (void* a : net->allocs) cudaFree(a);
+  for (void* a : net->act) cudaFree(a);
   cudaFree(net->part);
   for (auto& w : net->ws) cudaFree(w.first);
   delete net;
