@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "devinfo.h"
+#include "rcp.cuh"
 #include "umma.cuh"
 #include "fhmg.h"
 
@@ -429,16 +430,6 @@ __global__ void __launch_bounds__(256) gemm_bf16_silu(int M, int N, int K, const
     }
 }
 
-// 1 / d, correctly rounded, for 1 <= d < 2^126 (or NaN): one Newton step (with FMA, after Markstein) from the
-// approximate reciprocal; compared with the division for every mantissa and exponent of the range.
-// The division's range checks put a branch behind every activation: the epilogues of mlp_bf16 took
-// 27 000 cycles per layer and 128 rows with it.
-__device__ __forceinline__ float rcp_1_up(float d) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(d));
-  return __fmaf_rn(y, __fmaf_rn(-d, y, 1.f), y);
-}
-
 // The whole BF16 network on 128 rows at a time, on the tcgen05 tensor cores: input layer, hidden layers
 // of width H and output layer, activations (BF16, SiLU) kept in shared memory between them.  Every
 // layer is a batch of MMAs (M = 128 rows, N = the layer's width, FP32 accumulators in tensor memory) by
@@ -694,7 +685,7 @@ __global__ void __launch_bounds__(kMlpBlock, 1) mlp_bf16(int H, const __grid_con
             const float4 b = bp[j / 4];
             v[j] += b.x, v[j + 1] += b.y, v[j + 2] += b.z, v[j + 3] += b.w;
           }
-          // SiLU with the correctly rounded reciprocal of sigm(), without a division's branches
+          // SiLU as sigm() computes it, the division only beyond the reciprocal's range
           float d[16], dmax = 0.f;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
@@ -706,7 +697,7 @@ __global__ void __launch_bounds__(kMlpBlock, 1) mlp_bf16(int H, const __grid_con
             for (int j = 0; j < 16; ++j) d[j] = 1.f / d[j];
           } else {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) d[j] = rcp_1_up(d[j]);
+            for (int j = 0; j < 16; ++j) d[j] = fhmg::rcp_1_up(d[j]);
           }
 #pragma unroll
           for (int j = 0; j < 16; ++j) v[j] = v[j] * d[j];
