@@ -156,14 +156,17 @@ __device__ __forceinline__ void sp_digit_pairs(long long y0, long long y1, uint3
   pk[0] = __byte_perm(f0, f1, 0x7632);
 }
 
-// S = cd c - x0 - x1 (- x2 - x3) (cd = 2 NX), the undivided stencil of FP64 values, in 64-bit fixed
-// point relative to the largest of them: each value's significand, 6 bits up, shifted right by its
-// distance from the largest exponent (truncated towards -inf within 2^-59 of the largest value, so
-// S is within 2^-55 of it; the FP64 subtractions would be within a few 2^-53), the sum widened to FP64
-// by one conversion.  Zeros and negligible values shift out.  Outside the middle of the exponent
-// range, and for Inf and NaN, the FP64 subtractions themselves.
+// S = NX c - x0 - x1 (- x2 - x3), the undivided stencil of FP64 values, in 64-bit fixed point relative to
+// the largest of them: each value's significand, `up` bits up, shifted right by its distance from the largest
+// exponent, complemented for a negative value.  That stands for the integer and a half, on either side of
+// zero: the halves cancel in S (NX against NX of them), so S changes its sign with the values and vanishes
+// for equal ones, and a value is off by half a unit at most.  The unit is 2^-up of the largest value's last
+// place: S is within NX 2^-59 of that value's power of two (the FP64 subtractions: a few 2^-53), then widened to
+// FP64 by one conversion.  |S| < 2^63 units.  Zeros and negligible values shift out.  Outside the middle of
+// the exponent range, and for Inf and NaN, the FP64 subtractions themselves.
 template <int NX>
 __device__ __forceinline__ double sp_stencil(unsigned long long c, const unsigned long long (&x)[NX]) {
+  constexpr int up = NX == 4 ? 7 : 8;
   auto ex = [](unsigned long long b) { return (uint32_t)(b >> 32) & 0x7FF00000u; };
   uint32_t q = ex(c);
 #pragma unroll
@@ -173,17 +176,17 @@ __device__ __forceinline__ double sp_stencil(unsigned long long c, const unsigne
     const double t = fma((double)NX, d(c), -d(x[0])) - d(x[1]);
     return NX == 4 ? t - (d(x[NX - 2]) + d(x[NX - 1])) : t;
   }
-  auto fixed = [&](unsigned long long b, int up) -> long long {
+  auto fixed = [&](unsigned long long b) -> long long {
     unsigned long long m = ((b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52)) << up;
     asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"((q - ex(b)) >> 20));  // shifts past 63 give 0
     return (long long)m ^ ((long long)b >> 63);
   };
-  long long D = fixed(c, NX == 4 ? 8 : 7);
+  long long D = NX * fixed(c);
 #pragma unroll
-  for (int i = 0; i < NX; ++i) D -= fixed(x[i], 6);
-  const double s = (double)D;  // times 2^{q - 1081}: exponent field added
+  for (int i = 0; i < NX; ++i) D -= fixed(x[i]);
+  const double s = (double)D;  // times 2^{q - 1075 - up}: exponent field added
   const int hi = __double2hiint(s);
-  return __hiloint2double(hi == 0 ? 0 : hi + (int)(q - (1081u << 20)), __double2loint(s));
+  return __hiloint2double(hi == 0 ? 0 : hi + (int)(q - ((1075u + up) << 20)), __double2loint(s));
 }
 
 constexpr int kPrepThreads = 256, kPrepM = 32;  // threads along a grid row; time levels per block
