@@ -57,12 +57,13 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12   # 80.5: FFMA units x clock (a
 DF_PEAK_TFLOPS = 152 * 128 * 2.07e9 * 2 / 11 / 1e12  # 7.32
 HEAD = dict(dim=2, N=1023, M=512, alpha=0.55, gamma=2.0, seed=999, K=24, nc=31)
 METRIC = "space-time DOF*cycles/s (time-to-1e-8 solve): mixed+warm-start vs plain FP64"
-# DRAM bytes per column of one launch at M time levels, from the ncu captures named beside each
-# (same kernels and tiles on the 2D 255^2 x 512 case, scaled by columns); traffic is reported as
-# null for another M, and the entries are dropped whenever the kernel they describe changes
+# DRAM bytes per column of one launch at M time levels, from the one-pass ncu captures named beside each, on
+# the headline grid itself (on 255^2 a tenth and more of what a launch writes is still in L2 when it ends);
+# traffic is reported as null for another M, and the entries are dropped whenever the kernel they
+# describe changes
 TRAFFIC_PER_COLUMN = {
-    "smooth": (512, (150.61e6 + 30.52e6) / 32513),                     # profiles/humma_smooth_2d_255x512.md
-    "defect": (512, (772.95e6 + 803.34e6) / 65025),       # profiles/split_defect_2d_255x512.md (both kernels)
+    "smooth": (512, (2176.77e6 + 1034.57e6) / 523264.5),    # profiles/humma_smooth_2d_255x512.md (mean of both colours)
+    "defect": (512, (12970.8e6 + 13745.9e6) / 1046529),     # profiles/split_defect_2d_255x512.md (both kernels)
 }
 
 
