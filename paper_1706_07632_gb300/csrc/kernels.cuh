@@ -107,6 +107,8 @@ __host__ __device__ inline NbrOffsets nbr_offsets(const Geo& g) {
 // range of blocks holds it.  Within an instance 2^lx threads run along a grid row (x) and 256 / 2^lx
 // along the time levels, so that short rows fill their blocks too.
 template <typename T>
+constexpr bool kPlain2D = sizeof(T) == 8;  // 2D FP32 grid functions are stored by colour: kernels of their own below
+template <typename T>
 struct TransferJob {
   const T* F;   // restriction: right-hand side
   T* U;         // fine grid function (restriction: read; prolongation: corrected)
@@ -193,7 +195,7 @@ __global__ void __launch_bounds__(256) restrict_pre_kernel(const __grid_constant
   T* __restrict__ Bc = J.Bc;
   T* __restrict__ E = J.E;
   const T ih2 = (T)J.inv_h2;
-  if (J.dim == 1) {
+  if (!kPlain2D<T> || J.dim == 1) {
     const bool l = cx > 0, r = 2 * cx + 2 < Nf - 1;  // the outer neighbours exist
     for (int m = q.m0; m < M; m += q.dm) {
       const long long pc = (long long)m * Nf + 2 * cx + 1;
@@ -281,7 +283,7 @@ __global__ void __launch_bounds__(256) prolong_add_kernel(const __grid_constant_
   int ax0, ax1;
   T wx0, wx1;
   lin_weights<T>(x, Nc, ax0, wx0, ax1, wx1);
-  if (J.dim == 1) {
+  if (!kPlain2D<T> || J.dim == 1) {
     for (int m = q.m0; m < M; m += q.dm) {
       const T* e = E + (long long)m * Nc;
       U[(long long)m * Nf + x] += wx0 * e[ax0] + wx1 * e[ax1];
