@@ -176,14 +176,14 @@ __device__ __forceinline__ double sp_stencil(unsigned long long c, const unsigne
     const double t = fma((double)NX, d(c), -d(x[0])) - d(x[1]);
     return NX == 4 ? t - (d(x[NX - 2]) + d(x[NX - 1])) : t;
   }
-  auto fixed = [&](unsigned long long b) -> long long {
-    unsigned long long m = ((b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52)) << up;
+  auto fixed = [&](unsigned long long b, int left) -> long long {
+    unsigned long long m = ((b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52)) << left;
     asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"((q - ex(b)) >> 20));  // shifts past 63 give 0
     return (long long)m ^ ((long long)b >> 63);
   };
-  long long D = NX * fixed(c);
+  long long D = fixed(c, NX == 4 ? up + 2 : up + 1) & ~(NX - 1LL);  // NX times the point's integer
 #pragma unroll
-  for (int i = 0; i < NX; ++i) D -= fixed(x[i]);
+  for (int i = 0; i < NX; ++i) D -= fixed(x[i], up);
   const double s = (double)D;  // times 2^{q - 1075 - up}: exponent field added
   const int hi = __double2hiint(s);
   return __hiloint2double(hi == 0 ? 0 : hi + (int)(q - ((1075u + up) << 20)), __double2loint(s));
