@@ -254,8 +254,8 @@ int fhmg_problem_set_rtol_reference(fhmg_problem p, int ref);
  * tcgen05 tensor cores by error-free digit splitting (Ozaki et al. 2012) -- R~ (dense) and u are split
  * per time row / per grid point into 7 base-2^7 digits of 49 bits (fhmg_hmatrix_split_digits), the
  * digit products are summed exactly in FP32 tensor memory per digit-sum group and the groups are
- * combined in double-float; the stencil part B = F - A_h u is formed by a pre-pass in FP64 (every
- * third time level exactly, in 64-bit fixed point).  For time row m = 0..M-1 and grid point c,
+ * combined in double-float; the stencil part B = F - A_h u is formed by a pre-pass, its sum in 64-bit
+ * fixed point (within 2^-57 of the power of two of the largest value it takes), widened to FP64.  For time row m = 0..M-1 and grid point c,
  * |r - r_exact| <= (m+2) 2^{E_m + F_c - 46} + 2^-45 (|R~| |u|)_{m,c} + 2^-50 ((|A_h| |u|)_{m,c} + |F_{m,c}|)
  * (2^E_m > max_k |R~_mk|, 2^F_c > max_k |u_kc|).  The mode solves use double-float in modes 1 and 2.
  * EINVAL for mode 2 where it is not available. */

@@ -107,8 +107,6 @@ __host__ __device__ inline NbrOffsets nbr_offsets(const Geo& g) {
 // range of blocks holds it.  Within an instance 2^lx threads run along a grid row (x) and 256 / 2^lx
 // along the time levels, so that short rows fill their blocks too.
 template <typename T>
-constexpr bool kPlain2D = sizeof(T) == 8;  // 2D FP32 grid functions are stored by colour: kernels of their own below
-template <typename T>
 struct TransferJob {
   const T* F;   // restriction: right-hand side
   T* U;         // fine grid function (restriction: read; prolongation: corrected)
@@ -124,6 +122,8 @@ struct TransferBatch {
   TransferJob<T> job[NJ];
   int n;
 };
+template <typename T>
+constexpr bool kPlain2D = sizeof(T) == 8;  // 2D FP32 grid functions are stored by colour: kernels of their own below
 
 // Launch shape for n instances (restriction: a thread per coarse point, else per fine point): returns the
 // number of blocks, about 16 per SM over all of them, each with an equal share of the time levels' work.

@@ -11,10 +11,11 @@
 // Network: F = 6 input features -> H -> H -> H -> 1, SiLU activations, FP32 training (Adam), FP32
 // or BF16 inference.  Layer l maps width n_l to n_{l+1} with weights W_l (n_{l+1} x n_l,
 // row-major) and bias b_l; all parameters live in one FP32 array in layer order (W_0, b_0, W_1,
-// b_1, ...).  Kernels: tiled FP32 GEMM (64 x 64 tiles, 4 x 4 per thread, both transposes),
-// BF16 tensor-core GEMMs for inference (hidden layers with bias and SiLU fused), bias + SiLU forward /
-// backward, MSE loss, column sums, Adam, feature build, spectral
-// projection and synthesis.
+// b_1, ...).  Kernels: FP32 GEMM (64 x 64 tiles, 8 x 4 per thread, both transposes; bias, SiLU and its
+// derivative in the epilogue; weight gradients split over the rows, with the bias gradients), the
+// output layer's two passes, MSE loss, Adam; the BF16 network in one tcgen05 kernel (mlp_bf16), a BF16
+// tensor-core GEMM per layer for the widths it does not serve; feature build, spectral projection and
+// synthesis.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -437,8 +438,8 @@ __global__ void __launch_bounds__(256) gemm_bf16_silu(int M, int N, int K, const
 // 128-byte swizzle).  The hidden weights pass through a two-stage ring of K tiles of 64 (bulk copies of
 // the operand layout, prepared by pack_weights); the input layer's (K = 6, padded to 16), the output
 // layer's (one row, padded to 16) and the biases stay in shared memory.  The sums run over k16 steps in
-// order and round as mma.sync m16n8k16 does, so the results are those of the one-launch-per-layer path
-// bit for bit.  Bound by the epilogues (two special-function operations per activation).  294912 rows of
+// order and round as mma.sync m16n8k16 does here: the results are those of the one-launch-per-layer path bit
+// for bit (tests/test_gpu_network_paths.py).  Bound by the epilogues (two special-function operations per activation).  294912 rows of
 // width 320: 1.25 ms over six launches; fused with mma.sync 0.74 ms; 0.34 ms now.
 struct MlpArgs {
   int n, layers;                    // rows, hidden layers
@@ -451,6 +452,8 @@ struct MlpArgs {
   long long spin, withhold;         // polls of the MMA and epilogue warps' waits; 1-based tile never loaded (test hook)
 };
 
+// kMlpMaxH: the widest multiple of 64 for which every depth the network may have (8 hidden layers) fits in shared
+// memory: 200 KB at 320, where 384 would fit up to three layers only (tensor memory would hold 448).
 constexpr int kMlpRows = 128, kMlpMaxH = 320, kMlpEpi = 256, kMlpBlock = kMlpEpi + 64;
 // bytes of the packed weights: input layer (H x 16), output layer (16 x H), then per hidden layer H / 64
 // tiles of H x 64

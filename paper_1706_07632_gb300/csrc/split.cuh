@@ -19,7 +19,8 @@
 // the truncation coming from the 49-bit rounding of both factors and from the dropped groups
 // g >= 7.  The group sums are combined in double-float arithmetic and joined to FP64 with integer
 // operations (the FP64 pipe runs at 1/64 of the FP32 rate on GB300); a pre-pass at full occupancy
-// forms B = F - A_h u in FP64 and the exponents F_c, and the kernel's epilogue writes r = B - R~ u.
+// forms B = F - A_h u (the stencil in 64-bit fixed point, sp_stencil) and the exponents F_c, and the
+// kernel's epilogue writes r = B - R~ u.
 //
 // Kernel.  A CTA owns tiles of 64 grid points (64 MMA columns per digit, up to four digits in one MMA) and
 // walks the output blocks I of 128 time rows (MMA M = 128; TMEM lane = time row).  For every K-block

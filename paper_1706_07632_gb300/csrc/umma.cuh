@@ -211,8 +211,8 @@ __host__ __device__ inline long long umma_tiles(const Geo& g, long long ncols) {
 // (a line solve of 100003 x 512 columns 214 -> 176 us; with room for the L1 cache 151).  What bounds the
 // memory warps is the loads they can keep in flight: a finest half-sweep of a 1023^2 x 512 grid took 2.37
 // ms with loads by the walk, 2.31 with memory warps, 1.60 with grid functions stored by colour (whole
-// sectors), 1.47 with rolled loops (instruction cache), 1.04 with 60 instead of 28 KB of L1; its bytes
-// need 0.48 ms.  96 registers and at most 97 KB of shared memory: two CTAs per SM.
+// sectors), 1.47 with rolled loops (instruction cache), 1.04 with 60 instead of 28 KB of L1, 0.99 with a
+// pointer per neighbour; its bytes need 0.48 ms.  96 registers and at most 97 KB of shared memory: two CTAs per SM.
 template <int MODE>
 __global__ void __launch_bounds__(kUmmaBlock, 2) humma_kernel(const __grid_constant__ WalkBatch<float, uint16_t> B) {
   constexpr int L = kUmmaL, NT = kUmmaCols;

@@ -13,7 +13,7 @@ constexpr size_t kUmmaSmemMax = 227 * 1024;
 constexpr size_t kUmmaTwoPerSM = 112 * 1024;  // two CTAs share an SM's 228 KB (1 KB reserved each)
 // ... and in the 196 KB configuration, which leaves 60 KB of L1 instead of 28.  Loads in flight hold L1
 // lines, and their number bounded the memory warps: with two chunk slots in the small size instead of three
-// in the large one the finest half-sweep of a 1023^2 x 512 grid takes 1.04 ms instead of 1.44, the product of
+// in the large one the finest half-sweep of a 1023^2 x 512 grid took 1.04 ms instead of 1.44, the line solve of
 // 100,003 columns x M = 512 151 us instead of 174.
 constexpr size_t kUmmaTwoSmall = 97 * 1024;
 
